@@ -6,6 +6,7 @@
 
 #include "blas.h"
 #include "eofa.h"
+#include "fixed64.cuh"
 #include "learned.h"
 
 namespace eofa {
@@ -356,6 +357,39 @@ __global__ void __launch_bounds__(BT) k_zero(VecRef v, long n5, int Ls, const in
 #pragma unroll
     for (int i = 0; i < 24; ++i) z[i] = (R)0;
     store_sp<S, R>(v.d, v.n, xcb, s, Ls, z);
+}
+
+// FP64 hop input: psi, or chi = psi + z L psi (CHI: z = c5 / b5, mz = m1 c5 / b5,
+// so that b5 chi = D~ psi) in fixed point.  One pass over memory; inside the
+// hop the same work would be done eight times per site.
+template <bool CHI>
+__global__ void __launch_bounds__(BT) k_hop_input(VecRef out, VecRef psi, long n5, int Ls, double z, double mz,
+                                                  const int* skip) {
+    if (skip && *skip) return;
+    const long t = (long)blockIdx.x * BT + threadIdx.x;
+    if (t >= n5) return;
+    const long xcb = t / Ls;
+    const int s = (int)(t - xcb * Ls);
+    double v[24];
+    load_sp<double, double>(psi.d, nullptr, xcb, s, Ls, v);
+    if constexpr (CHI) {
+        double q[12];
+        load_half<double, double>(psi.d, nullptr, xcb, s == 0 ? Ls - 1 : s - 1, Ls, 0, q);
+        const double fu = s == 0 ? -mz : z, fd = s == Ls - 1 ? -mz : z;
+#pragma unroll
+        for (int i = 0; i < 12; ++i) v[i] += fu * q[i];
+        load_half<double, double>(psi.d, nullptr, xcb, s == Ls - 1 ? 0 : s + 1, Ls, 1, q);
+#pragma unroll
+        for (int i = 0; i < 12; ++i) v[12 + i] += fd * q[i];
+    }
+    fx_store(out.d, out.n, xcb, s, Ls, v);
+}
+
+cudaError_t blas_hop_input(VecRef out, VecRef psi, long n5, int Ls, bool chi, double z, double mz, cudaStream_t st,
+                           const int* skip) {
+    if (chi) k_hop_input<true><<<grid_for(n5), BT, 0, st>>>(out, psi, n5, Ls, z, mz, skip);
+    else k_hop_input<false><<<grid_for(n5), BT, 0, st>>>(out, psi, n5, Ls, z, mz, skip);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------

@@ -46,6 +46,10 @@ cudaError_t blas_acc(VecRef x, int eprec, VecRef e, long n5, int Ls, const DevSc
                      cudaStream_t st, const int* skip = nullptr);
 cudaError_t blas_sub(VecRef r, VecRef b, VecRef q, long n5, int Ls, Reduce rd, cudaStream_t st,
                      const int* skip = nullptr);
+// fixed-point input of the FP64 hop kernels: psi, or (chi) psi + z L psi for
+// the kinds with the D~ pre-op
+cudaError_t blas_hop_input(VecRef out, VecRef psi, long n5, int Ls, bool chi, double z, double mz, cudaStream_t st,
+                           const int* skip = nullptr);
 cudaError_t blas_zero(int prec, VecRef v, long n5, int Ls, cudaStream_t st, const int* skip = nullptr);
 cudaError_t layout_import(VecRef dst, const double* src, const Geom& g, int par, int g5r5, cudaStream_t st);
 cudaError_t layout_export(double* dst, VecRef src, const Geom& g, int par, int g5r5, cudaStream_t st);

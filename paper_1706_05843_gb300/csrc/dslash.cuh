@@ -29,6 +29,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "fixed64.cuh"
 
 namespace eofa {
 
@@ -60,6 +61,10 @@ template <int K> struct KindTraits {
                                 K == KIND_D_EO_DAG || K == KIND_D_OE_DAG;
     static constexpr bool PRE = K == KIND_EO_MINV || K == KIND_RECON || K == KIND_FULL;
     static constexpr bool HASY = !(K == KIND_EO_MINV || K == KIND_EO_MINV_DAG || K == KIND_D_EO || K == KIND_D_EO_DAG);
+    // FP64: the output is only ever the hop input of the next kernel and is
+    // stored in its fixed-point form (fixed64.cuh)
+    static constexpr bool FXOUT = K == KIND_EO_MINV || K == KIND_EO_MINV_DAG || K == KIND_D_EO ||
+                                  K == KIND_D_EO_DAG || K == KIND_LOC_DTMINV;
     // site-local kinds: the fifth-dimension part reaches only slices s-1, s+1
     // and the fixed slice of the rank-one shift, so each thread finishes its
     // own 5D site without the shared-memory column phase
@@ -70,7 +75,7 @@ struct HopArgs {
     Geom g;
     int out_par;
     int tile_var;                            // CTA tile variant (autotuner)
-    const void* in;  const float* in_nrm;    // hop input, parity 1 - out_par
+    const void* in;  const float* in_nrm;    // hop input, parity 1 - out_par (FP64: fixed point, exponents in in_nrm)
     const void* y;   const float* y_nrm;     // site-local input, parity out_par
     void* out;       float* out_nrm;         // output, parity out_par
     const void* lk_out;                      // links of parity out_par
@@ -701,6 +706,101 @@ __device__ __forceinline__ void link_from_raw(const unsigned char* raw, R* u) {
     }
 }
 
+// The hop sum of one 5D site in FP64 arithmetic from the fixed-point links:
+// the rare threads of hop_fixed whose neighbours are not finite or of
+// extreme magnitude.  LS is a runtime value here: one copy for all kernels.
+static __device__ __noinline__ void hop_fp64_slow(const longlong2* in, const int* ex, const int4* lk,
+                                                  const unsigned* nb, int s, int Ls, int FS, double* out) {
+    double acc[24];
+    for (int i = 0; i < 24; ++i) acc[i] = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < 8; ++k) {
+        const int l = (k & 1) * 4 + (k >> 1);
+        double p[24], W[18];
+        const long n = (long)(nb[l] & 0x7fffffffu);
+        const int e5 = ex[n * Ls + s];
+        for (int c = 0; c < 12; ++c) {
+            const longlong2 q = in[(n * 12 + c) * Ls + s];
+            p[2 * c] = e5 == kFxRaw ? __longlong_as_double(q.x) : fx_to(q.x, e5);
+            p[2 * c + 1] = e5 == kFxRaw ? __longlong_as_double(q.y) : fx_to(q.y, e5);
+        }
+        for (int e = 0; e < 9; ++e) {
+            const int4 q = lk[l * 9 + e];
+            W[2 * e] = ldexp((double)(((i64)q.x << kFxLimb) + q.y), -2 * kFxLimb);
+            W[2 * e + 1] = ldexp((double)(((i64)q.z << kFxLimb) + q.w), -2 * kFxLimb);
+        }
+        switch (FS > 0 ? k : k ^ 1) {
+            case 0: hop_dir<double, 0, 1, false>(acc, p, W); break;
+            case 1: hop_dir<double, 0, -1, false>(acc, p, W); break;
+            case 2: hop_dir<double, 1, 1, false>(acc, p, W); break;
+            case 3: hop_dir<double, 1, -1, false>(acc, p, W); break;
+            case 4: hop_dir<double, 2, 1, false>(acc, p, W); break;
+            case 5: hop_dir<double, 2, -1, false>(acc, p, W); break;
+            case 6: hop_dir<double, 3, 1, false>(acc, p, W); break;
+            default: hop_dir<double, 3, -1, false>(acc, p, W); break;
+        }
+    }
+    for (int i = 0; i < 24; ++i) out[i] = acc[i];
+}
+
+// The hop sum of one 5D site in fixed point (fixed64.cuh): lk the site's 8
+// staged links (backward ones daggered), nb its neighbour indices.  The
+// direction loop stays rolled: one copy of the products fits the
+// instruction cache (unrolled eight times it is about 100 KB).
+template <int LS, bool DAG>
+__device__ __forceinline__ void hop_fixed(const void* __restrict__ in, const float* __restrict__ nrm,
+                                          const int4* __restrict__ lk, const unsigned* __restrict__ nb, int s,
+                                          double* out) {
+    const longlong2* base = reinterpret_cast<const longlong2*>(in) + s;
+    const int* ex = reinterpret_cast<const int*>(nrm) + s;
+    i64 acc[24];
+#pragma unroll
+    for (int i = 0; i < 24; ++i) acc[i] = 0;
+    int E = 64;         // exponent field of the units of acc
+    bool raw = false;   // a neighbour is kept as doubles
+#pragma unroll 1
+    for (int k = 0; k < 8; ++k) {  // k = 2 mu + dir (dir 0 forward, 1 backward)
+        const int l = (k & 1) * 4 + (k >> 1);
+        const long n = (long)(nb[l] & 0x7fffffffu);
+        const longlong2* q = base + n * (12 * LS);
+        const int e = ex[n * LS];
+        i64 p[24], h[12], w[12];
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const longlong2 t = q[c * LS];
+            p[2 * c] = t.x;
+            p[2 * c + 1] = t.y;
+        }
+        raw = raw || e == kFxRaw;
+        if (e > E) {
+            const int sh = min(e - E, 63);
+#pragma unroll
+            for (int i = 0; i < 24; ++i) acc[i] >>= sh;
+            E = e;
+        }
+        const int kp = DAG ? k : k ^ 1;  // forward projector 1 + gamma for D^dag, 1 - gamma for D
+        fx_project(kp, p, h);
+        if (e < E) {
+            const int sh = min(E - e, 63);
+            const i64 half = 1ll << (sh - 1);
+#pragma unroll
+            for (int i = 0; i < 12; ++i) h[i] = (h[i] + half) >> sh;
+        }
+        fx_mul(lk + l * 9, h, w);
+        fx_reconstruct(kp, w, acc);
+    }
+    if (!raw) {
+#pragma unroll
+        for (int i = 0; i < 24; ++i) out[i] = fx_to(acc[i], E);
+    } else {
+        double r[24];
+        hop_fp64_slow(reinterpret_cast<const longlong2*>(in), reinterpret_cast<const int*>(nrm), lk, nb, s, LS,
+                      DAG ? 1 : -1, r);
+#pragma unroll
+        for (int i = 0; i < 24; ++i) out[i] = r[i];
+    }
+}
+
 // Persistent CTAs: a CTA walks the site blocks blockIdx.x, +gridDim.x, ...
 // While it works on one block, the links and neighbour indices of its next
 // block are already on their way (cp.async into a second staging buffer),
@@ -717,6 +817,7 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
     constexpr int LK = LinkStride<R>::V;
     constexpr int NL = NS * 8;  // staged links (and neighbour indices) per block
     constexpr int RAWB = LinkRaw<S>::PAD;
+    constexpr bool FX = sizeof(S) == 8;  // the hop in fixed point (fixed64.cuh)
 
     if (a.done && *a.done) return;
 
@@ -796,6 +897,11 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
                 R* dl = sl + (b * NL + j) * LK;
                 if constexpr (LinkRaw<S>::SEP) link_from_raw<S, R>(sraw + (b * NL + j) * RAWB, u);
                 else link_from_raw<S, R>(reinterpret_cast<const unsigned char*>(dl), u);
+                if constexpr (FX) {
+                    fx_stage_link(u, (g.gpmask | g.apmask) && (snb[b * NL + j] >> 31), (j & 7) >= 4,
+                                  reinterpret_cast<int4*>(dl));
+                    continue;
+                }
                 rebuild_row2(u);
                 // the factor -1 of an antiperiodic or G-parity boundary hop
                 // rides on the staged link; the branch is uniform over the grid
@@ -841,6 +947,10 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
         if (valid) {
             if constexpr (KT::HOP) {
                 constexpr int FS = KT::DAG ? +1 : -1;  // forward projector 1 + FS gamma
+                if constexpr (FX) {
+                    hop_fixed<LS, KT::DAG>(a.in, a.in_nrm, reinterpret_cast<const int4*>(slc + il * 8 * LK),
+                                           snc + il * 8, s, acc);
+                } else
                 // hop k = 2 mu + dir (dir 0 forward, 1 backward)
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
@@ -930,7 +1040,8 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
                 ld_half(sh + rp, o);
                 ld_half(sh + rm, o + 12);
             }
-            store_sp<S, R>(a.out, a.out_nrm, xcb, s, LS, o);
+            if constexpr (FX && KT::FXOUT) fx_store(a.out, a.out_nrm, xcb, s, LS, o);
+            else store_sp<S, R>(a.out, a.out_nrm, xcb, s, LS, o);
             if (a.rd.fin != FIN_NONE) {
 #pragma unroll
                 for (int i = 0; i < 24; ++i) nn += o[i] * o[i];
@@ -945,9 +1056,12 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
     if (a.rd.fin != FIN_NONE) block_reduce_finalize<NT>(nn, a.rd);
 }
 
-// the kernel with the compiler's own register choice (variants 0, 1) ...
+// the kernel with the compiler's own register choice (variants 0, 1; FP64:
+// 16 warps per SM, 128 registers and 76 bytes of spills, 228 us against 297 us
+// for the compiler's 168 registers at 16^4, Ls = 16) ...
 template <typename S, int LS, int KIND, int VAR = 0>
-__global__ void __launch_bounds__(Tile<LS, VAR>::NT) hop_kernel(const HopArgs a, const SCoef<typename Traits<S>::R> cf) {
+__global__ void __launch_bounds__(Tile<LS, VAR>::NT, sizeof(S) == 8 ? 512 / Tile<LS, VAR>::NT : 1)
+    hop_kernel(const HopArgs a, const SCoef<typename Traits<S>::R> cf) {
     hop_body<S, LS, KIND, VAR>(a, cf);
 }
 

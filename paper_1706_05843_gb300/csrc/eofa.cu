@@ -144,11 +144,13 @@ eofa_status dalloc(eofa_ctx* c, void** p, size_t bytes) {
     return EOFA_OK;
 }
 
-eofa_status vec_alloc(eofa_ctx* c, int prec, VecRef* v) {
+// hop_in: the vector may hold an FP64 hop input (fixed point with an exponent
+// per 5D site)
+eofa_status vec_alloc(eofa_ctx* c, int prec, VecRef* v, bool hop_in = false) {
     eofa_status s = dalloc(c, &v->d, (size_t)c->n5 * 24 * kWidth[prec]);
     if (s != EOFA_OK) return s;
     v->n = nullptr;
-    if (prec == EOFA_F16) {
+    if (prec == EOFA_F16 || hop_in) {
         void* n = nullptr;
         s = dalloc(c, &n, (size_t)c->n5 * sizeof(float));
         if (s != EOFA_OK) return s;
@@ -282,8 +284,25 @@ double hop_bytes_of(const eofa_ctx* c, int prec, int with_local) {
     return c->n5 * per5 + (double)c->g.Vh * 8.0 * 12.0 * w;
 }
 
+// FP64 hop kinds whose input is an FP64 field that a pass turns into the
+// kernel's fixed-point input (the others read what such a kernel wrote):
+// 2 with the D~ pre-op, 1 without
+int hop_input_pass(int kind) {
+    switch (kind) {
+        case KIND_EO_MINV: case KIND_RECON: case KIND_FULL: return 2;
+        case KIND_EO_MINV_DAG: case KIND_FULL_DAG: case KIND_D_EO: case KIND_D_EO_DAG: return 1;
+        default: return 0;
+    }
+}
+
 eofa_status hop(eofa_ctx* c, int prec, int kind, int out_par, VecRef in, VecRef y, VecRef out, Reduce rd,
                 const int* done, cudaStream_t st, bool timed = false) {
+    if (const int pass = prec == EOFA_F64 ? hop_input_pass(kind) : 0) {
+        // into c->ro, which holds nothing live at any of these launches
+        // (outer_residual writes it last)
+        CKL(blas_hop_input(c->ro, in, c->n5, c->g.Ls, pass == 2, c->c64.zb, c->c64.mzb, st, done), "hop input");
+        in = c->ro;
+    }
     HopArgs a;
     std::memset(&a, 0, sizeof(a));
     a.g = c->g;
@@ -353,7 +372,7 @@ eofa_status ensure_inner(eofa_ctx* c, int P) {
     if (in.ready) return EOFA_OK;
     eofa_status s;
     if ((s = vec_alloc(c, P, &in.r)) || (s = vec_alloc(c, P, &in.p)) || (s = vec_alloc(c, P, &in.q)) ||
-        (s = vec_alloc(c, P, &in.z)) || (s = vec_alloc(c, P, &in.t)) ||
+        (s = vec_alloc(c, P, &in.z)) || (s = vec_alloc(c, P, &in.t, P == EOFA_F64)) ||
         (s = vec_alloc(c, P == EOFA_F64 ? EOFA_F64 : EOFA_F32, &in.x)))
         return s;
     in.ready = true;
@@ -1086,8 +1105,8 @@ void drop_batch_graphs(unsigned long long uid) {
 
 // kernels of one system in one chunk of the batch graph (outer gate, step,
 // decision and restart included), and of the first residual and start
-constexpr int kBatchBodyKernels = 6 * kChunk + 11;
-constexpr int kBatchStartKernels = 10;
+constexpr int kBatchBodyKernels = 6 * kChunk + 12;
+constexpr int kBatchStartKernels = 11;
 
 // The outer step and the inner restart of system c in precision P: each
 // kernel is gated by its device flag.
@@ -1707,10 +1726,10 @@ static eofa_status create_impl(const eofa_params* p, const void* gauge, int gpma
             if ((s = dalloc(c, &c->links[pr][par], (size_t)g.Vh * 4 * 12 * kWidth[pr]))) return bail(s);
     for (int par = 0; par < 2; ++par) {
         if ((s = vec_alloc(c, 0, &c->b[par])) || (s = vec_alloc(c, 0, &c->x[par])) ||
-            (s = vec_alloc(c, 0, &c->t[par])))
+            (s = vec_alloc(c, 0, &c->t[par], true)))
             return bail(s);
     }
-    if ((s = vec_alloc(c, 0, &c->ro)) || (s = vec_alloc(c, 0, &c->bto)) || (s = vec_alloc(c, 0, &c->qo)))
+    if ((s = vec_alloc(c, 0, &c->ro, true)) || (s = vec_alloc(c, 0, &c->bto)) || (s = vec_alloc(c, 0, &c->qo)))
         return bail(s);
     const int maxgrid = std::max(blas_max_grid(c->n5), g.Vh / 8 + 2);
     void* tmp = nullptr;
@@ -2056,7 +2075,8 @@ constexpr size_t kNaLinks[4] = {kNaHalf * 4 * 12 * 8, kNaHalf * 4 * 12 * 4, kNaH
                                 kNaHalf * 4 * 12 * 2};  // one parity, per precision
 constexpr size_t kNaField = (size_t)(kNoAllocMaxSites5 / 2) * 24 * 8;  // one parity, FP64
 constexpr size_t kNaLinkTotal = 2 * (kNaLinks[0] + kNaLinks[1] + kNaLinks[2] + kNaLinks[3]);
-constexpr size_t kNaScratchBytes = kNaLinkTotal + 4 * kNaField + 256;
+constexpr size_t kNaExpo = (size_t)(kNoAllocMaxSites5 / 2) * 4;  // exponents of one hop input
+constexpr size_t kNaScratchBytes = kNaLinkTotal + 4 * kNaField + kNaExpo + 256;
 
 constexpr int kNaMaxDevices = 64;
 unsigned char* g_noalloc_ptr[kNaMaxDevices] = {};  // device address of the scratch, per device
@@ -2134,6 +2154,8 @@ extern "C" eofa_status eofa_apply_noalloc(const eofa_params* p, const void* gaug
         fout[par] = VecRef{base + off, nullptr};
         off += kNaField;
     }
+    float* expo = reinterpret_cast<float*>(base + off);
+    off += kNaExpo;
     int* bad = reinterpret_cast<int*>(base + off);
 
     // the flag must start at zero: the array keeps the previous call's contents
@@ -2147,20 +2169,25 @@ extern "C" eofa_status eofa_apply_noalloc(const eofa_params* p, const void* gaug
     for (int par = 0; par < 2; ++par)
         if (layout_import(fin[par], (const double*)in, g, par, 0, st) != cudaSuccess) return EOFA_ERR_CUDA;
     for (int par = 0; par < 2; ++par) {
+        // the hop input of the other parity in that parity's output field,
+        // which is written after (par 0) or exported before (par 1)
+        const VecRef chi{fout[1 - par].d, expo};
+        if (blas_hop_input(chi, fin[1 - par], (long)g.Vh * g.Ls, g.Ls, true, k.zb, k.mzb, st) != cudaSuccess)
+            return EOFA_ERR_CUDA;
         HopArgs a;
         std::memset(&a, 0, sizeof(a));
         a.g = g;
         a.out_par = par;
-        a.in = fin[1 - par].d;
+        a.in = chi.d;
+        a.in_nrm = chi.n;
         a.y = fin[par].d;
         a.out = fout[par].d;
         a.lk_out = links[EOFA_F64][par];
         a.lk_in = links[EOFA_F64][1 - par];
         a.rd.fin = FIN_NONE;
         if (launch_hop_f64(KIND_FULL, a, &k, st) != cudaSuccess) return EOFA_ERR_CUDA;
-    }
-    for (int par = 0; par < 2; ++par)
         if (layout_export((double*)out, fout[par], g, par, 0, st) != cudaSuccess) return EOFA_ERR_CUDA;
+    }
     return EOFA_OK;
 }
 

@@ -1,0 +1,253 @@
+// fixed64.cuh -- the FP64 Wilson hop in 64-bit fixed point on the integer pipe.
+//
+// GB300 issues 1.9 FP64 lanes per clock and SM (measured; one warp
+// instruction every 17 clocks) but 60 lanes of 32 x 32 + 64 bit integer
+// multiply-adds (mad.wide.s32), so the SU(3) products of the FP64 hop are
+// integer work here:
+//
+//  * a spinor that a hop reads is kept in memory as 24 signed integers in
+//    units of 2^(E-56) and E, the exponent field of its largest real (fx_pack,
+//    by the kernel that makes it): 57 bits, so every real within 2^-4 of the
+//    largest is exact and the others keep an absolute error below one unit,
+//    2^-3 of the ulp of the largest;
+//  * spin projection and reconstruction are 64-bit integer additions (exact);
+//  * a link's reals are 58-bit fixed point (Uh, Ul): u = (Uh 2^29 + Ul) 2^-58,
+//    |Ul| <= 2^28; a projected component is H = Hh 2^29 + Hl likewise, and
+//    U H = sum Uh Hh + 2^-29 sum (Uh Hl + Ul Hh): three mad.wide a product.
+//    The dropped 2^-58 Ul Hl is below 1/4 unit and has zero mean;
+//  * the eight directions accumulate in 64-bit integers at the largest
+//    exponent met so far (a larger one shifts the sums right).  Bound: reals
+//    below 2^57 units, |h| <= sqrt(3) 2 sqrt(2) 2^57 for a projected colour
+//    vector, |U h| = |h|, eight directions: below 2^62.3.
+//
+// The result is rounded to FP64 once.  A spinor with Inf, NaN or extreme
+// magnitude (exponent field of the largest real outside [64, 2030]) is kept
+// as its doubles (E = kFxRaw); threads that meet one redo their sums in FP64
+// arithmetic (hop_fp64_slow).
+//
+// Measured, one launch at 16^4, Ls = 16 (524288 5D sites): FP64 arithmetic
+// 1.04 ms (mean of kinds 0 to 3, FP64 pipe 88-90% busy), this form 0.22 to
+// 0.34 ms (the fifth dimension is FP64 still: 41% of its pipe) plus 0.026 to
+// 0.036 ms for the input pass.  Error of K against 64-bit values: 1.8e-16 to
+// 2.5e-16 relative, 1.9e-16 to 2.6e-16 with FP64 arithmetic.
+#pragma once
+
+#include "common.cuh"
+
+namespace eofa {
+
+typedef long long i64;
+
+constexpr int kFxFrac = 56;  // fraction bits below the block exponent
+constexpr int kFxLimb = 29;  // bits of a low limb
+
+// a 58-bit fixed-point value as its two limbs
+__device__ __forceinline__ int2 fx_split(i64 v) {
+    const int lo = ((int)v << 3) >> 3;  // low 29 bits, signed
+    return make_int2((int)((v + (1 << (kFxLimb - 1))) >> kFxLimb), lo);
+}
+
+// the double (hi, lo) in units of 2^(E - 1023 - frac), truncated; E at least
+// its exponent field, frac 56 (spinors) or 58 (links)
+template <int FRAC>
+__device__ __forceinline__ i64 fx_from(int hi, unsigned lo, int E) {
+    const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+    const int sh = min(E - (int)(((unsigned)hi >> 20) & 0x7ffu), 63);
+    const i64 m = (i64)((((unsigned long long)mh << 32) | lo) << (FRAC - 52) >> sh);
+    return hi < 0 ? -m : m;
+}
+
+// a link real (|u| <= 1 + 1e-10) as 58-bit fixed point
+__device__ __forceinline__ i64 fx_link(double u) {
+    return fx_from<2 * kFxLimb>(__double2hiint(u), (unsigned)__double2loint(u), 1023);
+}
+
+constexpr int kFxRaw = 2047;  // exponent mark of a spinor kept as doubles
+
+// 24 doubles -> their fixed-point form; returns E (0 for a zero spinor)
+__device__ __forceinline__ int fx_pack(const double* v, i64* m) {
+    int top = 0;
+#pragma unroll
+    for (int i = 0; i < 24; ++i) top = max(top, __double2hiint(v[i]) & 0x7fffffff);
+    const int E = top >> 20;
+    if (E < 64 || E > 2030) {
+        bool zero = true;
+#pragma unroll
+        for (int i = 0; i < 24; ++i) {
+            zero = zero && v[i] == 0.0;
+            m[i] = __double_as_longlong(v[i]);
+        }
+        if (!zero) return kFxRaw;
+#pragma unroll
+        for (int i = 0; i < 24; ++i) m[i] = 0;
+        return 0;
+    }
+#pragma unroll
+    for (int i = 0; i < 24; ++i) m[i] = fx_from<kFxFrac>(__double2hiint(v[i]), (unsigned)__double2loint(v[i]), E);
+    return E;
+}
+
+// the fixed-point spinor of 5D site (xcb, s) stored in place of 24 doubles,
+// its exponent in the site's scale slot
+__device__ __forceinline__ void fx_store(void* base, float* nrm, long xcb, int s, int Ls, const double* v) {
+    i64 m[24];
+    const int E = fx_pack(v, m);
+    longlong2* p = reinterpret_cast<longlong2*>(base) + xcb * 12 * Ls + s;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) p[c * Ls] = make_longlong2(m[2 * c], m[2 * c + 1]);
+    reinterpret_cast<int*>(nrm)[xcb * Ls + s] = E;
+}
+
+// units of 2^(E - 1023 - 56) -> double, E in [64, 2030]
+__device__ __forceinline__ double fx_to(i64 v, int E) {
+    const double d = (double)v;  // |v| < 2^63: rounded to nearest
+    const int hi = __double2hiint(d) + ((E - 1023 - kFxFrac) << 20);
+    return v == 0 ? 0.0 : __hiloint2double(hi, __double2loint(d));
+}
+
+// a b + c; the C++ expression compiles to an unsigned wide product and two
+// sign corrections
+__device__ __forceinline__ i64 fx_mad(int a, int b, i64 c) {
+    i64 d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
+
+// a link element: x, y the limbs of the real part, z, w of the imaginary part
+__device__ __forceinline__ int4 fx_elem(i64 re, i64 im) {
+    const int2 r = fx_split(re), i = fx_split(im);
+    return make_int4(r.x, r.y, i.x, i.y);
+}
+
+// rows 0 and 1 of a link (12 doubles) -> the 9 elements of W, the link or
+// (dag) its adjoint; row 2 = conj(row 0 x row 1) in fixed point; neg: the
+// hop's boundary sign
+__device__ __forceinline__ void fx_stage_link(const double* u, bool neg, bool dag, int4* dst) {
+    int4 e[9];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) e[i] = fx_elem(fx_link(u[2 * i]), fx_link(u[2 * i + 1]));
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int4 a = e[(j + 1) % 3], b = e[3 + (j + 2) % 3], c = e[(j + 2) % 3], d = e[3 + (j + 1) % 3];
+        // re(a b - c d) and -im(a b - c d)
+        i64 rh = 0, rm = 1 << (kFxLimb - 1), ih = 0, im = 1 << (kFxLimb - 1);
+        auto acc = [](int xh, int xl, int yh, int yl, i64& h, i64& m) {
+            h = fx_mad(xh, yh, h);
+            m = fx_mad(xh, yl, m);
+            m = fx_mad(xl, yh, m);
+        };
+        acc(a.x, a.y, b.x, b.y, rh, rm);
+        acc(a.z, a.w, -b.z, -b.w, rh, rm);
+        acc(c.x, c.y, -d.x, -d.y, rh, rm);
+        acc(c.z, c.w, d.z, d.w, rh, rm);
+        acc(a.x, a.y, -b.z, -b.w, ih, im);
+        acc(a.z, a.w, -b.x, -b.y, ih, im);
+        acc(c.x, c.y, d.z, d.w, ih, im);
+        acc(c.z, c.w, d.x, d.y, ih, im);
+        e[6 + j] = fx_elem(rh + (rm >> kFxLimb), ih + (im >> kFxLimb));
+    }
+    const int sr = neg ? -1 : 1, si = neg != dag ? -1 : 1;
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+        dst[dag ? (i % 3) * 3 + i / 3 : i] = make_int4(sr * e[i].x, sr * e[i].y, si * e[i].z, si * e[i].w);
+}
+
+// spin projection of a hop (see hop_dir): k = 2 mu + (SG < 0), h = the two
+// colour vectors of (1 + SG gamma_mu) p; exact
+__device__ __forceinline__ void fx_project(int k, const i64* __restrict__ p, i64* __restrict__ h) {
+    const i64 *u0 = p, *u1 = p + 6, *d0 = p + 12, *d1 = p + 18;
+#define FX_PROJ(K, R0, I0, R1, I1)                                  \
+    case K:                                                         \
+        _Pragma("unroll") for (int c = 0; c < 6; c += 2) {          \
+            h[c] = u0[c] R0; h[c + 1] = u0[c + 1] I0;               \
+            h[6 + c] = u1[c] R1; h[7 + c] = u1[c + 1] I1;           \
+        }                                                           \
+        break;
+    switch (k) {
+        FX_PROJ(0, +d1[c + 1], -d1[c], +d0[c + 1], -d0[c])
+        FX_PROJ(1, -d1[c + 1], +d1[c], -d0[c + 1], +d0[c])
+        FX_PROJ(2, -d1[c], -d1[c + 1], +d0[c], +d0[c + 1])
+        FX_PROJ(3, +d1[c], +d1[c + 1], -d0[c], -d0[c + 1])
+        FX_PROJ(4, +d0[c + 1], -d0[c], -d1[c + 1], +d1[c])
+        FX_PROJ(5, -d0[c + 1], +d0[c], +d1[c + 1], -d1[c])
+        FX_PROJ(6, +d0[c], +d0[c + 1], +d1[c], +d1[c + 1])
+        default:
+        FX_PROJ(7, -d0[c], -d0[c + 1], -d1[c], -d1[c + 1])
+    }
+#undef FX_PROJ
+}
+
+// reconstruction (see hop_dir): acc += the four spins of the projected w
+__device__ __forceinline__ void fx_reconstruct(int k, const i64* __restrict__ w, i64* __restrict__ acc) {
+#pragma unroll
+    for (int i = 0; i < 12; ++i) acc[i] += w[i];
+    i64 *d0 = acc + 12, *d1 = acc + 18;
+    const i64 *w0 = w, *w1 = w + 6;
+#define FX_REC(K, R0, I0, R1, I1)                                   \
+    case K:                                                         \
+        _Pragma("unroll") for (int c = 0; c < 6; c += 2) {          \
+            d0[c] R0; d0[c + 1] I0; d1[c] R1; d1[c + 1] I1;         \
+        }                                                           \
+        break;
+    switch (k) {
+        FX_REC(0, -= w1[c + 1], += w1[c], -= w0[c + 1], += w0[c])
+        FX_REC(1, += w1[c + 1], -= w1[c], += w0[c + 1], -= w0[c])
+        FX_REC(2, += w1[c], += w1[c + 1], -= w0[c], -= w0[c + 1])
+        FX_REC(3, -= w1[c], -= w1[c + 1], += w0[c], += w0[c + 1])
+        FX_REC(4, -= w0[c + 1], += w0[c], += w1[c + 1], -= w1[c])
+        FX_REC(5, += w0[c + 1], -= w0[c], -= w1[c + 1], += w1[c])
+        FX_REC(6, += w0[c], += w0[c + 1], += w1[c], += w1[c + 1])
+        default:
+        FX_REC(7, -= w0[c], -= w0[c + 1], -= w1[c], -= w1[c + 1])
+    }
+#undef FX_REC
+}
+
+// w = W h for both colour vectors of a projected spinor, W the staged link
+// (already daggered for a backward hop)
+__device__ __forceinline__ void fx_mul(const int4* __restrict__ W, const i64* __restrict__ h, i64* __restrict__ w) {
+    int2 hr[2][3], hi[2][3], hn[2][3];  // limbs of re, im and -im
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            hr[s][c] = fx_split(h[6 * s + 2 * c]);
+            hi[s][c] = fx_split(h[6 * s + 2 * c + 1]);
+            hn[s][c] = make_int2(-hi[s][c].x, -hi[s][c].y);
+        }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        i64 H[2][2], M[2][2];  // [spin][re, im]: high products; middle products, from 1/2
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            H[s][0] = H[s][1] = 0;
+            M[s][0] = M[s][1] = 1 << (kFxLimb - 1);
+        }
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int4 e = W[a * 3 + b];
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                H[s][0] = fx_mad(e.x, hr[s][b].x, H[s][0]);
+                M[s][0] = fx_mad(e.x, hr[s][b].y, M[s][0]);
+                M[s][0] = fx_mad(e.y, hr[s][b].x, M[s][0]);
+                H[s][0] = fx_mad(e.z, hn[s][b].x, H[s][0]);
+                M[s][0] = fx_mad(e.z, hn[s][b].y, M[s][0]);
+                M[s][0] = fx_mad(e.w, hn[s][b].x, M[s][0]);
+                H[s][1] = fx_mad(e.x, hi[s][b].x, H[s][1]);
+                M[s][1] = fx_mad(e.x, hi[s][b].y, M[s][1]);
+                M[s][1] = fx_mad(e.y, hi[s][b].x, M[s][1]);
+                H[s][1] = fx_mad(e.z, hr[s][b].x, H[s][1]);
+                M[s][1] = fx_mad(e.z, hr[s][b].y, M[s][1]);
+                M[s][1] = fx_mad(e.w, hr[s][b].x, M[s][1]);
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            w[6 * s + 2 * a] = H[s][0] + (M[s][0] >> kFxLimb);
+            w[6 * s + 2 * a + 1] = H[s][1] + (M[s][1] >> kFxLimb);
+        }
+    }
+}
+
+}  // namespace eofa
