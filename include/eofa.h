@@ -103,7 +103,9 @@ typedef struct {
     int rhs_form;        /* 0: H form, rhs = phi, sol = psi.  1: K form, rhs = b, sol = psi' (K psi' = b) */
     int kernel_timing;   /* 1: time every hop kernel with CUDA events (no graph capture) */
     int method;          /* inner operator.  0: the Cayley form (right preconditioning by
-                            D~(m1)^-1, O(Ls) site-diagonal inverse, App. B).  1: even-odd
+                            D~(m1)^-1, O(Ls) site-diagonal inverse, App. B); its Schur system
+                            S e = r is solved by CG on the normal equations of S D~^-1, with
+                            e = D~^-1 y, which takes fewer iterations.  1: even-odd
                             on Eq. (non_hermit_sys) directly, with the dense Ls x Ls inverse
                             of its site-diagonal block (the "dense" scheme the paper compares
                             against, Sec. V.B); same outer loop, for comparison */

@@ -59,6 +59,17 @@ struct SCoef {
     R um[LSMAX];      // u of the shift (App. B)
     R xm[LSMAX];      // x = A^-1 u
     R ym[LSMAX];      // y = A^-T (k e_{j*})
+    // the right-preconditioned inner operator, with T = D~ M^-1 = A_ee^-1 of
+    // the unpreconditioned system and kT = b5 / alpha (kernel kinds R_*)
+    R g1;             // c5/b5 - gamma/alpha
+    R fR;             // -kT^2 / 4
+    R kTb;            // kT / b5
+    R wu[LSMAX];      // alpha wa
+    R wv[LSMAX];      // b5 wb
+    R xD[LSMAX];      // D~ x sbk_den / (alpha kT)
+    R uT[LSMAX];      // u sbk kT / b5
+    R yn[LSMAX];      // y sb_den
+    R eD[LSMAX];      // D~^-T e_{j*} sbk kT
 };
 
 // ---------------------------------------------------------------------------

@@ -5,7 +5,7 @@
 
 namespace eofa {
 cudaError_t launch_hop_f64(int kind, const HopArgs& a, const void* coef, cudaStream_t st) {
-    return kind <= KIND_OE_SCHUR_DAG ? launch_inner_t<double>(kind, a, coef, st)
+    return (kind >= KIND_R_EO && kind <= KIND_R_OE_DAG) ? launch_inner_t<double>(kind, a, coef, st)
                                      : launch_hop_f64_outer(kind, a, coef, st);
 }
 }  // namespace eofa

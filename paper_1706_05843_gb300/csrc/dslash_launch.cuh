@@ -92,25 +92,41 @@ template <typename S, int LS>
 static cudaError_t launch_inner_ls(int kind, const HopArgs& a, const SCoef<typename Traits<S>::R>& c,
                                    cudaStream_t st) {
     switch (kind) {
-        case KIND_EO_MINV: return launch_var<S, LS, KIND_EO_MINV>(a, c, st);
-        case KIND_OE_SCHUR: return launch_var<S, LS, KIND_OE_SCHUR>(a, c, st);
-        case KIND_EO_MINV_DAG: return launch_var<S, LS, KIND_EO_MINV_DAG>(a, c, st);
-        case KIND_OE_SCHUR_DAG: return launch_var<S, LS, KIND_OE_SCHUR_DAG>(a, c, st);
+        case KIND_R_EO: return launch_var<S, LS, KIND_R_EO>(a, c, st);
+        case KIND_R_OE: return launch_var<S, LS, KIND_R_OE>(a, c, st);
+        case KIND_R_EO_DAG: return launch_var<S, LS, KIND_R_EO_DAG>(a, c, st);
+        case KIND_R_OE_DAG: return launch_var<S, LS, KIND_R_OE_DAG>(a, c, st);
         default: return cudaErrorNotSupported;
     }
 }
 
+// FP32: the adjoint halves serve the training solves; FP64: the operators
+// of the outer solver and of the applications
 template <typename S, int LS>
 static cudaError_t launch_outer_ls(int kind, const HopArgs& a, const SCoef<typename Traits<S>::R>& c,
                                    cudaStream_t st) {
+    if constexpr (sizeof(S) == 8) {
+        switch (kind) {
+            case KIND_RECON: return launch_one<S, LS, KIND_RECON, 0>(a, c, st);
+            case KIND_SRC: return launch_one<S, LS, KIND_SRC, 0>(a, c, st);
+            case KIND_FULL: return launch_one<S, LS, KIND_FULL, 0>(a, c, st);
+            case KIND_FULL_DAG: return launch_one<S, LS, KIND_FULL_DAG, 0>(a, c, st);
+            case KIND_LOC_DTMINV: return launch_one<S, LS, KIND_LOC_DTMINV, 0>(a, c, st);
+            case KIND_LOC_DT: return launch_one<S, LS, KIND_LOC_DT, 0>(a, c, st);
+            default: break;
+        }
+    } else {
+        switch (kind) {
+            case KIND_EO_MINV_DAG: return launch_one<S, LS, KIND_EO_MINV_DAG, 0>(a, c, st);
+            case KIND_OE_SCHUR_DAG: return launch_one<S, LS, KIND_OE_SCHUR_DAG, 0>(a, c, st);
+            default: break;
+        }
+    }
     switch (kind) {
-        case KIND_RECON: return launch_one<S, LS, KIND_RECON, 0>(a, c, st);
-        case KIND_SRC: return launch_one<S, LS, KIND_SRC, 0>(a, c, st);
-        case KIND_FULL: return launch_one<S, LS, KIND_FULL, 0>(a, c, st);
-        case KIND_FULL_DAG: return launch_one<S, LS, KIND_FULL_DAG, 0>(a, c, st);
-        case KIND_LOC_DTMINV: return launch_one<S, LS, KIND_LOC_DTMINV, 0>(a, c, st);
-        case KIND_LOC_DT: return launch_one<S, LS, KIND_LOC_DT, 0>(a, c, st);
+        case KIND_EO_MINV: return launch_one<S, LS, KIND_EO_MINV, 0>(a, c, st);
+        case KIND_OE_SCHUR: return launch_one<S, LS, KIND_OE_SCHUR, 0>(a, c, st);
         case KIND_LOC_DTINV: return launch_one<S, LS, KIND_LOC_DTINV, 0>(a, c, st);
+        case KIND_R_BACK: return launch_one<S, LS, KIND_R_BACK, 0>(a, c, st);
         case KIND_D_EO: return launch_one<S, LS, KIND_D_EO, 0>(a, c, st);
         case KIND_D_OE: return launch_one<S, LS, KIND_D_OE, 0>(a, c, st);
         case KIND_D_EO_DAG: return launch_one<S, LS, KIND_D_EO_DAG, 0>(a, c, st);
@@ -119,7 +135,7 @@ static cudaError_t launch_outer_ls(int kind, const HopArgs& a, const SCoef<typen
     }
 }
 
-// kinds 0..3 (every storage type)
+// the halves of the inner operator (every storage type)
 template <typename S>
 static cudaError_t launch_inner_t(int kind, const HopArgs& a, const void* coef, cudaStream_t st) {
     typedef typename Traits<S>::R R;
@@ -133,7 +149,7 @@ static cudaError_t launch_inner_t(int kind, const HopArgs& a, const void* coef, 
     }
 }
 
-// kinds 4..14 (FP64 and FP32 storage)
+// every other kind (FP64 and FP32 storage)
 template <typename S>
 static cudaError_t launch_outer_t(int kind, const HopArgs& a, const void* coef, cudaStream_t st) {
     typedef typename Traits<S>::R R;

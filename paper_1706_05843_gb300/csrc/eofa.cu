@@ -193,7 +193,10 @@ void cast_coef(const SCoef<double>& d, SCoef<R>& r) {
     for (int i = 0; i < LSMAX; ++i) {
         r.wa[i] = (R)d.wa[i]; r.wb[i] = (R)d.wb[i];
         r.um[i] = (R)d.um[i]; r.xm[i] = (R)d.xm[i]; r.ym[i] = (R)d.ym[i];
+        r.wu[i] = (R)d.wu[i]; r.wv[i] = (R)d.wv[i]; r.xD[i] = (R)d.xD[i];
+        r.uT[i] = (R)d.uT[i]; r.yn[i] = (R)d.yn[i]; r.eD[i] = (R)d.eD[i];
     }
+    r.g1 = (R)d.g1; r.fR = (R)d.fR; r.kTb = (R)d.kTb;
 }
 
 // App. B: A = (D_DWF)_ee = alpha + gamma L(m1), alpha = b5 (4 - M5) + 1,
@@ -253,6 +256,24 @@ eofa_status coef_from_params(const eofa_params& p, SCoef<double>& k, const char*
     k.sbk = sb * kk;
     k.sbk_den = k.has_shift ? sb * kk / den : 0.0;
     k.sb_den = k.has_shift ? sb / den : 0.0;
+    // T = D~ M^-1 = kT [1 + g1 L U] - shift, U = alpha A^-1, kT = b5 / alpha, and
+    // T^-1 = M D~^-1 = (1 / kT) [1 - g1 L W] + shift, W = b5 D~^-1
+    const double kT = b5 / alpha;
+    k.g1 = zb - za;
+    k.fR = -0.25 * kT * kT;
+    k.kTb = kT / b5;
+    double eD[LSMAX];
+    e[Ls - 1] = 1.0;
+    host_invT(Ls, b5, c5, m, e, eD);
+    for (int s = 0; s < Ls; ++s) {
+        k.wu[s] = alpha * k.wa[s];
+        k.wv[s] = b5 * k.wb[s];
+        const double dx = b5 * k.xm[s] + c5 * (s ? k.xm[s - 1] : -m * k.xm[Ls - 1]);
+        k.xD[s] = dx * k.sbk_den / (alpha * kT);
+        k.uT[s] = k.um[s] * k.sbk * kT / b5;
+        k.yn[s] = k.ym[s] * k.sb_den;
+        k.eD[s] = eD[s] * k.sbk * kT;
+    }
     return EOFA_OK;
 }
 
@@ -290,7 +311,7 @@ double hop_bytes_of(const eofa_ctx* c, int prec, int with_local) {
 int hop_input_pass(int kind) {
     switch (kind) {
         case KIND_EO_MINV: case KIND_RECON: case KIND_FULL: return 2;
-        case KIND_EO_MINV_DAG: case KIND_FULL_DAG: case KIND_D_EO: case KIND_D_EO_DAG: return 1;
+        case KIND_FULL_DAG: case KIND_D_EO: case KIND_D_EO_DAG: case KIND_R_EO: case KIND_R_EO_DAG: return 1;
         default: return 0;
     }
 }
@@ -313,7 +334,7 @@ eofa_status hop(eofa_ctx* c, int prec, int kind, int out_par, VecRef in, VecRef 
     a.lk_out = c->links[prec][out_par];
     a.lk_in = c->links[prec][1 - out_par];
     a.rd = rd;
-    a.tile_var = (kind <= KIND_OE_SCHUR_DAG && c->tuned[prec]) ? c->tile[prec][kind] : 0;
+    a.tile_var = (kind >= KIND_R_EO && kind <= KIND_R_OE_DAG && c->tuned[prec]) ? c->tile[prec][kind - KIND_R_EO] : 0;
     a.done = done;
     if (kind >= KIND_D_EO && kind <= KIND_D_OE_DAG && prec <= EOFA_F32)
         a.dense = c->dense[prec][(kind == KIND_D_OE || kind == KIND_D_OE_DAG) ? 1 : 0];
@@ -340,7 +361,7 @@ eofa_status hop(eofa_ctx* c, int prec, int kind, int out_par, VecRef in, VecRef 
     ++c->launches;
     if (tm) {
         CK(cudaEventRecord(c->evs[c->ev_used + 1], st), "cudaEventRecord");
-        const bool wl = kind == KIND_OE_SCHUR || kind == KIND_OE_SCHUR_DAG;
+        const bool wl = kind == KIND_R_OE || kind == KIND_R_OE_DAG || kind == KIND_D_OE || kind == KIND_D_OE_DAG;
         if ((int)c->ev_bytes.size() < c->ev_used / 2 + 1) c->ev_bytes.resize(c->ev_used / 2 + 1);
         c->ev_bytes[c->ev_used / 2] = hop_bytes_of(c, prec, wl);
         c->ev_used += 2;
@@ -438,8 +459,17 @@ eofa_status autotune(eofa_ctx* c, int P, cudaStream_t st) {
     CK(cudaEventCreate(&e1), "event");
     const VecRef none{};
     eofa_status s = EOFA_OK;
+    // the kinds that a captured solve launches beside the tuned ones: once
+    // here, because their set-up must not run inside a capture
+    const int xp = P == EOFA_F64 ? EOFA_F64 : EOFA_F32;
+    s = hop(c, xp, KIND_R_BACK, 1, none, P == EOFA_F64 ? odd_a : c->inner[P].x, VecRef{c->ro.d, nullptr},
+            red(c, FIN_NONE), nullptr, st);
+    if (s == EOFA_OK && P == EOFA_F64)
+        s = hop(c, P, KIND_EO_MINV, 0, odd_a, none, even_t, red(c, FIN_NONE), nullptr, st);
+    if (s == EOFA_OK && P == EOFA_F64)
+        s = hop(c, P, KIND_OE_SCHUR, 1, even_t, odd_a, odd_b, red(c, FIN_NONE), nullptr, st);
     for (int k = 0; k < 4 && s == EOFA_OK; ++k) {
-        const bool even_out = (k == KIND_EO_MINV || k == KIND_EO_MINV_DAG);
+        const bool even_out = (k & 1) == 0;  // kernel kinds KIND_R_EO + k
         const int nvar = (P == EOFA_F64) ? 2 : 4;  // register-capped variants for FP32 arithmetic
         float best[4] = {1e30f, 1e30f, 1e30f, 1e30f};
         // three interleaved rounds; each variant keeps its fastest round
@@ -449,8 +479,9 @@ eofa_status autotune(eofa_ctx* c, int P, cudaStream_t st) {
                 c->tuned[P] = true;
                 c->tile[P][k] = v;
                 auto launch = [&]() {
-                    return even_out ? hop(c, P, k, 0, odd_a, none, even_t, red(c, FIN_NONE), nullptr, st)
-                                    : hop(c, P, k, 1, even_t, odd_a, odd_b, red(c, FIN_NONE), nullptr, st);
+                    const int kind = KIND_R_EO + k;
+                    return even_out ? hop(c, P, kind, 0, odd_a, none, even_t, red(c, FIN_NONE), nullptr, st)
+                                    : hop(c, P, kind, 1, even_t, odd_a, odd_b, red(c, FIN_NONE), nullptr, st);
                 };
                 if ((s = launch())) {  // warm-up; a variant the device cannot launch is skipped
                     if (v == 0 || forced >= 0) break;
@@ -498,10 +529,25 @@ double since(Clock::time_point t0) {
     return std::chrono::duration<double>(Clock::now() - t0).count();
 }
 
-// Inner CGNR on the Schur complement in storage precision P, unit source in
-// inner.r, solution in inner.x; stops at |r|^2 <= tol^2 (source norm 1).
-// one CGNR iteration on the Schur complement (6 launches); every kernel
-// returns at once when the device flag scal->done is set
+// The four Schur halves of the inner operator (consecutive kinds).  Method 0
+// solves the Cayley-form Schur system S e = r by CGNR on kT S D~^-1, with
+// e = kT D~^-1 y (cg_back): the right preconditioner D~ leaves the residual
+// as it is and takes the condition number of D~ out of the normal equations
+// (iterations against CGNR on S itself: 115 to 145 at 8^4 Ls = 8, 165 to 190
+// at 4^3x8 Ls = 16, 345 to 370 at Ls = 12 on rough links, 60 to 80 at m1 =
+// 0.15), and its site-diagonal factors D~ M^-1 and M D~^-1 keep O(Ls) forms
+// without the D~ pre-op.  Method 1 is the dense scheme; the training of the
+// learned preconditioner takes its iterates from CGNR on S (kPlainCayley).
+constexpr int kPlainCayley = 2;
+
+int cg_kind(const eofa_ctx* c) {
+    return c->method == 1 ? KIND_D_EO : c->method == kPlainCayley ? KIND_EO_MINV : KIND_R_EO;
+}
+
+// kernels of one CGNR iteration: four hops and two vector kernels, and in
+// FP64 two input passes
+constexpr int cg_kernels(int P) { return P == EOFA_F64 ? 8 : 6; }
+
 // One CGNR iteration on the Schur complement (6 launches; every kernel
 // returns at once when scal->done is set): q = S p (|q|^2 -> alpha),
 // r -= alpha q (|r|^2: convergence), z = S^dag r (|z|^2 -> beta), then
@@ -512,9 +558,7 @@ eofa_status cg_iteration(eofa_ctx* c, int P, cudaStream_t st, bool timed, cudaEv
     const int xp = P == EOFA_F64 ? EOFA_F64 : EOFA_F32;
     const int* done = &c->scal->done;
     const VecRef none{};
-    const bool dn = c->method == 1;  // the four Schur halves of the chosen inner operator
-    const int k0 = dn ? KIND_D_EO : KIND_EO_MINV, k1 = dn ? KIND_D_OE : KIND_OE_SCHUR;
-    const int k2 = dn ? KIND_D_EO_DAG : KIND_EO_MINV_DAG, k3 = dn ? KIND_D_OE_DAG : KIND_OE_SCHUR_DAG;
+    const int k0 = cg_kind(c), k1 = k0 + 1, k2 = k0 + 2, k3 = k0 + 3;
     eofa_status s;
     auto mark = [&](int i) -> eofa_status {
         // External: under stream capture this becomes an event record node
@@ -547,14 +591,22 @@ eofa_status cg_start(eofa_ctx* c, int P, const int* skip, cudaStream_t st) {
     const int xp = P == EOFA_F64 ? EOFA_F64 : EOFA_F32;
     const VecRef none{};
     eofa_status s;
-    const bool dn = c->method == 1;
+    const int k0 = cg_kind(c);
     CKL(blas_zero(xp, in.x, c->n5, c->g.Ls, st, skip), "blas_zero");
-    if ((s = hop(c, P, dn ? KIND_D_EO_DAG : KIND_EO_MINV_DAG, 0, in.r, none, in.t, red(c, FIN_NONE), skip, st)))
+    if ((s = hop(c, P, k0 + 2, 0, in.r, none, in.t, red(c, FIN_NONE), skip, st)))
         return s;
-    if ((s = hop(c, P, dn ? KIND_D_OE_DAG : KIND_OE_SCHUR_DAG, 1, in.t, in.r, in.z, red(c, FIN_ZZ), skip, st)))
+    if ((s = hop(c, P, k0 + 3, 1, in.t, in.r, in.z, red(c, FIN_ZZ), skip, st)))
         return s;
     CKL(blas_copy(P, in.p, P, in.z, c->n5, c->g.Ls, 1.0, -1, red(c, FIN_NONE), st, skip), "blas_copy");
     return EOFA_OK;
+}
+
+// The inner solution y in the Cayley variables of the outer iterate: e = kT
+// D~^-1 y (method 0) or D~^-1 y (method 1), in precision xp, into c->ro's
+// memory (free until the next outer residual).  skip as in cg_start.
+eofa_status cg_back(eofa_ctx* c, int xp, VecRef y, VecRef* e, const int* skip, cudaStream_t st) {
+    *e = VecRef{c->ro.d, nullptr};
+    return hop(c, xp, c->method == 1 ? KIND_LOC_DTINV : KIND_R_BACK, 1, VecRef{}, y, *e, red(c, FIN_NONE), skip, st);
 }
 
 // After a graph-path inner solve: the four hop launches of its first
@@ -675,7 +727,7 @@ eofa_status run_cgnr(eofa_ctx* c, int P, double tol, int maxit, int* iters, doub
         *iters = h.iters;
         *rr_out = h.rr;
         if ((s = fold_graph_sample(c, P))) return s;
-        c->launches += 6 + (long)(6 * kChunk + 1) * std::max(1, (h.iters - 1 + kChunk - 1) / kChunk);
+        c->launches += cg_kernels(P) + (long)(cg_kernels(P) * kChunk + 1) * std::max(1, (h.iters - 1 + kChunk - 1) / kChunk);
         if (h.nonfinite) return fail(c, EOFA_ERR_NONFINITE, "NaN or Inf in the inner CG reductions");
         if (h.done) return EOFA_OK;
         if (h.timed_out) return fail(c, EOFA_ERR_TIMEOUT, "solve exceeded timeout_ms");
@@ -1047,15 +1099,8 @@ eofa_status solve_impl(eofa_ctx* c, const double* rhs, double* sol, const eofa_s
             ss.result = is;
             break;
         }
-        VecRef e = c->inner[ss.P].x;
-        if (c->method == 1) {
-            // the dense scheme's correction is in psi; the outer iterate is
-            // psi' = D~^-1 psi
-            if ((s = hop(c, ss.xp, KIND_LOC_DTINV, 1, VecRef{}, e, c->inner[ss.P].z, red(c, FIN_NONE), nullptr,
-                         st)))
-                return s;
-            e = c->inner[ss.P].z;
-        }
+        VecRef e = c->inner[ss.P].x;  // flexible GCR returns it in the outer variables
+        if (o.precond == 0 && (s = cg_back(c, ss.xp, c->inner[ss.P].x, &e, nullptr, st))) return s;
         CKL(blas_acc(c->x[1], ss.xp, e, c->n5, Ls, c->scal, 0, st), "acc");
         ss.x_zero = false;
     }
@@ -1105,8 +1150,8 @@ void drop_batch_graphs(unsigned long long uid) {
 
 // kernels of one system in one chunk of the batch graph (outer gate, step,
 // decision and restart included), and of the first residual and start
-constexpr int kBatchBodyKernels = 6 * kChunk + 12;
-constexpr int kBatchStartKernels = 11;
+constexpr int batch_body_kernels(int P) { return cg_kernels(P) * kChunk + (P == EOFA_F64 ? 14 : 13); }
+constexpr int batch_start_kernels(int P) { return P == EOFA_F64 ? 12 : 11; }
 
 // The outer step and the inner restart of system c in precision P: each
 // kernel is gated by its device flag.
@@ -1201,7 +1246,9 @@ eofa_status build_batch_graph(eofa_ctx* const* cs, int n, int P, cudaGraphExec_t
         if (r != EOFA_OK) return r;
         CKL(outer_gate(sc, st), "outer_gate");
         const int* os = &sc->o_skip_step;
-        CKL(blas_acc(ci->x[1], xp, ci->inner[P].x, ci->n5, ci->g.Ls, sc, 0, st, os), "acc");
+        VecRef e;
+        if ((r = cg_back(ci, xp, ci->inner[P].x, &e, os, st))) return r;
+        CKL(blas_acc(ci->x[1], xp, e, ci->n5, ci->g.Ls, sc, 0, st, os), "acc");
         if ((r = hop(ci, 0, KIND_EO_MINV, 0, ci->x[1], none, ci->t[0], red(ci, FIN_NONE), os, st))) return r;
         if ((r = hop(ci, 0, KIND_OE_SCHUR, 1, ci->t[0], ci->x[1], ci->qo, red(ci, FIN_NONE), os, st))) return r;
         CKL(blas_sub(ci->ro, ci->bto, ci->qo, ci->n5, ci->g.Ls, red(ci, FIN_STORE, 0), st, os), "sub");
@@ -1313,7 +1360,7 @@ eofa_status solve_batched_impl(eofa_ctx* const* cs, int n, const void* const* rh
     for (int i = 0; i < n; ++i) {
         eofa_ctx* c = cs[i];
         const DevScal& h = *c->h_scal;
-        c->launches += kBatchStartKernels + (long)kBatchBodyKernels * chunks + (i == 0 ? chunks : 0);
+        c->launches += batch_start_kernels(P) + (long)batch_body_kernels(P) * chunks + (i == 0 ? chunks : 0);
         if (ss[i].finished) continue;  // zero right-hand side
         ss[i].outer = h.outer;
         ss[i].total = h.total;
@@ -2453,7 +2500,11 @@ eofa_status run_fgcr(eofa_ctx* c, double tol, int maxit, int* iters, cudaStream_
             double crr = 0.0;
             eofa_status cs = run_cgnr(c, EOFA_F32, tol / rn, maxit - *iters, &cits, &crr, st, t0, timeout_ms);
             *iters += cits;
-            CKL(caxpby(in.x, c->gx, n5, Ls, 1.f, 0.f, (float)rn, st), "caxpby");
+            VecRef e;
+            eofa_status bs = cg_back(c, EOFA_F32, in.x, &e, nullptr, st);
+            if (bs != EOFA_OK) return bs;
+            CKL(blas_copy(EOFA_F32, in.x, EOFA_F32, e, n5, Ls, rn, -1, red(c, FIN_NONE), st), "copy");
+            CKL(caxpby(in.x, c->gx, n5, Ls, 1.f, 0.f, 1.f, st), "caxpby");
             return cs;
         }
     }
@@ -2538,6 +2589,7 @@ extern "C" eofa_status eofa_train_preconditioner(eofa_ctx* ctx, const void* cons
         if ((s = outer_residual(c, ss, st))) return s;
         CKL(blas_copy(EOFA_F32, in.r, 0, c->ro, n5, Ls, 1.0, 0, red(c, FIN_NONE), st), "copy");
         const double tol = opts->solve_tol;
+        c->method = kPlainCayley;  // (solve_begin sets the method of every solve)
         CKL(scal_init(c->scal, tol * tol, 100000, 0ull, st), "scal_init");
         if ((s = cg_start(c, EOFA_F32, nullptr, st))) return s;
         int ns = 1;  // snapshot 0 is the zero start vector

@@ -1,0 +1,45 @@
+"""GPU test of the inner operator (CG on S D~^-1, the correction mapped back
+by D~^-1) over the Moebius coefficients its recurrences take: Shamir (c = 0),
+c / b near 1 and negative, both chiralities of the shift, no shift, every
+compiled Ls, every storage precision.  The oracle's operator judges each
+solution at the solver's own target, 1e-10.
+"""
+import numpy as np
+import pytest
+
+from paper_1706_05843_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    (4, dict(b=1.0, c=0.0, pm=1, beta=-1.0)),
+    (8, dict(b=1.0, c=0.9, pm=-1, beta=0.7)),
+    (12, dict(b=1.2, c=-0.2, pm=1, beta=0.5)),
+    (16, dict(b=1.5, c=0.5, pm=-1, beta=0.0)),
+    (12, dict(b=2.0, c=1.0, pm=1, beta=-1.0)),
+]
+
+
+@pytest.mark.parametrize("Ls,kw", CASES)
+@pytest.mark.parametrize("inner", ["f64", "f32", "f16", "bf16"])
+def test_solution_judged_by_the_oracle(Ls, kw, inner):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import oracle as O
+    from paper_1706_05843_gb300 import binding as B
+    from paper_1706_05843_gb300 import build
+    build.build()
+    O.build()
+    dims = (4, 2, 4, 6)
+    act = dict(M5=1.8, m1=0.1, m2=1.0, m3=0.2, t_bc=-1, **kw)
+    U = I.gauge_field(dims, 0.5, 3)
+    phi = I.gaussian_fermion(dims, Ls, 1001)
+    o = O.Oracle(O.Action(dims=dims, Ls=Ls, **act), U)
+    s = B.Solver(U, dims, Ls, **act)
+    x = torch.from_numpy(phi).cuda()
+    for form, op in ((0, o.hsys), (1, o.k)):
+        sol, st = s.solve(x, tol=1e-10, inner=inner, rhs_form=form)
+        r = np.linalg.norm(phi - op(sol.cpu().numpy())) / np.linalg.norm(phi)
+        assert r <= 1e-10 * (1 + 1e-3), (form, r, st.inner_iters)
+    s.close()
