@@ -10,6 +10,8 @@
 // mma.sync and reduced into the FP32 gradient with atomics.
 #include "learned.h"
 
+#include <algorithm>
+
 namespace eofa {
 
 namespace {
@@ -19,11 +21,6 @@ __device__ __forceinline__ unsigned smem_u32(const void* p) {
 }
 __device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(sdst)), "l"(gsrc));
-}
-// L1-allocating copy: the neighbour rows of consecutive taps overlap
-// almost entirely within a CTA's 128 rows, so they are served from L1
-__device__ __forceinline__ void cp_async16_ca(void* sdst, const void* gsrc) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(smem_u32(sdst)), "l"(gsrc));
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N>
@@ -71,48 +68,79 @@ enum Epi { EPI_LEAKY_BF16 = 0, EPI_F32 = 1, EPI_DMASK_BF16 = 2 };
 // ---------------------------------------------------------------------------
 // The convolution on the 5th-generation tensor cores (tcgen05).
 //
-// A CTA owns 128 output rows (sites) x 32 output channels: the accumulator
-// is a 128-lane x 32-column FP32 block of tensor memory (TMEM), allocated by
-// warp 0.  Per tap, the 128 neighbour rows (32 BF16 channels each) and the
-// tap's 32 x 32 weight block are copied with cp.async (the rows through L1:
-// consecutive taps of a CTA read almost the same rows) into shared memory in
-// the tensor cores' canonical K-major layout without swizzle: 8-row x
-// 16-byte core matrices, 128 bytes apart along K and 512 bytes apart along
-// M (N); two buffers, so the copies of tap t+1 overlap the MMAs of tap t.
-// One thread issues the tap's two M128 x N32 x K16 MMAs (kind::f16, BF16 in,
-// FP32 accumulate) and commits them to the buffer's mbarrier, which frees
-// the buffer for tap t+2.  The epilogue: each warp reads its 32 TMEM lanes
-// (its threads' rows) with tcgen05.ld.  Every mbarrier wait is bounded; on
-// expiry the CTA records the event in tc_fault, skips its output, frees
-// its tensor memory and returns.
+// A CTA keeps all 81 weight blocks in shared memory (166 KB) and walks
+// columns: 128 rows of one slice's (z, y, x) volume over a range of t.  The
+// volume is numbered with a halo, [z][Y + 2][x + 2], so that every spatial
+// tap is a constant offset in that numbering: a time slice's rows for one dz
+// (a segment: 128 + 2 (line + 1) positions) are loaded once, in the canonical
+// no-swizzle K-major layout with 16-byte rows, and the nine (dy, dx) taps
+// read it through matrix descriptors that start at other rows.  Rows of the
+// halo are computed and dropped.
+//
+// One input slice t' serves the outputs t' - 1, t', t' + 1 (dt = 1, 0, -1) in
+// one M128 x N96 x K16 MMA: the accumulators of consecutive outputs are
+// consecutive 32-column slots of tensor memory, a ring of 16.  Walking t'
+// upwards keeps every output's sum in the order of the taps (dt, dz, dy, dx),
+// K16 halves innermost.  A slot is read out (tcgen05.ld), zeroed and given
+// back by the epilogue warps while the MMAs of the next slices run.
+//
+// Roles: warps 0-3 epilogue (one TMEM lane a thread), warp 4 one thread
+// issues the MMAs, warps 5-7 load segments (cp.async) through a ring.  Every
+// mbarrier wait is bounded; on expiry the CTA records the event in
+// g_tc_fault, every role leaves its loop, the copies and MMAs in flight are
+// waited for and the tensor memory is freed.
+//
+// What bounds it: shared-memory reads of the operands (7 KB an MMA, 56 clocks
+// at 128 bytes each, against 48 clocks of tensor work); the kernel it
+// replaces gathered the 128 neighbour rows of every tap through L1 (97% of
+// its peak, tensor pipe 7%).
 // ---------------------------------------------------------------------------
 __device__ int g_tc_fault;  // set when a bounded wait of the tcgen05 convolution expired
 
-constexpr int kTcStageA = 128 * 64;  // bytes of one A buffer (128 rows x 32 BF16)
-constexpr int kTcStageB = 32 * 64;   // bytes of one B buffer (32 rows x 32 BF16)
-// dynamic shared memory of an NST-buffer ring: buffers, NST mbarriers, the TMEM address
-constexpr int tc_smem_bytes(int nst) { return nst * (kTcStageA + kTcStageB) + 8 * nst + 16; }
-constexpr long kTcSpin = 1L << 22;   // mbarrier polls before a wait counts as expired
+constexpr int kCvRows = 128;                 // output positions of a tile (MMA M)
+constexpr int kCvSlots = 16;                 // accumulator slots of 32 columns
+constexpr int kCvWBytes = 81 * 32 * 32 * 2;  // the packed weights
+constexpr int kCvTapBytes = 96 * 32 * 2;     // one spatial tap: [q = ci / 8][n = 96][8]
+constexpr int kCvThreads = 256;
+constexpr int kCvLoaders = 96;
+constexpr int kCvMaxSeg = 6;
+constexpr int kCvBarBytes = (2 * kCvMaxSeg + 2 * kCvSlots + 2) * 8;
+constexpr int kCvSmemMax = 232448;
+constexpr long kTcSpin = 1L << 22;           // mbarrier polls before a wait counts as expired
 
-// byte offset of 16-byte chunk q (K elements 8q..8q+7) of row r in a
-// canonical no-swizzle K-major tile with 4 core matrices along K
-__device__ __forceinline__ int tc_off(int r, int q) { return ((r >> 3) * 4 + q) * 128 + (r & 7) * 16; }
-
-// shared-memory matrix descriptor: start, leading (K) and stride (M/N)
-// byte offsets, descriptor version 1, no swizzle
-__device__ __forceinline__ unsigned long long tc_desc(unsigned saddr) {
-    const unsigned long long lbo = 128, sbo = 512;
-    return (unsigned long long)((saddr >> 4) & 0x3FFF) | (((lbo >> 4) & 0x3FFF) << 16) |
-           (((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
+// shared-memory matrix descriptor of a canonical K-major tile without
+// swizzle: start and the stride between core matrices along K (lbo) in the
+// low word, 128 bytes between 8-row groups and descriptor version 1 in the
+// high word.  Adding n to the low word moves the start by 16 n bytes.
+__device__ __forceinline__ unsigned tc_desc_lo(unsigned saddr, unsigned lbo) {
+    return ((saddr >> 4) & 0x3FFF) | ((lbo >> 4) << 16);
 }
-// instruction descriptor: D FP32, A and B BF16, both K-major, N = 32, M = 128
-constexpr unsigned kTcIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((32u >> 3) << 17) | ((128u >> 4) << 24);
-
+__device__ __forceinline__ unsigned long long tc_desc(unsigned lo) {
+    return ((unsigned long long)((128u >> 4) | (1u << 14)) << 32) | lo;
+}
+// instruction descriptor: D FP32, A and B BF16, both K-major, M = 128
+__device__ __forceinline__ unsigned tc_idesc(unsigned n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
+}
+__device__ __forceinline__ void tc_mma(unsigned d, unsigned a_lo, unsigned b_lo, unsigned idesc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 1, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+        "l"(tc_desc(a_lo)), "l"(tc_desc(b_lo)), "r"(idesc)
+        : "memory");
+}
+__device__ __forceinline__ void tc_commit(unsigned bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ void mbar_init(unsigned a, unsigned n) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(n) : "memory");
 }
-// true when the phase of the given parity has completed; gives up after kTcSpin polls
-__device__ __forceinline__ bool mbar_wait(unsigned a, unsigned parity) {
+__device__ __forceinline__ void mbar_arrive(unsigned a) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(a) : "memory");
+}
+// true when the phase of the given parity has completed; gives up after
+// kTcSpin polls (setting *fault) or when another role has
+__device__ __forceinline__ bool mbar_wait(unsigned a, unsigned parity, volatile int* fault) {
     for (long i = 0; i < kTcSpin; ++i) {
         unsigned done;
         asm volatile(
@@ -122,156 +150,279 @@ __device__ __forceinline__ bool mbar_wait(unsigned a, unsigned parity) {
             : "r"(a), "r"(parity)
             : "memory");
         if (done) return true;
+        if ((i & 63) == 63 && *fault) return false;
     }
+    *fault = 1;
     return false;
 }
 
-template <int EPI, int NST>
-__global__ void __launch_bounds__(128) k_conv_tc(const bf16* __restrict__ in, const bf16* __restrict__ W,
-                                                 void* __restrict__ out, const bf16* __restrict__ mask, ConvGeom g) {
-    extern __shared__ __align__(1024) unsigned char tc_smem[];
-    unsigned char* sA = tc_smem;                         // [NST][kTcStageA]
-    unsigned char* sB = tc_smem + NST * kTcStageA;       // [NST][kTcStageB]
-    unsigned long long* bar = reinterpret_cast<unsigned long long*>(sB + NST * kTcStageB);  // [NST]
-    unsigned* tmem_slot = reinterpret_cast<unsigned*>(bar + NST);
-    __shared__ int s_fault;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const long rows = (long)g.V * g.S;
-    const long gi = (long)blockIdx.x * 128 + tid;
-    const bool rv = gi < rows;
-    const int sl = rv ? (int)(gi / g.V) : 0;
-    const int site = rv ? (int)(gi - (long)sl * g.V) : 0;
-    const Coord c = coord_of(g, site);
+// how the lattice is cut into columns (host; the same for every layer)
+struct ConvPlan {
+    int nxb, wb;      // blocks in x and their width
+    int line, plane;  // positions of a haloed line (wb + 2) and plane ((Y + 2) line)
+    int vol;          // positions of one block's volume
+    int tiles;        // 128-position tiles of it
+    int nt, nts;      // outputs of a column along t, columns along t
+    int np, nseg;     // positions of a segment, ring of segments
+    long cols;
+};
+
+template <int EPI>
+__global__ void __launch_bounds__(kCvThreads, 1)
+    k_conv_tc(const bf16* __restrict__ in, const bf16* __restrict__ W, void* __restrict__ out,
+              const bf16* __restrict__ mask, ConvGeom g, ConvPlan pl, int ostride) {
+    extern __shared__ __align__(128) unsigned char tc_smem[];
+    unsigned char* sW = tc_smem;                      // [27][4][96][16 bytes]
+    unsigned char* sA = tc_smem + kCvWBytes;          // [nseg][4][np][16 bytes]
+    int2* tab = reinterpret_cast<int2*>(sA + (size_t)pl.nseg * pl.np * 64);  // [np]: (y X + x, z) of a position
+    unsigned long long* bars = reinterpret_cast<unsigned long long*>(tab + pl.np);
+    const unsigned b_full = smem_u32(bars), b_empty = b_full + 8 * kCvMaxSeg;
+    const unsigned b_accf = b_empty + 8 * kCvMaxSeg, b_acce = b_accf + 8 * kCvSlots, b_fin = b_acce + 8 * kCvSlots;
+    __shared__ unsigned s_tmem;
+    __shared__ volatile int s_fault;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
-        for (int b = 0; b < NST; ++b) mbar_init(smem_u32(bar + b), 1);
         s_fault = 0;
+        for (int i = 0; i < pl.nseg; ++i) {
+            mbar_init(b_full + 8 * i, kCvLoaders);
+            mbar_init(b_empty + 8 * i, 1);
+        }
+        for (int i = 0; i < kCvSlots; ++i) {
+            mbar_init(b_accf + 8 * i, 1);
+            mbar_init(b_acce + 8 * i, kCvRows);
+        }
+        mbar_init(b_fin, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;" ::"r"(smem_u32(tmem_slot))
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&s_tmem))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    for (int i = tid; i < kCvWBytes / 16; i += kCvThreads) cp_async16(sW + 16 * i, W + 8 * i);
+    cp_commit();
+    cp_wait<0>();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const unsigned tmem = *tmem_slot;
+    const unsigned tmem = s_tmem;
 
-    auto load_tap = [&](int tap, int buf) {
-        unsigned char* a = sA + buf * kTcStageA;
-        if (rv) {
-            const int ns = shifted_site(g, c, tap);
-            const bf16* src = in + ((long)sl * g.V + ns) * kCP;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) cp_async16_ca(a + tc_off(tid, q), src + q * 8);
-        } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) *reinterpret_cast<uint4*>(a + tc_off(tid, q)) = make_uint4(0u, 0u, 0u, 0u);
-        }
-        const int wr = tid >> 2, wq = tid & 3;
-        cp_async16(sB + buf * kTcStageB + tc_off(wr, wq), W + ((long)tap * 32 + wr) * 32 + wq * 8);
-        cp_commit();
+    // column -> (slice, x block, tile, first output t, outputs)
+    struct Col {
+        int sl, xb, p0, t0, nt;
+    };
+    auto column = [&](long c) {
+        Col k;
+        k.t0 = (int)(c % pl.nts) * pl.nt;
+        c /= pl.nts;
+        k.p0 = (int)(c % pl.tiles) * kCvRows;
+        c /= pl.tiles;
+        k.xb = (int)(c % pl.nxb);
+        k.sl = (int)(c / pl.nxb);
+        k.nt = min(pl.nt, g.T - k.t0);
+        return k;
+    };
+    auto zero_slot = [&](unsigned taddr) {
+        const unsigned z = 0u;
+        asm volatile(
+            "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
+            "%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
+            "r"(z)
+            : "memory");
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     };
 
-    // ring of NST buffers: taps 0 .. NST-2 are in flight before the first
-    // MMA; tap t + NST - 1 goes into the buffer of tap t - 1 once the MMAs
-    // of tap t - 1 have been committed as complete.  Tap t is the
-    // (t / NST)-th commit on bar[t % NST] (phase parity (t / NST) & 1).
-    bool ok = true;
-    for (int t = 0; t < NST - 1; ++t) load_tap(t, t);
-    for (int tap = 0; tap < 81; ++tap) {
-        const int buf = tap % NST;
-        const int nx = tap + NST - 1;
-        if (nx < 81) {
-            if (tap >= 1) {
-                const int pt = tap - 1;
-                if (!mbar_wait(smem_u32(bar + pt % NST), (pt / NST) & 1)) ok = false;
-            }
-            load_tap(nx, nx % NST);
-            cp_wait<NST - 1>();
-        } else {
-            cp_wait<0>();
+    if (warp < 4) {
+        // ------------------------------------------------ epilogue
+        const unsigned tlane = tmem + ((unsigned)(warp * 32) << 16);
+        for (int i = 0; i < kCvSlots; ++i) {
+            zero_slot(tlane + 32 * i);
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            mbar_arrive(b_acce + 8 * i);
         }
-        // this thread's copies of tap's buffer are visible to the tensor cores
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const unsigned a0 = smem_u32(sA + buf * kTcStageA), b0 = smem_u32(sB + buf * kTcStageB);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const unsigned long long ad = tc_desc(a0 + h * 256), bd = tc_desc(b0 + h * 256);
-                const unsigned acc = (tap > 0 || h > 0) ? 1u : 0u;
+        long o = 0;
+        bool ok = true;
+        for (long cc = blockIdx.x; cc < pl.cols && ok; cc += gridDim.x) {
+            const Col k = column(cc);
+            const int p = k.p0 + tid;
+            const int z = p / pl.plane, r = p - z * pl.plane, yp = r / pl.line, xp = r - yp * pl.line;
+            const int x = k.xb * pl.wb + xp - 1;
+            const bool valid = p < pl.vol && yp >= 1 && yp <= g.Y && xp >= 1 && xp <= pl.wb && x < g.X;
+            const long site0 = (long)k.sl * g.V + ((long)z * g.Y + (yp - 1)) * g.X + x;
+            for (int i = 0; i < k.nt; ++i, ++o) {
+                const int slot = (int)(o % kCvSlots);
+                ok = __all_sync(0xffffffffu, mbar_wait(b_accf + 8 * slot, (unsigned)(o / kCvSlots) & 1, &s_fault));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                unsigned r32[32];
                 asm volatile(
-                    "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-                    "l"(ad), "l"(bd), "r"(kTcIdesc), "r"(acc)
-                    : "memory");
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_u32(bar + buf))
-                         : "memory");
-        }
-    }
-    // the last commit covers every MMA of the CTA
-    if (!mbar_wait(smem_u32(bar + 80 % NST), (80 / NST) & 1)) ok = false;
-    if (!ok) s_fault = 1;
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!s_fault) {
-        unsigned r[32];
-        const unsigned taddr = tmem + ((unsigned)(warp * 32) << 16);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-            "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-              "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]),
-              "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]),
-              "=r"(r[30]), "=r"(r[31])
-            : "r"(taddr));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (rv) {
-            if constexpr (EPI == EPI_F32) {
-                float4* o = reinterpret_cast<float4*>(reinterpret_cast<float*>(out) + gi * kCP);
+                    "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+                    "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                    : "=r"(r32[0]), "=r"(r32[1]), "=r"(r32[2]), "=r"(r32[3]), "=r"(r32[4]), "=r"(r32[5]),
+                      "=r"(r32[6]), "=r"(r32[7]), "=r"(r32[8]), "=r"(r32[9]), "=r"(r32[10]), "=r"(r32[11]),
+                      "=r"(r32[12]), "=r"(r32[13]), "=r"(r32[14]), "=r"(r32[15]), "=r"(r32[16]), "=r"(r32[17]),
+                      "=r"(r32[18]), "=r"(r32[19]), "=r"(r32[20]), "=r"(r32[21]), "=r"(r32[22]), "=r"(r32[23]),
+                      "=r"(r32[24]), "=r"(r32[25]), "=r"(r32[26]), "=r"(r32[27]), "=r"(r32[28]), "=r"(r32[29]),
+                      "=r"(r32[30]), "=r"(r32[31])
+                    : "r"(tlane + 32 * slot));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                zero_slot(tlane + 32 * slot);
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                mbar_arrive(b_acce + 8 * slot);
+                if (!valid) continue;
+                const long gi = site0 + (long)(k.t0 + i) * g.Z * g.Y * g.X;
+                if constexpr (EPI == EPI_F32) {
+                    float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(out) + gi * ostride);
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    o[q] = make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
-                                       __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
-            } else {
-                uint4* o = reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out) + gi * kCP);
-                const uint4* mk = reinterpret_cast<const uint4*>(mask + gi * kCP);
+                    for (int q = 0; q < 8; ++q)
+                        if (4 * q < ostride)
+                            dst[q] = make_float4(__uint_as_float(r32[4 * q]), __uint_as_float(r32[4 * q + 1]),
+                                                 __uint_as_float(r32[4 * q + 2]), __uint_as_float(r32[4 * q + 3]));
+                } else {
+                    uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<bf16*>(out) + gi * kCP);
+                    const uint4* mk = reinterpret_cast<const uint4*>(mask + gi * kCP);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint4 mq = make_uint4(0u, 0u, 0u, 0u);
-                    if constexpr (EPI == EPI_DMASK_BF16) mq = mk[q];
-                    const unsigned* mw = reinterpret_cast<const unsigned*>(&mq);
-                    unsigned w[4];
+                    for (int q = 0; q < 4; ++q) {
+                        uint4 mq = make_uint4(0u, 0u, 0u, 0u);
+                        if constexpr (EPI == EPI_DMASK_BF16) mq = mk[q];
+                        const unsigned* mw = reinterpret_cast<const unsigned*>(&mq);
+                        unsigned w[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        float v0 = __uint_as_float(r[8 * q + 2 * e]), v1 = __uint_as_float(r[8 * q + 2 * e + 1]);
-                        if constexpr (EPI == EPI_LEAKY_BF16) {
-                            v0 = v0 > 0.f ? v0 : kLeaky * v0;
-                            v1 = v1 > 0.f ? v1 : kLeaky * v1;
-                        } else {
-                            const __nv_bfloat162 m = *reinterpret_cast<const __nv_bfloat162*>(&mw[e]);
-                            v0 *= __bfloat162float(m.x) > 0.f ? 1.f : kLeaky;
-                            v1 *= __bfloat162float(m.y) > 0.f ? 1.f : kLeaky;
+                        for (int e = 0; e < 4; ++e) {
+                            float v0 = __uint_as_float(r32[8 * q + 2 * e]), v1 = __uint_as_float(r32[8 * q + 2 * e + 1]);
+                            if constexpr (EPI == EPI_LEAKY_BF16) {
+                                v0 = v0 > 0.f ? v0 : kLeaky * v0;
+                                v1 = v1 > 0.f ? v1 : kLeaky * v1;
+                            } else {
+                                const __nv_bfloat162 m = *reinterpret_cast<const __nv_bfloat162*>(&mw[e]);
+                                v0 *= __bfloat162float(m.x) > 0.f ? 1.f : kLeaky;
+                                v1 *= __bfloat162float(m.y) > 0.f ? 1.f : kLeaky;
+                            }
+                            const __nv_bfloat162 b = __floats2bfloat162_rn(v0, v1);
+                            w[e] = *reinterpret_cast<const unsigned*>(&b);
                         }
-                        const __nv_bfloat162 b = __floats2bfloat162_rn(v0, v1);
-                        w[e] = *reinterpret_cast<const unsigned*>(&b);
+                        dst[q] = make_uint4(w[0], w[1], w[2], w[3]);
                     }
-                    o[q] = make_uint4(w[0], w[1], w[2], w[3]);
                 }
             }
         }
-    } else if (tid == 0) {
-        atomicExch(&g_tc_fault, 1);
+    } else if (warp == 4) {
+        // ------------------------------------------------ MMA issue
+        if (lane == 0) {
+            const unsigned hA = 2 * (unsigned)pl.np, hB = 2 * 96;  // 16-byte units between the K16 halves
+            const unsigned line = (unsigned)pl.line;
+            const unsigned w0 = tc_desc_lo(smem_u32(sW), 96 * 16);
+            unsigned o = 0;           // outputs of the columns before this one
+            unsigned slot = 0, par = 0;  // segment ring
+            bool ok = true;
+            for (long cc = blockIdx.x; cc < pl.cols && ok; cc += gridDim.x) {
+                const int nt = column(cc).nt;
+                for (int i = 0; i < nt + 2 && ok; ++i) {  // input slice t0 - 1 + i serves outputs i - 2, i - 1, i
+                    const int lo = max(0, i - 2), hi = min(nt - 1, i);
+                    if (i < nt) {
+                        const unsigned q = o + (unsigned)i;  // the output this slice starts
+                        if (!mbar_wait(b_acce + 8 * (q % kCvSlots), (q / kCvSlots) & 1, &s_fault)) {
+                            ok = false;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    }
+                    const unsigned s0 = (o + (unsigned)lo) % kCvSlots, n = (unsigned)(hi - lo + 1);
+                    const unsigned n1 = min(n, kCvSlots - s0), n2 = n - n1;  // n2: the part that wraps to slot 0
+                    const unsigned wlo = w0 + (unsigned)(lo - (i - 2)) * 32;
+                    const unsigned d = tmem + 32 * s0, id1 = tc_idesc(32 * n1), id2 = tc_idesc(32 * n2);
+                    for (int dz = 0; dz < 3; ++dz) {
+                        if (!mbar_wait(b_full + 8 * slot, par, &s_fault)) {
+                            ok = false;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const unsigned as = tc_desc_lo(smem_u32(sA) + slot * (unsigned)pl.np * 64, (unsigned)pl.np * 16);
+                        const unsigned ws = wlo + (unsigned)dz * 9 * (kCvTapBytes / 16);
+                        if (n2 == 0) {
+#pragma unroll
+                            for (unsigned tp = 0; tp < 9; ++tp) {
+                                const unsigned at = as + (tp / 3) * line + tp % 3, wt = ws + tp * (kCvTapBytes / 16);
+                                tc_mma(d, at, wt, id1);
+                                tc_mma(d, at + hA, wt + hB, id1);
+                            }
+                        } else {
+#pragma unroll 1
+                            for (unsigned tp = 0; tp < 9; ++tp) {
+                                const unsigned at = as + (tp / 3) * line + tp % 3, wt = ws + tp * (kCvTapBytes / 16);
+                                tc_mma(d, at, wt, id1);
+                                tc_mma(tmem, at, wt + n1 * 32, id2);
+                                tc_mma(d, at + hA, wt + hB, id1);
+                                tc_mma(tmem, at + hA, wt + hB + n1 * 32, id2);
+                            }
+                        }
+                        tc_commit(b_empty + 8 * slot);
+                        if (++slot == (unsigned)pl.nseg) slot = 0, par ^= 1;
+                    }
+                    if (ok && i >= 2) tc_commit(b_accf + 8 * ((o + (unsigned)i - 2) % kCvSlots));
+                }
+                o += (unsigned)nt;
+            }
+            // every MMA issued has completed before the tensor memory is freed
+            volatile int none = 0;
+            tc_commit(b_fin);
+            mbar_wait(b_fin, 0, &none);
+        }
+        __syncwarp();
+    } else {
+        // ------------------------------------------------ segment loads
+        // a warp loads a third of the positions; four lanes a position
+        const int part = (pl.np + 2) / 3, lo = (warp - 5) * part, hi = min(pl.np, lo + part);
+        int slot = 0, par = 1;  // the first round finds the ring empty
+        int pend = -1;          // slot whose copies have not been published yet
+        bool ok = true;
+        for (long cc = blockIdx.x; cc < pl.cols && ok; cc += gridDim.x) {
+            const Col c = column(cc);
+            __syncwarp();
+            for (int pos = lo + lane; pos < hi; pos += 32) {
+                // positions outside the volume feed dropped rows only
+                const int p = min(max(c.p0 - pl.line - 1 + pos, 0), pl.vol - 1);
+                const int z = p / pl.plane, r = p - z * pl.plane, yp = r / pl.line;
+                const int y = wrapi(yp - 1, g.Y), x = wrapi(c.xb * pl.wb + (r - yp * pl.line) - 1, g.X);
+                tab[pos] = make_int2(y * g.X + x, z);
+            }
+            __syncwarp();
+            for (int i = 0; i < c.nt + 2 && ok; ++i) {
+                int t = c.t0 - 1 + i;
+                t = t < 0 ? t + g.T : (t >= g.T ? t - g.T : t);
+                const bf16* base = in + ((long)c.sl * g.V + (long)t * g.Z * g.Y * g.X) * kCP + 8 * (lane & 3);
+                for (int dz = -1; dz <= 1; ++dz) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(b_empty + 8 * slot, (unsigned)par, &s_fault));
+                    if (!ok) break;
+                    unsigned char* dst = sA + ((size_t)slot * 4 + (lane & 3)) * pl.np * 16;
+                    for (int pos = lo + (lane >> 2); pos < hi; pos += 8) {
+                        const int2 e = tab[pos];
+                        const long n = (long)wrapi(e.y + dz, g.Z) * g.Y * g.X + e.x;
+                        cp_async16(dst + pos * 16, base + n * kCP);
+                    }
+                    cp_commit();
+                    if (pend >= 0) {  // the previous segment has arrived
+                        cp_wait<1>();
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        mbar_arrive(b_full + 8 * pend);
+                    }
+                    pend = slot;
+                    if (++slot == pl.nseg) slot = 0, par ^= 1;
+                }
+            }
+        }
+        cp_wait<0>();
+        if (ok && pend >= 0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            mbar_arrive(b_full + 8 * pend);
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem) : "memory");
+    if (tid == 0 && s_fault) atomicExch(&g_tc_fault, 1);
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
 // dW[tap][co][ci] += sum_rows dy[row][co] * in[shift(row, tap)][ci]
@@ -372,6 +523,13 @@ __global__ void __launch_bounds__(128) k_conv_wgrad(const bf16* __restrict__ in,
     }
 }
 
+// place of W[tap][co][ci] in the packed weights: per spatial tap [ci / 8][n][8]
+// with n = 32 (1 - dt) + co, dt = -1, 0, 1 (the outputs of an input slice in
+// ascending t)
+__device__ __forceinline__ int packed_w(int tap, int co, int ci) {
+    return (((tap % 27) * 4 + (ci >> 3)) * 96 + 32 * (2 - tap / 27) + co) * 8 + (ci & 7);
+}
+
 // public FP32 weights -> padded BF16 forward and mirrored/transposed backward operands
 __global__ void k_convert(const float* __restrict__ Wm, bf16* __restrict__ Wf, bf16* __restrict__ Wb, int cout,
                           int cin) {
@@ -379,9 +537,8 @@ __global__ void k_convert(const float* __restrict__ Wm, bf16* __restrict__ Wf, b
     if (e >= 81 * 32 * 32) return;
     const int tap = e / 1024, co = (e / 32) % 32, ci = e % 32;
     const float v = (co < cout && ci < cin) ? Wm[((long)tap * cout + co) * cin + ci] : 0.f;
-    Wf[e] = __float2bfloat16(v);
-    // Wb[80 - tap][ci][co] = W[tap][co][ci]
-    Wb[((long)(80 - tap) * 32 + ci) * 32 + co] = __float2bfloat16(v);
+    Wf[packed_w(tap, co, ci)] = __float2bfloat16(v);
+    Wb[packed_w(80 - tap, ci, co)] = __float2bfloat16(v);
 }
 
 __global__ void k_pack(const float* __restrict__ in24, bf16* __restrict__ a32, long rows) {
@@ -426,14 +583,48 @@ __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float
 
 inline int blocks_for(long n, int bt) { return (int)((n + bt - 1) / bt); }
 
-constexpr int kTcStages = 2;  // deeper rings measured no faster
+// The cut of a lattice into columns.  x is split into blocks of at most 64
+// (a segment then leaves room for at least three in the ring); t is split so
+// that the columns fill the SMs: the cost of a split is its rounds of
+// columns times the input slices a column reads (two more than its outputs).
+ConvPlan conv_plan(const ConvGeom& g, int sms) {
+    ConvPlan p;
+    p.nxb = (g.X + 63) / 64;
+    p.wb = (g.X + p.nxb - 1) / p.nxb;
+    p.line = p.wb + 2;
+    p.plane = (g.Y + 2) * p.line;
+    p.vol = g.Z * p.plane;
+    p.tiles = (p.vol + kCvRows - 1) / kCvRows;
+    p.np = kCvRows + 2 * p.line + 2;
+    p.nseg = std::min(kCvMaxSeg, (kCvSmemMax - 1024 - kCvWBytes - kCvBarBytes - p.np * 8) / (p.np * 64));
+    const long base = (long)g.S * p.nxb * p.tiles;
+    double best = 0.0;
+    p.nt = g.T;
+    for (int n = 1; n <= g.T; ++n) {  // n columns along t
+        const int nt = (g.T + n - 1) / n;
+        const long cols = base * ((g.T + nt - 1) / nt);
+        const double cost = (double)((cols + sms - 1) / sms) * (nt + 2);
+        if (n == 1 || cost < best) best = cost, p.nt = nt;
+        if (cols > 64L * sms) break;
+    }
+    p.nts = (g.T + p.nt - 1) / p.nt;
+    p.cols = base * p.nts;
+    return p;
+}
 
 template <int EPI>
-cudaError_t conv(const bf16* in, const bf16* W, void* out, const bf16* mask, const ConvGeom& g, cudaStream_t st) {
-    const long rows = (long)g.V * g.S;
-    if (rows == 0) return cudaSuccess;
-    static_assert(tc_smem_bytes(kTcStages) <= 48 * 1024, "no opt-in shared memory needed");
-    k_conv_tc<EPI, kTcStages><<<blocks_for(rows, 128), 128, tc_smem_bytes(kTcStages), st>>>(in, W, out, mask, g);
+cudaError_t conv(const bf16* in, const bf16* W, void* out, const bf16* mask, const ConvGeom& g, cudaStream_t st,
+                 int ostride = kCP) {
+    if ((long)g.V * g.S == 0) return cudaSuccess;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_conv_tc<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCvSmemMax - 1024);
+    if (e != cudaSuccess) return e;
+    const ConvPlan p = conv_plan(g, sms);
+    const size_t smem = kCvWBytes + (size_t)p.np * (p.nseg * 64 + 8) + kCvBarBytes;
+    k_conv_tc<EPI><<<(int)std::min<long>(p.cols, sms), kCvThreads, smem, st>>>(in, W, out, mask, g, p, ostride);
     return cudaGetLastError();
 }
 
