@@ -2260,13 +2260,35 @@ struct DevBuf {
     }
 };
 
-cudaError_t net_alloc(DevBuf& B, NetDev& n) {
-    cudaError_t e = B.get(&n.Wm, (size_t)kNetWeights);
-    for (int l = 0; l < kNetLayers && e == cudaSuccess; ++l) {
-        e = B.get(&n.Wf[l], (size_t)81 * 32 * 32);
-        if (e == cudaSuccess) e = B.get(&n.Wb[l], (size_t)81 * 32 * 32);
+// One device allocation for the work space of a call (a cudaMalloc and
+// cudaFree pair costs 0.1 to 0.3 ms): the first pass of `lay` over it adds up
+// the sizes, the second hands out the pieces.
+struct WorkSpace {
+    unsigned char* base = nullptr;
+    size_t used = 0;
+    ~WorkSpace() { cudaFree(base); }
+    template <typename T>
+    void get(T** out, size_t n) {
+        *out = reinterpret_cast<T*>(base + used);
+        used += (n * sizeof(T) + 255) / 256 * 256;
     }
-    return e;
+    template <typename F>
+    cudaError_t make(F&& lay) {
+        lay(*this);
+        const cudaError_t e = cudaMalloc((void**)&base, used);
+        if (e != cudaSuccess) return e;
+        used = 0;
+        lay(*this);
+        return cudaSuccess;
+    }
+};
+
+void net_lay(WorkSpace& B, NetDev& n) {
+    B.get(&n.Wm, (size_t)kNetWeights);
+    for (int l = 0; l < kNetLayers; ++l) {
+        B.get(&n.Wf[l], (size_t)81 * 32 * 32);
+        B.get(&n.Wb[l], (size_t)81 * 32 * 32);
+    }
 }
 
 bool conv_geom(const int dims[4], int nslices, ConvGeom* g) {
@@ -2289,20 +2311,18 @@ extern "C" eofa_status eofa_net_forward(const float* weights, const int dims[4],
     if (!weights || !in || !out || !conv_geom(dims, nslices, &g)) return EOFA_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     const long rows = (long)g.V * g.S;
-    DevBuf B;
+    WorkSpace B;
     NetDev n;
-    bf16 *a0, *a1, *a2;
-    float* o32;
-    cudaError_t e = net_alloc(B, n);
-    if (e == cudaSuccess) e = B.get(&a0, rows * kCP);
-    if (e == cudaSuccess) e = B.get(&a1, rows * kCP);
-    if (e == cudaSuccess) e = B.get(&a2, rows * kCP);
-    if (e == cudaSuccess) e = B.get(&o32, rows * kCP);
+    bf16 *a0, *a1;
+    cudaError_t e = B.make([&](WorkSpace& b) {
+        net_lay(b, n);
+        b.get(&a0, rows * kCP);
+        b.get(&a1, rows * kCP);
+    });
     if (e == cudaSuccess) e = cudaMemcpyAsync(n.Wm, weights, sizeof(float) * kNetWeights, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = net_convert(n, st);
     if (e == cudaSuccess) e = pack_act((const float*)in, a0, rows, st);
-    if (e == cudaSuccess) e = net_forward(n, g, a0, a1, a2, o32, st);
-    if (e == cudaSuccess) e = unpack_out(o32, (float*)out, rows, st);
+    if (e == cudaSuccess) e = net_forward(n, g, a0, a1, a0, (float*)out, st, 24);  // a0 -> a1 -> a0 -> out
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     int fault = 0;
     if (e == cudaSuccess) e = net_fault(&fault);
@@ -2316,26 +2336,22 @@ extern "C" eofa_status eofa_net_backward(const float* weights, const int dims[4]
     if (!weights || !in || !dout || !dweights || !conv_geom(dims, nslices, &g)) return EOFA_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     const long rows = (long)g.V * g.S;
-    DevBuf B;
+    WorkSpace B;
     NetDev n;
     bf16 *a0, *a1, *a2, *dob, *d1, *d2;
-    float *o32, *dout32, *dW, *din32 = nullptr;
-    cudaError_t e = net_alloc(B, n);
-    bf16** bufs[] = {&a0, &a1, &a2, &dob, &d1, &d2};
-    for (auto b : bufs)
-        if (e == cudaSuccess) e = B.get(b, rows * kCP);
-    if (e == cudaSuccess) e = B.get(&o32, rows * kCP);
-    if (e == cudaSuccess) e = B.get(&dout32, rows * kCP);
-    if (e == cudaSuccess) e = B.get(&dW, (size_t)kNetWeights);
-    if (e == cudaSuccess && din) e = B.get(&din32, rows * kCP);
+    float* dW;
+    cudaError_t e = B.make([&](WorkSpace& b) {
+        net_lay(b, n);
+        for (bf16** p : {&a0, &a1, &a2, &dob, &d1, &d2}) b.get(p, rows * kCP);
+        b.get(&dW, (size_t)kNetWeights);
+    });
     if (e == cudaSuccess) e = cudaMemcpyAsync(n.Wm, weights, sizeof(float) * kNetWeights, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(dW, 0, sizeof(float) * kNetWeights, st);
     if (e == cudaSuccess) e = net_convert(n, st);
     if (e == cudaSuccess) e = pack_act((const float*)in, a0, rows, st);
-    if (e == cudaSuccess) e = net_forward(n, g, a0, a1, a2, o32, st);
-    if (e == cudaSuccess) e = pad_f32((const float*)dout, dout32, rows, st);
-    if (e == cudaSuccess) e = net_backward(n, g, a0, a1, a2, dout32, dW, din32, dob, d1, d2, st);
-    if (e == cudaSuccess && din) e = unpack_out(din32, (float*)din, rows, st);
+    if (e == cudaSuccess) e = net_hidden(n, g, a0, a1, a2, st);
+    if (e == cudaSuccess) e = pack_act((const float*)dout, dob, rows, st);
+    if (e == cudaSuccess) e = net_backward(n, g, a0, a1, a2, dob, dW, (float*)din, d1, d2, st, 24);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dweights, dW, sizeof(float) * kNetWeights, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     int fault = 0;
@@ -2678,7 +2694,8 @@ extern "C" eofa_status eofa_train_preconditioner(eofa_ctx* ctx, const void* cons
         Geom gB = g;  // loss over B slices of the full lattice
         CK(loss_grad(o32, et, wdev, dout, gB, B, red(c, FIN_STORE, 4), st), "loss");
         CK(cudaMemsetAsync(dW, 0, sizeof(float) * kNetWeights, st), "memset");
-        CK(net_backward(c->net, cgB, a0, a1, a2, dout, dW, nullptr, dob, d1, d2, st), "backward");
+        CK(to_bf16(dout, dob, (long)B * V * kCP, st), "convert");
+        CK(net_backward(c->net, cgB, a0, a1, a2, dob, dW, nullptr, d1, d2, st), "backward");
         CK(adam_step(c->net.Wm, dW, am, av, kNetWeights, (float)opts->lr, 0.9f, 0.999f, 1e-8f, step + 1, st), "adam");
         CK(net_convert(c->net, st), "convert");
         if (step == 0 || step == steps - 1) {

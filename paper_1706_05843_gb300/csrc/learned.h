@@ -37,27 +37,28 @@ struct ConvGeom {
 // device copies of one network
 struct NetDev {
     float* Wm = nullptr;          // master FP32, public layout
-    bf16* Wf[3] = {};             // forward operands [81][32 co][32 ci], zero padded
-    bf16* Wb[3] = {};             // backward-data operands [81][32 ci][32 co], taps mirrored
+    bf16* Wf[3] = {};             // forward operands, packed for the convolution (81 x 32 x 32, zero padded)
+    bf16* Wb[3] = {};             // backward-data operands, taps mirrored and transposed, packed likewise
 };
 
-// activations [S][V][32] BF16; out [S][V][32] FP32 (channels >= 24 are zero)
+// activations [S][V][32] BF16; out FP32 rows of ostride (24 or 32) floats
+// (channels >= 24 are zero); net_hidden: the two hidden layers alone
 cudaError_t net_convert(const NetDev& n, cudaStream_t st);
+cudaError_t net_hidden(const NetDev& n, const ConvGeom& g, const bf16* a0, bf16* a1, bf16* a2, cudaStream_t st);
 cudaError_t net_forward(const NetDev& n, const ConvGeom& g, const bf16* a0, bf16* a1, bf16* a2, float* out,
-                        cudaStream_t st);
-// gradients: dout [S][V][32] FP32 -> dW (FP32 public layout, accumulated), din [S][V][32] FP32 or NULL;
-// work buffers d1, d2 [S][V][32] BF16 and dob [S][V][32] BF16.
+                        cudaStream_t st, int ostride = kCP);
+// gradients: dob = dL/d(out) [S][V][32] BF16 -> dW (FP32 public layout, accumulated), din FP32 rows of dstride
+// floats or NULL; work buffers d1, d2 [S][V][32] BF16.
 cudaError_t net_backward(const NetDev& n, const ConvGeom& g, const bf16* a0, const bf16* a1, const bf16* a2,
-                         const float* dout, float* dW, float* din, bf16* dob, bf16* d1, bf16* d2,
-                         cudaStream_t st);
+                         const bf16* dob, float* dW, float* din, bf16* d1, bf16* d2, cudaStream_t st,
+                         int dstride = kCP);
+cudaError_t to_bf16(const float* a, bf16* b, long n, cudaStream_t st);
 // after a synchronisation: *fault = 1 (and the flag cleared) when a
 // convolution gave up on a bounded wait and skipped its output since the
 // last call; the results computed meanwhile are not valid
 cudaError_t net_fault(int* fault);
-// FP32 [S][V][24] <-> BF16/FP32 [S][V][32]
+// FP32 [S][V][24] -> BF16 [S][V][32]
 cudaError_t pack_act(const float* in24, bf16* a32, long rows, cudaStream_t st);
-cudaError_t unpack_out(const float* out32, float* out24, long rows, cudaStream_t st);
-cudaError_t pad_f32(const float* in24, float* out32, long rows, cudaStream_t st);
 // Adam on the FP32 master weights
 cudaError_t adam_step(float* w, const float* g, float* m, float* v, long n, float lr, float b1, float b2,
                       float eps, int t, cudaStream_t st);
