@@ -395,16 +395,6 @@ cudaError_t blas_hop_input(VecRef out, VecRef psi, long n5, int Ls, bool chi, do
 // ---------------------------------------------------------------------------
 // layout conversion: canonical complex128 <-> internal FP64, one parity
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ long lex_of(const Geom& g, long xcb, int par) {
-    int rem = (int)xcb;
-    const int xh = rem % g.Xh; rem /= g.Xh;
-    const int y = rem % g.Y; rem /= g.Y;
-    const int z = rem % g.Z;
-    const int t = rem / g.Z;
-    const int x = 2 * xh + ((par + y + z + t) & 1);
-    return (((long)t * g.Z + z) * g.Y + y) * g.X + x;
-}
-
 // g5r5: read slice Ls-1-s and flip the sign of spins 2, 3 (gamma_5 R_5)
 __global__ void __launch_bounds__(BT) k_import(VecRef dst, const double* __restrict__ src, Geom g, int par,
                                                int g5r5) {
@@ -413,7 +403,7 @@ __global__ void __launch_bounds__(BT) k_import(VecRef dst, const double* __restr
     if (t >= n5) return;
     const long xcb = t / g.Ls;
     const int s = (int)(t - xcb * g.Ls);
-    const long lex = lex_of(g, xcb, par);
+    const long lex = lex_site(g, xcb, par);
     const int ss = g5r5 ? g.Ls - 1 - s : s;
     const double2* p = reinterpret_cast<const double2*>(src) + (lex * g.Ls + ss) * 12;
     double v[24];
@@ -434,7 +424,7 @@ __global__ void __launch_bounds__(BT) k_export(double* __restrict__ dst, VecRef 
     if (t >= n5) return;
     const long xcb = t / g.Ls;
     const int s = (int)(t - xcb * g.Ls);
-    const long lex = lex_of(g, xcb, par);
+    const long lex = lex_site(g, xcb, par);
     double v[24];
     load_sp<double, double>(src.d, nullptr, xcb, s, g.Ls, v);
     const int ss = g5r5 ? g.Ls - 1 - s : s;
@@ -444,6 +434,49 @@ __global__ void __launch_bounds__(BT) k_export(double* __restrict__ dst, VecRef 
         const double f = (g5r5 && c >= 6) ? -1.0 : 1.0;
         p[c] = make_double2(f * v[2 * c], f * v[2 * c + 1]);
     }
+}
+
+// both parities of a canonical field -> FP64 hop inputs (k_hop_input), one
+// thread per 5D site in canonical order
+template <bool CHI>
+__global__ void __launch_bounds__(BT) k_import_hop(VecRef o0, VecRef o1, const double* __restrict__ src, Geom g,
+                                                   double z, double mz) {
+    const long t = (long)blockIdx.x * BT + threadIdx.x;
+    if (t >= 2L * g.Vh * g.Ls) return;
+    const long lex = t / g.Ls;
+    const int s = (int)(t - lex * g.Ls);
+    int rem = (int)lex;
+    const int x = rem % g.X; rem /= g.X;
+    const int y = rem % g.Y; rem /= g.Y;
+    const int zz = rem % g.Z;
+    const bool odd = (x + y + zz + rem / g.Z) & 1;
+    double v[24];
+    auto half = [&](int sl, int hi, double f, bool add) {
+        const double2* p = reinterpret_cast<const double2*>(src) + (lex * g.Ls + sl) * 12 + 6 * hi;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const double2 q = p[c];
+            double* d = v + 12 * hi + 2 * c;
+            d[0] = add ? d[0] + f * q.x : q.x;
+            d[1] = add ? d[1] + f * q.y : q.y;
+        }
+    };
+    half(s, 0, 1.0, false);
+    half(s, 1, 1.0, false);
+    if constexpr (CHI) {
+        half(s == 0 ? g.Ls - 1 : s - 1, 0, s == 0 ? -mz : z, true);
+        half(s == g.Ls - 1 ? 0 : s + 1, 1, s == g.Ls - 1 ? -mz : z, true);
+    }
+    const VecRef o = odd ? o1 : o0;
+    fx_store(o.d, o.n, lex >> 1, s, g.Ls, v);
+}
+
+cudaError_t import_hop(VecRef o0, VecRef o1, const double* src, const Geom& g, bool chi, double z, double mz,
+                       cudaStream_t st) {
+    const int grid = grid_for(2L * g.Vh * g.Ls);
+    if (chi) k_import_hop<true><<<grid, BT, 0, st>>>(o0, o1, src, g, z, mz);
+    else k_import_hop<false><<<grid, BT, 0, st>>>(o0, o1, src, g, z, mz);
+    return cudaGetLastError();
 }
 
 // gauge: canonical U[lex][mu][3][3] complex128 -> two-row links per parity in
@@ -659,7 +692,7 @@ __global__ void __launch_bounds__(BT) k_extract_odd(const float* __restrict__ ou
     if (t >= n5) return;
     const long xcb = t / g.Ls;
     const int s = (int)(t - xcb * g.Ls);
-    const long lex = lex_of(g, xcb, 1);
+    const long lex = lex_site(g, xcb, 1);
     const float* src = out32 + ((long)s * 2 * g.Vh + lex) * kCP;
     float v[24];
 #pragma unroll

@@ -50,6 +50,9 @@ cudaError_t blas_sub(VecRef r, VecRef b, VecRef q, long n5, int Ls, Reduce rd, c
 // the kinds with the D~ pre-op
 cudaError_t blas_hop_input(VecRef out, VecRef psi, long n5, int Ls, bool chi, double z, double mz, cudaStream_t st,
                            const int* skip = nullptr);
+// both parities' hop inputs straight from a canonical field
+cudaError_t import_hop(VecRef o0, VecRef o1, const double* src, const Geom& g, bool chi, double z, double mz,
+                       cudaStream_t st);
 cudaError_t blas_zero(int prec, VecRef v, long n5, int Ls, cudaStream_t st, const int* skip = nullptr);
 cudaError_t layout_import(VecRef dst, const double* src, const Geom& g, int par, int g5r5, cudaStream_t st);
 cudaError_t layout_export(double* dst, VecRef src, const Geom& g, int par, int g5r5, cudaStream_t st);

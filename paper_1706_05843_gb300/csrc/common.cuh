@@ -64,6 +64,7 @@ struct SCoef {
     R g1;             // c5/b5 - gamma/alpha
     R fR;             // -kT^2 / 4
     R kTb;            // kT / b5
+    R kTi;            // 1 / kT
     R wu[LSMAX];      // alpha wa
     R wv[LSMAX];      // b5 wb
     R xD[LSMAX];      // D~ x sbk_den / (alpha kT)
@@ -335,6 +336,17 @@ template <typename S, typename R>
 __device__ __forceinline__ void store_sp(void* __restrict__ base, float* __restrict__ nrm, long xcb,
                                          int s, int Ls, const R* v) {
     store_raw<S, R>(base, nrm, xcb, s, Ls, v);
+}
+
+// canonical site index of site xcb of a parity
+__device__ __forceinline__ long lex_site(const Geom& g, long xcb, int par) {
+    int rem = (int)xcb;
+    const int xh = rem % g.Xh; rem /= g.Xh;
+    const int y = rem % g.Y; rem /= g.Y;
+    const int z = rem % g.Z;
+    const int t = rem / g.Z;
+    const int x = 2 * xh + ((par + y + z + t) & 1);
+    return (((long)t * g.Z + z) * g.Y + y) * g.X + x;
 }
 
 // ---------------------------------------------------------------------------

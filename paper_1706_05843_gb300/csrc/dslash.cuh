@@ -59,12 +59,13 @@ enum Kind {
     KIND_R_EO_DAG = 17,    // out = T^T h / kT
     KIND_R_OE_DAG = 18,    // out = kT T^-T y - kT^2 / 4 h
     KIND_R_BACK = 19,      // out = kT D~^-1 y
-    NKIND = 20
+    KIND_H = 20,           // out = T^-1 y - 1/2 D_h y = K D~^-1 y, one parity (in = y; FP64)
+    NKIND = 21
 };
 
 template <int K> struct KindTraits {
     static constexpr bool DENSE = K >= KIND_D_EO && K <= KIND_D_OE_DAG;
-    static constexpr bool HOP = K <= KIND_FULL_DAG || DENSE || (K >= KIND_R_EO && K <= KIND_R_OE_DAG);
+    static constexpr bool HOP = K <= KIND_FULL_DAG || DENSE || (K >= KIND_R_EO && K <= KIND_R_OE_DAG) || K == KIND_H;
     static constexpr bool DAG = K == KIND_EO_MINV_DAG || K == KIND_OE_SCHUR_DAG || K == KIND_FULL_DAG ||
                                 K == KIND_D_EO_DAG || K == KIND_D_OE_DAG || K == KIND_R_EO_DAG || K == KIND_R_OE_DAG;
     static constexpr bool PRE = K == KIND_EO_MINV || K == KIND_RECON || K == KIND_FULL;
@@ -72,7 +73,9 @@ template <int K> struct KindTraits {
                                    K == KIND_R_EO || K == KIND_R_EO_DAG);
     // the column program acts on y alone and runs before the hop, whose
     // result stays in registers: one staged tile instead of two
-    static constexpr bool YCOL = K == KIND_R_OE || K == KIND_R_OE_DAG;
+    static constexpr bool YCOL = K == KIND_R_OE || K == KIND_R_OE_DAG || K == KIND_H;
+    // the operator applications: y and out may be the caller's canonical fields
+    static constexpr bool APPLY = K == KIND_FULL || K == KIND_FULL_DAG || K == KIND_H;
     // FP64: the output is only ever the hop input of the next kernel and is
     // stored in its fixed-point form (fixed64.cuh)
     static constexpr bool FXOUT = K == KIND_EO_MINV || K == KIND_EO_MINV_DAG || K == KIND_D_EO ||
@@ -94,6 +97,8 @@ struct HopArgs {
     const void* lk_in;                       // links of parity 1 - out_par
     Reduce rd;                               // rd.fin == FIN_NONE: no reduction
     const int* done;                         // early exit when *done != 0 (may be NULL)
+    int canon;                               // KT::APPLY kinds, bit 0: y and out are canonical complex128 fields
+                                             // of the whole lattice; bit 1: out takes gamma_5 R_5
     // dense kinds: the Ls x Ls s-space matrix of each chirality in compute
     // precision, [chirality][row][col] in mirrored coordinates
     // (A_ee^-1 for the EO kinds, A_oo for the OE kinds)
@@ -528,7 +533,7 @@ __device__ __forceinline__ void column_program(R* hcol, const R* ycol, const SCo
             const C2<R> d = op_dot<R, LS>(v, cf.um);
             op_axpy<R, LS>(v, cf.yn, {-d.re, -d.im});
         }
-    } else if constexpr (KIND == KIND_R_OE) {
+    } else if constexpr (KIND == KIND_R_OE || KIND == KIND_H) {
         col_load<R, LS, ST>(hcol, v);  // the staged y
         const C2<R> l = op_pade<R, LS>(v, cf.zb, -cf.g1, cf.m, cf.wv);
         if (shv) op_axpy<R, LS>(v, cf.uT, l);
@@ -586,27 +591,27 @@ __device__ __forceinline__ void column_program(R* hcol, const R* ycol, const SCo
 // P+ half takes slice s-1, the P- half slice s+1 (antiperiodic through -m),
 // and the shift chirality the rank-one term sbk u_k y(last) of Eq. (Mooee_shift)
 // with k the mirrored index and "last" slice Ls-1 (P+) or 0 (P-).
-template <typename S, typename R, int LS>
-__device__ __forceinline__ void site_M(const void* __restrict__ y, const float* __restrict__ ynrm, long xcb,
-                                       int s, const SCoef<R>& cf, R* v) {
+// half(s, hi, q): the half hi of slice s of y at this site.
+template <typename R, int LS, typename HALF>
+__device__ __forceinline__ void site_M(HALF&& half, int s, const SCoef<R>& cf, R* v) {
     R q[12];
     {
         const int sm = (s == 0) ? LS - 1 : s - 1;
         const R gu = (s == 0) ? -cf.m * cf.gamma : cf.gamma;
-        load_half<S, R>(y, ynrm, xcb, sm, LS, 0, q);
+        half(sm, 0, q);
 #pragma unroll
         for (int i = 0; i < 12; ++i) v[i] = cf.alpha * v[i] + gu * q[i];
     }
     {
         const int sp = (s == LS - 1) ? 0 : s + 1;
         const R gd = (s == LS - 1) ? -cf.m * cf.gamma : cf.gamma;
-        load_half<S, R>(y, ynrm, xcb, sp, LS, 1, q);
+        half(sp, 1, q);
 #pragma unroll
         for (int i = 0; i < 12; ++i) v[12 + i] = cf.alpha * v[12 + i] + gd * q[i];
     }
     if (cf.has_shift) {
         const int cs = cf.cs;
-        load_half<S, R>(y, ynrm, xcb, cs == 0 ? LS - 1 : 0, LS, cs, q);
+        half(cs == 0 ? LS - 1 : 0, cs, q);
         const R f = cf.sbk * cf.um[cs == 0 ? s : LS - 1 - s];
         if (cs == 0) {
 #pragma unroll
@@ -918,6 +923,7 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
     constexpr int NL = NS * 8;  // staged links (and neighbour indices) per block
     constexpr int RAWB = LinkRaw<S>::PAD;
     constexpr bool FX = sizeof(S) == 8;  // the hop in fixed point (fixed64.cuh)
+    constexpr bool CANON = FX && KT::APPLY;
 
     if (a.done && *a.done) return;
 
@@ -1039,10 +1045,41 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
         const long xcb = blk * NS + il;
         const bool valid = xcb < g.Vh;
 
+        // the site-local input, and the canonical site where the fields are the caller's
+        long lex = 0;
+        if constexpr (CANON) {
+            if (a.canon && valid) lex = lex_site(g, xcb, a.out_par);
+        }
+        auto y_half = [&](int sl, int hi, R* q) {
+            if constexpr (CANON) {
+                if (a.canon) {
+                    const double2* p = reinterpret_cast<const double2*>(a.y) + (lex * LS + sl) * 12 + 6 * hi;
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) {
+                        const double2 t = p[c];
+                        q[2 * c] = t.x;
+                        q[2 * c + 1] = t.y;
+                    }
+                    return;
+                }
+            }
+            load_half<S, R>(a.y, a.y_nrm, xcb, sl, LS, hi, q);
+        };
+        auto y_load = [&](R* v) {
+            if constexpr (CANON) {
+                if (a.canon) {
+                    y_half(s, 0, v);
+                    y_half(s, 1, v + 12);
+                    return;
+                }
+            }
+            load_sp<S, R>(a.y, a.y_nrm, xcb, s, LS, v);
+        };
+
         if constexpr (KT::YCOL) {
             if (valid) {
                 R v[24];
-                load_sp<S, R>(a.y, a.y_nrm, xcb, s, LS, v);
+                y_load(v);
                 st_half(sh + rp, v);
                 st_half(sh + rm, v + 12);
             }
@@ -1107,8 +1144,8 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
                     // out = [M] y + f h, finished in registers
                     const R f = ((KIND == KIND_FULL) ? (R)-0.5 : (R)0.5) * (KT::PRE ? cf.b5 : (R)1);
                     R v[24];
-                    load_sp<S, R>(a.y, a.y_nrm, xcb, s, LS, v);
-                    if constexpr (KIND != KIND_SRC) site_M<S, R, LS>(a.y, a.y_nrm, xcb, s, cf, v);
+                    y_load(v);
+                    if constexpr (KIND != KIND_SRC) site_M<R, LS>(y_half, s, cf, v);
 #pragma unroll
                     for (int i = 0; i < 24; ++i) o[i] = v[i] + f * acc[i];
                 } else if constexpr (COLS && !KT::YCOL) {
@@ -1118,7 +1155,7 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
             }
             if constexpr (KT::HASY && COLS && !KT::YCOL) {
                 R v[24];
-                load_sp<S, R>(a.y, a.y_nrm, xcb, s, LS, v);
+                y_load(v);
                 st_half(sy + rp, v);
                 st_half(sy + rm, v + 12);
             }
@@ -1127,7 +1164,7 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
             // out = M^T y + f D~^T h with the slice neighbours from the site's lanes
             R v[24];
             if (valid) {
-                load_sp<S, R>(a.y, a.y_nrm, xcb, s, LS, v);
+                y_load(v);
             } else {
 #pragma unroll
                 for (int i = 0; i < 24; ++i) v[i] = (R)0;
@@ -1160,10 +1197,22 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
             }
             if constexpr (KT::YCOL) {
 #pragma unroll
-                for (int i = 0; i < 24; ++i) o[i] += cf.fR * acc[i];
+                for (int i = 0; i < 24; ++i)
+                    o[i] = KIND == KIND_H ? cf.kTi * o[i] - (R)0.5 * acc[i] : o[i] + cf.fR * acc[i];
             }
-            if constexpr (FX && KT::FXOUT) fx_store(a.out, a.out_nrm, xcb, s, LS, o);
-            else store_sp<S, R>(a.out, a.out_nrm, xcb, s, LS, o);
+            if constexpr (FX && KT::FXOUT) {
+                fx_store(a.out, a.out_nrm, xcb, s, LS, o);
+            } else if (CANON && a.canon) {
+                const bool g5 = a.canon & 2;
+                double2* p = reinterpret_cast<double2*>(a.out) + (lex * LS + (g5 ? LS - 1 - s : s)) * 12;
+#pragma unroll
+                for (int c = 0; c < 12; ++c) {
+                    const double f = (g5 && c >= 6) ? -1.0 : 1.0;
+                    p[c] = make_double2(f * o[2 * c], f * o[2 * c + 1]);
+                }
+            } else {
+                store_sp<S, R>(a.out, a.out_nrm, xcb, s, LS, o);
+            }
             if (a.rd.fin != FIN_NONE) {
 #pragma unroll
                 for (int i = 0; i < 24; ++i) nn += o[i] * o[i];

@@ -111,6 +111,7 @@ static cudaError_t launch_outer_ls(int kind, const HopArgs& a, const SCoef<typen
             case KIND_SRC: return launch_one<S, LS, KIND_SRC, 0>(a, c, st);
             case KIND_FULL: return launch_one<S, LS, KIND_FULL, 0>(a, c, st);
             case KIND_FULL_DAG: return launch_one<S, LS, KIND_FULL_DAG, 0>(a, c, st);
+            case KIND_H: return launch_one<S, LS, KIND_H, 0>(a, c, st);
             case KIND_LOC_DTMINV: return launch_one<S, LS, KIND_LOC_DTMINV, 0>(a, c, st);
             case KIND_LOC_DT: return launch_one<S, LS, KIND_LOC_DT, 0>(a, c, st);
             default: break;

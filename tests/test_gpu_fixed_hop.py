@@ -99,3 +99,27 @@ def test_non_finite_stays_local(env, bad):
             near |= np.roll(hit, d, ax)
     assert np.array_equal(got[~near], ref[~near])
     assert not np.isfinite(got[near][:, sl]).all(axis=(1, 2)).any()
+
+
+@pytest.mark.parametrize("which", ["k", "kdag", "h"])
+@pytest.mark.parametrize("shift", [0, 24])
+def test_canonical_fields(env, which, shift):
+    """The applications read and write the caller's fields in place: a ragged
+    lattice with Ls = 12 and 16 against the oracle, into a separate field and
+    into one that overlaps the input (shift complex elements further on)."""
+    torch, B, O = env
+    for dims, Ls, pm in (((2, 4, 6, 2), 12, -1), ((6, 2, 2, 4), 16, 1)):
+        act = dict(ACT, pm=pm)
+        U = I.gauge_field(dims, 0.5, 3)
+        x = I.gaussian_fermion(dims, Ls, 1001)
+        o = O.Oracle(O.Action(dims=dims, Ls=Ls, **act), U)
+        ref = {"k": o.k, "kdag": lambda v: o.k(v, dag=True), "h": o.hsys}[which](x)
+        s = B.Solver(U, dims, Ls, **act)
+        buf = torch.zeros(x.size + max(shift, 1) * 12, dtype=torch.complex128, device="cuda")
+        xin = buf[:x.size].view(x.shape)
+        xin.copy_(torch.from_numpy(x))
+        out = buf[shift * 12:shift * 12 + x.size].view(x.shape) if shift else torch.empty_like(xin)
+        {"k": B.eofa_apply, "kdag": B.eofa_apply_dag, "h": B.eofa_apply_h}[which](s.ctx, xin, out)
+        got = out.cpu().numpy()
+        s.close()
+        assert np.linalg.norm(got - ref) <= 1e-14 * np.linalg.norm(ref)
