@@ -28,6 +28,8 @@
 //   K_ee = K_oo = M (site-local), K_eo = K_oe = -1/2 D_h D~.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "fixed64.cuh"
 
@@ -221,130 +223,103 @@ __device__ __forceinline__ void rebuild_row2(R* u) {
 // ---------------------------------------------------------------------------
 // fifth-dimension column operators (mirrored coordinates: always L+ / L-)
 // ---------------------------------------------------------------------------
+// A column holds one value per slice: a complex number for FP32 arithmetic, a
+// real one for FP64 (every coefficient is real), so that the few sites of an
+// FP64 tile still give 24 columns each.
+template <typename R> struct C1 { R re; };
+template <typename R> struct ColVal { typedef C2<R> V; };
+template <> struct ColVal<double> { typedef C1<double> V; };
+
+template <typename R> __device__ __forceinline__ C2<R> vmul(R a, C2<R> x) { return {a * x.re, a * x.im}; }
+template <typename R> __device__ __forceinline__ C1<R> vmul(R a, C1<R> x) { return {a * x.re}; }
+// a x + y
+template <typename R> __device__ __forceinline__ C2<R> vfma(R a, C2<R> x, C2<R> y) {
+    return {fma(a, x.re, y.re), fma(a, x.im, y.im)};
+}
+template <typename R> __device__ __forceinline__ C1<R> vfma(R a, C1<R> x, C1<R> y) { return {fma(a, x.re, y.re)}; }
+
 // (a + g L+) v,  L+: v_s <- v_{s-1}, v_0 <- -m v_{Ls-1}
-template <typename R, int LS>
-__device__ __forceinline__ void op_fwd(C2<R>* v, R a, R g, R mg) {
-    C2<R> last = v[LS - 1];
+template <typename R, int LS, typename V>
+__device__ __forceinline__ void op_fwd(V* v, R a, R g, R mg) {
+    const V last = v[LS - 1];
 #pragma unroll
-    for (int s = LS - 1; s >= 1; --s) {
-        v[s].re = a * v[s].re + g * v[s - 1].re;
-        v[s].im = a * v[s].im + g * v[s - 1].im;
-    }
-    v[0].re = a * v[0].re - mg * last.re;
-    v[0].im = a * v[0].im - mg * last.im;
+    for (int s = LS - 1; s >= 1; --s) v[s] = vfma(a, v[s], vmul(g, v[s - 1]));
+    v[0] = vfma(a, v[0], vmul(-mg, last));
 }
 // (a + g L-) v = (a + g L+^T) v
-template <typename R, int LS>
-__device__ __forceinline__ void op_fwdT(C2<R>* v, R a, R g, R mg) {
-    C2<R> first = v[0];
+template <typename R, int LS, typename V>
+__device__ __forceinline__ void op_fwdT(V* v, R a, R g, R mg) {
+    const V first = v[0];
 #pragma unroll
-    for (int s = 0; s < LS - 1; ++s) {
-        v[s].re = a * v[s].re + g * v[s + 1].re;
-        v[s].im = a * v[s].im + g * v[s + 1].im;
-    }
-    v[LS - 1].re = a * v[LS - 1].re - mg * first.re;
-    v[LS - 1].im = a * v[LS - 1].im - mg * first.im;
+    for (int s = 0; s < LS - 1; ++s) v[s] = vfma(a, v[s], vmul(g, v[s + 1]));
+    v[LS - 1] = vfma(a, v[LS - 1], vmul(-mg, first));
+}
+// v += f a (a a vector in s, f a column value)
+template <typename R, int LS, typename V>
+__device__ __forceinline__ void op_axpy(V* v, const R* a, V f) {
+#pragma unroll
+    for (int s = 0; s < LS; ++s) v[s] = vfma(a[s], f, v[s]);
+}
+template <typename R, int LS, typename V>
+__device__ __forceinline__ V op_dot(const V* v, const R* a) {
+    V d = {};
+#pragma unroll
+    for (int s = 0; s < LS; ++s) d = vfma(a[s], v[s], d);
+    return d;
+}
+// sum_j w_j v_{Ls-1-j}
+template <typename R, int LS, typename V>
+__device__ __forceinline__ V op_rdot(const V* v, const R* w) {
+    V d = {};
+#pragma unroll
+    for (int j = 0; j < LS; ++j) d = vfma(w[j], v[LS - 1 - j], d);
+    return d;
 }
 // solve (a + g L+) t = v in place: t_{Ls-1} = sum_j w_j v_{Ls-1-j},
 // t_0 = v_0/a + m z t_{Ls-1}, t_s = v_s/a - z t_{s-1}.
-template <typename R, int LS>
-__device__ __forceinline__ void op_inv(C2<R>* v, R ia, R z, R mz, const R* w) {
-    C2<R> tl = {0, 0};
+template <typename R, int LS, typename V>
+__device__ __forceinline__ void op_inv(V* v, R ia, R z, R mz, const R* w) {
+    const V tl = op_rdot<R, LS>(v, w);
+    v[0] = vfma(ia, v[0], vmul(mz, tl));
 #pragma unroll
-    for (int j = 0; j < LS; ++j) {
-        tl.re += w[j] * v[LS - 1 - j].re;
-        tl.im += w[j] * v[LS - 1 - j].im;
-    }
-    v[0].re = ia * v[0].re + mz * tl.re;
-    v[0].im = ia * v[0].im + mz * tl.im;
-#pragma unroll
-    for (int s = 1; s < LS - 1; ++s) {
-        v[s].re = ia * v[s].re - z * v[s - 1].re;
-        v[s].im = ia * v[s].im - z * v[s - 1].im;
-    }
+    for (int s = 1; s < LS - 1; ++s) v[s] = vfma(ia, v[s], vmul(-z, v[s - 1]));
     v[LS - 1] = tl;
 }
 // solve (a + g L-) t = v in place (the mirror image of op_inv)
-template <typename R, int LS>
-__device__ __forceinline__ void op_invT(C2<R>* v, R ia, R z, R mz, const R* w) {
-    C2<R> t0 = {0, 0};
+template <typename R, int LS, typename V>
+__device__ __forceinline__ void op_invT(V* v, R ia, R z, R mz, const R* w) {
+    const V t0 = op_dot<R, LS>(v, w);
+    v[LS - 1] = vfma(ia, v[LS - 1], vmul(mz, t0));
 #pragma unroll
-    for (int j = 0; j < LS; ++j) {
-        t0.re += w[j] * v[j].re;
-        t0.im += w[j] * v[j].im;
-    }
-    v[LS - 1].re = ia * v[LS - 1].re + mz * t0.re;
-    v[LS - 1].im = ia * v[LS - 1].im + mz * t0.im;
-#pragma unroll
-    for (int s = LS - 2; s >= 1; --s) {
-        v[s].re = ia * v[s].re - z * v[s + 1].re;
-        v[s].im = ia * v[s].im - z * v[s + 1].im;
-    }
+    for (int s = LS - 2; s >= 1; --s) v[s] = vfma(ia, v[s], vmul(-z, v[s + 1]));
     v[0] = t0;
 }
 
 // M = A + pm beta u (x) v  on the shift chirality
-template <typename R, int LS>
-__device__ __forceinline__ void op_M(C2<R>* v, const SCoef<R>& c, bool sh) {
-    C2<R> vl = v[LS - 1];
+template <typename R, int LS, typename V>
+__device__ __forceinline__ void op_M(V* v, const SCoef<R>& c, bool sh) {
+    const V vl = v[LS - 1];
     op_fwd<R, LS>(v, c.alpha, c.gamma, c.m * c.gamma);
-    if (sh) {
-#pragma unroll
-        for (int s = 0; s < LS; ++s) {
-            R f = c.sbk * c.um[s];
-            v[s].re += f * vl.re;
-            v[s].im += f * vl.im;
-        }
-    }
+    if (sh) op_axpy<R, LS>(v, c.um, vmul(c.sbk, vl));
 }
-template <typename R, int LS>
-__device__ __forceinline__ void op_MT(C2<R>* v, const SCoef<R>& c, bool sh) {
-    C2<R> d = {0, 0};
-    if (sh) {
-#pragma unroll
-        for (int s = 0; s < LS; ++s) {
-            d.re += c.um[s] * v[s].re;
-            d.im += c.um[s] * v[s].im;
-        }
-    }
+template <typename R, int LS, typename V>
+__device__ __forceinline__ void op_MT(V* v, const SCoef<R>& c, bool sh) {
+    V d = {};
+    if (sh) d = op_dot<R, LS>(v, c.um);
     op_fwdT<R, LS>(v, c.alpha, c.gamma, c.m * c.gamma);
-    if (sh) {
-        v[LS - 1].re += c.sbk * d.re;
-        v[LS - 1].im += c.sbk * d.im;
-    }
+    if (sh) v[LS - 1] = vfma(c.sbk, d, v[LS - 1]);
 }
 // Sherman-Morrison: M^-1 v = A^-1 v - (pm beta k (A^-1 v)_{j*} / den) x
-template <typename R, int LS>
-__device__ __forceinline__ void op_Minv(C2<R>* v, const SCoef<R>& c, bool sh) {
+template <typename R, int LS, typename V>
+__device__ __forceinline__ void op_Minv(V* v, const SCoef<R>& c, bool sh) {
     op_inv<R, LS>(v, c.ia, c.za, c.mza, c.wa);
-    if (sh) {
-        C2<R> t = {c.sbk_den * v[LS - 1].re, c.sbk_den * v[LS - 1].im};
-#pragma unroll
-        for (int s = 0; s < LS; ++s) {
-            v[s].re -= c.xm[s] * t.re;
-            v[s].im -= c.xm[s] * t.im;
-        }
-    }
+    if (sh) op_axpy<R, LS>(v, c.xm, vmul(-c.sbk_den, v[LS - 1]));
 }
 // M^-T v = A^-T v - (pm beta (u . A^-T v) / den) y
-template <typename R, int LS>
-__device__ __forceinline__ void op_MinvT(C2<R>* v, const SCoef<R>& c, bool sh) {
+template <typename R, int LS, typename V>
+__device__ __forceinline__ void op_MinvT(V* v, const SCoef<R>& c, bool sh) {
     op_invT<R, LS>(v, c.ia, c.za, c.mza, c.wa);
-    if (sh) {
-        C2<R> d = {0, 0};
-#pragma unroll
-        for (int s = 0; s < LS; ++s) {
-            d.re += c.um[s] * v[s].re;
-            d.im += c.um[s] * v[s].im;
-        }
-        d.re *= c.sb_den;
-        d.im *= c.sb_den;
-#pragma unroll
-        for (int s = 0; s < LS; ++s) {
-            v[s].re -= c.ym[s] * d.re;
-            v[s].im -= c.ym[s] * d.im;
-        }
-    }
+    if (sh) op_axpy<R, LS>(v, c.ym, vmul(-c.sb_den, op_dot<R, LS>(v, c.um)));
 }
 
 // The factors of the right-preconditioned inner operator (3.5 to 4.5
@@ -353,61 +328,29 @@ __device__ __forceinline__ void op_MinvT(C2<R>* v, const SCoef<R>& c, bool sh) {
 // 0.050 -> 0.038 ms for the first half, 0.042 ms for the second).  With a cyclic
 // bidiagonal Z = 1 + z L and v = Z q, one recurrence gives L q beside q:
 // (L q)_0 = -m q_last, q_s = v_s - z (L q)_s, (L q)_{s+1} = q_s.
-// v <- v + g L q;  last: q_last = sum_j w_j v_{Ls-1-j}
-template <typename R, int LS>
-__device__ __forceinline__ C2<R> op_pade(C2<R>* v, R z, R g, R m, const R* w) {
-    C2<R> last = {0, 0};
-#pragma unroll
-    for (int j = 0; j < LS; ++j) {
-        last.re += w[j] * v[LS - 1 - j].re;
-        last.im += w[j] * v[LS - 1 - j].im;
-    }
-    C2<R> l = {-m * last.re, -m * last.im};
+// v <- v + g L q;  returns q_last = sum_j w_j v_{Ls-1-j}
+template <typename R, int LS, typename V>
+__device__ __forceinline__ V op_pade(V* v, R z, R g, R m, const R* w) {
+    const V last = op_rdot<R, LS>(v, w);
+    V l = vmul(-m, last);
 #pragma unroll
     for (int s = 0; s < LS; ++s) {
-        const C2<R> q = {v[s].re - z * l.re, v[s].im - z * l.im};
-        v[s].re += g * l.re;
-        v[s].im += g * l.im;
+        const V q = vfma(-z, l, v[s]);
+        v[s] = vfma(g, l, v[s]);
         l = q;
     }
     return last;
 }
 // the transpose: Z = 1 + z L^T, v <- v + g L^T q
-template <typename R, int LS>
-__device__ __forceinline__ void op_padeT(C2<R>* v, R z, R g, R m, const R* w) {
-    C2<R> first = {0, 0};
-#pragma unroll
-    for (int j = 0; j < LS; ++j) {
-        first.re += w[j] * v[j].re;
-        first.im += w[j] * v[j].im;
-    }
-    C2<R> l = {-m * first.re, -m * first.im};
+template <typename R, int LS, typename V>
+__device__ __forceinline__ void op_padeT(V* v, R z, R g, R m, const R* w) {
+    V l = vmul(-m, op_dot<R, LS>(v, w));
 #pragma unroll
     for (int s = LS - 1; s >= 0; --s) {
-        const C2<R> q = {v[s].re - z * l.re, v[s].im - z * l.im};
-        v[s].re += g * l.re;
-        v[s].im += g * l.im;
+        const V q = vfma(-z, l, v[s]);
+        v[s] = vfma(g, l, v[s]);
         l = q;
     }
-}
-// v += f a (a a vector in s, f a complex number)
-template <typename R, int LS>
-__device__ __forceinline__ void op_axpy(C2<R>* v, const R* a, C2<R> f) {
-#pragma unroll
-    for (int s = 0; s < LS; ++s) {
-        v[s].re += a[s] * f.re;
-        v[s].im += a[s] * f.im;
-    }
-}
-template <typename R, int LS>
-__device__ __forceinline__ C2<R> op_dot(const C2<R>* v, const R* a) {
-    C2<R> d = {0, 0};
-#pragma unroll
-    for (int s = 0; s < LS; ++s) {
-        d.re += a[s] * v[s].re;
-        d.im += a[s] * v[s].im;
-    }
-    return d;
 }
 
 // ---------------------------------------------------------------------------
@@ -447,25 +390,25 @@ __device__ __forceinline__ void st_pair(R* p, const C2<R>& v) {
     q.y = v.im;
     *reinterpret_cast<typename Pair<R>::T*>(p) = q;
 }
-// 12 reals (one chirality half of a row) as 16-byte vectors
-template <typename R>
+// M reals (one chirality half of a row, or a lane's part of it) as 16-byte vectors
+template <int M, typename R>
 __device__ __forceinline__ void st_half(R* p, const R* v) {
     typedef typename Quad<R>::T Q;
     constexpr int N = Quad<R>::N;
 #pragma unroll
-    for (int i = 0; i < 12 / N; ++i) {
+    for (int i = 0; i < M / N; ++i) {
         Q q;
         if constexpr (N == 4) q = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         else q = make_double2(v[2 * i], v[2 * i + 1]);
         reinterpret_cast<Q*>(p)[i] = q;
     }
 }
-template <typename R>
+template <int M, typename R>
 __device__ __forceinline__ void ld_half(const R* p, R* v) {
     typedef typename Quad<R>::T Q;
     constexpr int N = Quad<R>::N;
 #pragma unroll
-    for (int i = 0; i < 12 / N; ++i) {
+    for (int i = 0; i < M / N; ++i) {
         const Q q = reinterpret_cast<const Q*>(p)[i];
         if constexpr (N == 4) {
             v[4 * i] = q.x; v[4 * i + 1] = q.y; v[4 * i + 2] = q.z; v[4 * i + 3] = q.w;
@@ -475,101 +418,102 @@ __device__ __forceinline__ void ld_half(const R* p, R* v) {
     }
 }
 
-// Column access of a shared tile: one complex per row, rows ST reals apart.
+// Column access of a shared tile: one value per row, rows ST reals apart.
 template <typename R, int LS, int ST>
 __device__ __forceinline__ void col_load(const R* p, C2<R>* v) {
 #pragma unroll
     for (int k = 0; k < LS; ++k) v[k] = ld_pair(p + k * ST);
 }
 template <typename R, int LS, int ST>
+__device__ __forceinline__ void col_load(const R* p, C1<R>* v) {
+#pragma unroll
+    for (int k = 0; k < LS; ++k) v[k] = {p[k * ST]};
+}
+template <typename R, int LS, int ST>
 __device__ __forceinline__ void col_store(R* p, const C2<R>* v) {
 #pragma unroll
     for (int k = 0; k < LS; ++k) st_pair(p + k * ST, v[k]);
 }
+template <typename R, int LS, int ST>
+__device__ __forceinline__ void col_store(R* p, const C1<R>* v) {
+#pragma unroll
+    for (int k = 0; k < LS; ++k) p[k * ST] = v[k].re;
+}
 
-// The fifth-dimension program of one (site, spin, colour) column, in the
-// mirrored coordinate.  hcol: the hop result (overwritten with the output),
-// ycol: the local input; consecutive slices are ST reals apart.
+// The fifth-dimension program of one (site, spin, colour) column (of its real
+// or imaginary part for FP64), in the mirrored coordinate.  hcol: the hop
+// result (overwritten with the output), ycol: the local input; consecutive
+// slices are ST reals apart.
 template <typename R, int LS, int KIND, int ST>
 __device__ __forceinline__ void column_program(R* hcol, const R* ycol, const SCoef<R>& cf, bool shv,
                                                R hb, const R* mat) {
     typedef KindTraits<KIND> KT;
-    C2<R> v[LS];
+    typedef typename ColVal<R>::V V;
+    V v[LS];
     if constexpr (KT::DENSE) {
         // dense s-space matrix (row-major in mirrored coordinates) times the
         // column, or its transpose for the adjoint kinds
         constexpr bool TR = KT::DAG;
         constexpr bool EO = (KIND == KIND_D_EO || KIND == KIND_D_EO_DAG);
         col_load<R, LS, ST>(EO ? hcol : ycol, v);
-        C2<R> w[LS];
+        V w[LS];
 #pragma unroll
         for (int k = 0; k < LS; ++k) {
-            R re = (R)0, im = (R)0;
+            w[k] = {};
 #pragma unroll
-            for (int j = 0; j < LS; ++j) {
-                const R a = TR ? mat[j * LS + k] : mat[k * LS + j];
-                re = fma(a, v[j].re, re);
-                im = fma(a, v[j].im, im);
-            }
-            w[k] = {re, im};
+            for (int j = 0; j < LS; ++j) w[k] = vfma(TR ? mat[j * LS + k] : mat[k * LS + j], v[j], w[k]);
         }
         if constexpr (EO) {
 #pragma unroll
-            for (int k = 0; k < LS; ++k) v[k] = {(R)(-0.5) * w[k].re, (R)(-0.5) * w[k].im};
+            for (int k = 0; k < LS; ++k) v[k] = vmul((R)-0.5, w[k]);
         } else {
-            C2<R> h[LS];
+            V h[LS];
             col_load<R, LS, ST>(hcol, h);
 #pragma unroll
-            for (int k = 0; k < LS; ++k) v[k] = {w[k].re + (R)0.5 * h[k].re, w[k].im + (R)0.5 * h[k].im};
+            for (int k = 0; k < LS; ++k) v[k] = vfma((R)0.5, h[k], w[k]);
         }
     } else if constexpr (KIND == KIND_R_EO) {
         col_load<R, LS, ST>(hcol, v);
-        const C2<R> l = op_pade<R, LS>(v, cf.za, cf.g1, cf.m, cf.wu);
-        if (shv) op_axpy<R, LS>(v, cf.xD, {-l.re, -l.im});
+        const V l = op_pade<R, LS>(v, cf.za, cf.g1, cf.m, cf.wu);
+        if (shv) op_axpy<R, LS>(v, cf.xD, vmul((R)-1, l));
     } else if constexpr (KIND == KIND_R_EO_DAG) {
         col_load<R, LS, ST>(hcol, v);
         op_padeT<R, LS>(v, cf.za, cf.g1, cf.m, cf.wu);
-        if (shv) {
-            const C2<R> d = op_dot<R, LS>(v, cf.um);
-            op_axpy<R, LS>(v, cf.yn, {-d.re, -d.im});
-        }
+        if (shv) op_axpy<R, LS>(v, cf.yn, vmul((R)-1, op_dot<R, LS>(v, cf.um)));
     } else if constexpr (KIND == KIND_R_OE || KIND == KIND_H) {
         col_load<R, LS, ST>(hcol, v);  // the staged y
-        const C2<R> l = op_pade<R, LS>(v, cf.zb, -cf.g1, cf.m, cf.wv);
+        const V l = op_pade<R, LS>(v, cf.zb, -cf.g1, cf.m, cf.wv);
         if (shv) op_axpy<R, LS>(v, cf.uT, l);
     } else if constexpr (KIND == KIND_R_OE_DAG) {
         col_load<R, LS, ST>(hcol, v);
-        const C2<R> d = shv ? op_dot<R, LS>(v, cf.um) : C2<R>{0, 0};
+        V d = {};
+        if (shv) d = op_dot<R, LS>(v, cf.um);
         op_padeT<R, LS>(v, cf.zb, -cf.g1, cf.m, cf.wv);
         if (shv) op_axpy<R, LS>(v, cf.eD, d);
     } else if constexpr (KIND == KIND_EO_MINV) {
         col_load<R, LS, ST>(hcol, v);
         op_Minv<R, LS>(v, cf, shv);
         op_fwd<R, LS>(v, cf.b5, cf.c5, cf.m * cf.c5);
-        const R f = (R)(-0.5) * hb;
 #pragma unroll
-        for (int k = 0; k < LS; ++k) { v[k].re *= f; v[k].im *= f; }
+        for (int k = 0; k < LS; ++k) v[k] = vmul((R)(-0.5) * hb, v[k]);
     } else if constexpr (KIND == KIND_EO_MINV_DAG) {
         col_load<R, LS, ST>(hcol, v);
         op_fwdT<R, LS>(v, cf.b5, cf.c5, cf.m * cf.c5);
         op_MinvT<R, LS>(v, cf, shv);
 #pragma unroll
-        for (int k = 0; k < LS; ++k) { v[k].re *= (R)-0.5; v[k].im *= (R)-0.5; }
+        for (int k = 0; k < LS; ++k) v[k] = vmul((R)-0.5, v[k]);
     } else {
         col_load<R, LS, ST>(ycol, v);
         if constexpr (KIND == KIND_OE_SCHUR || KIND == KIND_FULL) op_M<R, LS>(v, cf, shv);
         if constexpr (KIND == KIND_OE_SCHUR_DAG || KIND == KIND_FULL_DAG) op_MT<R, LS>(v, cf, shv);
         if constexpr (KT::HOP) {
-            C2<R> w[LS];
+            V w[LS];
             col_load<R, LS, ST>(hcol, w);
             if constexpr (KIND == KIND_OE_SCHUR_DAG || KIND == KIND_FULL_DAG)
                 op_fwdT<R, LS>(w, cf.b5, cf.c5, cf.m * cf.c5);
             const R f = ((KIND == KIND_FULL || KIND == KIND_FULL_DAG) ? (R)-0.5 : (R)0.5) * hb;
 #pragma unroll
-            for (int k = 0; k < LS; ++k) {
-                v[k].re += f * w[k].re;
-                v[k].im += f * w[k].im;
-            }
+            for (int k = 0; k < LS; ++k) v[k] = vfma(f, w[k], v[k]);
         }
         if constexpr (KIND == KIND_RECON) op_Minv<R, LS>(v, cf, shv);
         if constexpr (KIND == KIND_LOC_DTMINV) {
@@ -581,10 +525,27 @@ __device__ __forceinline__ void column_program(R* hcol, const R* ycol, const SCo
         if constexpr (KIND == KIND_R_BACK) {
             op_inv<R, LS>(v, cf.ib, cf.zb, cf.mzb, cf.wb);
 #pragma unroll
-            for (int k = 0; k < LS; ++k) { v[k].re *= cf.b5 * cf.kTb; v[k].im *= cf.b5 * cf.kTb; }
+            for (int k = 0; k < LS; ++k) v[k] = vmul(cf.b5 * cf.kTb, v[k]);
         }
     }
     col_store<R, LS, ST>(hcol, v);
+}
+
+// lane sp's reals of the half hi of slice s (HV = 2: spin 2 hi + sp; FP64)
+template <typename S, typename R, int HV>
+__device__ __forceinline__ void load_half_part(const void* __restrict__ base, const float* __restrict__ nrm, long xcb,
+                                               int s, int Ls, int hi, int sp, R* v) {
+    if constexpr (HV == 1) {
+        load_half<S, R>(base, nrm, xcb, s, Ls, hi, v);
+    } else {
+        const double2* p = reinterpret_cast<const double2*>(base) + (xcb * 12 + 6 * hi + 3 * sp) * Ls + s;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double2 t = p[c * Ls];
+            v[2 * c] = t.x;
+            v[2 * c + 1] = t.y;
+        }
+    }
 }
 
 // v <- M v for the 5D site (xcb, s) of field y, v = y(xcb, s) on entry: the
@@ -592,22 +553,22 @@ __device__ __forceinline__ void column_program(R* hcol, const R* ycol, const SCo
 // and the shift chirality the rank-one term sbk u_k y(last) of Eq. (Mooee_shift)
 // with k the mirrored index and "last" slice Ls-1 (P+) or 0 (P-).
 // half(s, hi, q): the half hi of slice s of y at this site.
-template <typename R, int LS, typename HALF>
+template <typename R, int LS, int HF, typename HALF>
 __device__ __forceinline__ void site_M(HALF&& half, int s, const SCoef<R>& cf, R* v) {
-    R q[12];
+    R q[HF];
     {
         const int sm = (s == 0) ? LS - 1 : s - 1;
         const R gu = (s == 0) ? -cf.m * cf.gamma : cf.gamma;
         half(sm, 0, q);
 #pragma unroll
-        for (int i = 0; i < 12; ++i) v[i] = cf.alpha * v[i] + gu * q[i];
+        for (int i = 0; i < HF; ++i) v[i] = cf.alpha * v[i] + gu * q[i];
     }
     {
         const int sp = (s == LS - 1) ? 0 : s + 1;
         const R gd = (s == LS - 1) ? -cf.m * cf.gamma : cf.gamma;
         half(sp, 1, q);
 #pragma unroll
-        for (int i = 0; i < 12; ++i) v[12 + i] = cf.alpha * v[12 + i] + gd * q[i];
+        for (int i = 0; i < HF; ++i) v[HF + i] = cf.alpha * v[HF + i] + gd * q[i];
     }
     if (cf.has_shift) {
         const int cs = cf.cs;
@@ -615,10 +576,10 @@ __device__ __forceinline__ void site_M(HALF&& half, int s, const SCoef<R>& cf, R
         const R f = cf.sbk * cf.um[cs == 0 ? s : LS - 1 - s];
         if (cs == 0) {
 #pragma unroll
-            for (int i = 0; i < 12; ++i) v[i] += f * q[i];
+            for (int i = 0; i < HF; ++i) v[i] += f * q[i];
         } else {
 #pragma unroll
-            for (int i = 0; i < 12; ++i) v[12 + i] += f * q[i];
+            for (int i = 0; i < HF; ++i) v[HF + i] += f * q[i];
         }
     }
 }
@@ -633,53 +594,55 @@ template <int K, int LS> struct ShflTail {
     static constexpr bool COLS = !KindTraits<K>::PTW && !ON;
 };
 
-// o = M^T v + f (b5 + c5 L^T) h for lane s of a group of LS lanes: L^T takes
+// o = M^T v + f (b5 + c5 L^T) h for slice s of a group of LS HV lanes (HV lanes
+// a slice, 24 / HV reals each): L^T takes
 // P+ from slice s+1 and P- from slice s-1, each with -m across the wall;
 // the rank-one part of M^T adds sbk (sum_k u_k v_k) to the last mirrored
 // slice of the shift chirality.  Every lane of the warp must call this.
-template <typename R, int LS>
-__device__ __forceinline__ void site_MT_dtT(int s, const SCoef<R>& cf, const R* v, const R* h, R f, R* o) {
+template <typename R, int LS, int HV>
+__device__ __forceinline__ void site_MT_dtT(int s, int sp, const SCoef<R>& cf, const R* v, const R* h, R f, R* o) {
     constexpr unsigned FULL = 0xffffffffu;
-    const int up = (s + 1) & (LS - 1), dn = (s - 1) & (LS - 1);
+    constexpr int HF = 12 / HV, W = LS * HV;
+    const int up = ((s + 1) & (LS - 1)) * HV + sp, dn = ((s - 1) & (LS - 1)) * HV + sp;
     const R wu = (s == LS - 1) ? -cf.m : (R)1;
     const R wd = (s == 0) ? -cf.m : (R)1;
     const R fb = f * cf.b5, fc = f * cf.c5;
 #pragma unroll
-    for (int i = 0; i < 12; ++i) {
-        const R yn = wu * __shfl_sync(FULL, v[i], up, LS);
-        const R hn = wu * __shfl_sync(FULL, h[i], up, LS);
+    for (int i = 0; i < HF; ++i) {
+        const R yn = wu * __shfl_sync(FULL, v[i], up, W);
+        const R hn = wu * __shfl_sync(FULL, h[i], up, W);
         o[i] = cf.alpha * v[i] + cf.gamma * yn + fb * h[i] + fc * hn;
     }
 #pragma unroll
-    for (int i = 12; i < 24; ++i) {
-        const R yn = wd * __shfl_sync(FULL, v[i], dn, LS);
-        const R hn = wd * __shfl_sync(FULL, h[i], dn, LS);
+    for (int i = HF; i < 2 * HF; ++i) {
+        const R yn = wd * __shfl_sync(FULL, v[i], dn, W);
+        const R hn = wd * __shfl_sync(FULL, h[i], dn, W);
         o[i] = cf.alpha * v[i] + cf.gamma * yn + fb * h[i] + fc * hn;
     }
     if (cf.has_shift) {
         const int cs = cf.cs;
         const R u = cf.um[cs == 0 ? s : LS - 1 - s];
         const bool last = s == (cs == 0 ? LS - 1 : 0);
-        R d[12];
+        R d[HF];
         if (cs == 0) {
 #pragma unroll
-            for (int i = 0; i < 12; ++i) d[i] = u * v[i];
+            for (int i = 0; i < HF; ++i) d[i] = u * v[i];
         } else {
 #pragma unroll
-            for (int i = 0; i < 12; ++i) d[i] = u * v[12 + i];
+            for (int i = 0; i < HF; ++i) d[i] = u * v[HF + i];
         }
 #pragma unroll
         for (int off = LS / 2; off > 0; off >>= 1) {
 #pragma unroll
-            for (int i = 0; i < 12; ++i) d[i] += __shfl_xor_sync(FULL, d[i], off, LS);
+            for (int i = 0; i < HF; ++i) d[i] += __shfl_xor_sync(FULL, d[i], off * HV, W);
         }
         if (last) {
             if (cs == 0) {
 #pragma unroll
-                for (int i = 0; i < 12; ++i) o[i] += cf.sbk * d[i];
+                for (int i = 0; i < HF; ++i) o[i] += cf.sbk * d[i];
             } else {
 #pragma unroll
-                for (int i = 0; i < 12; ++i) o[12 + i] += cf.sbk * d[i];
+                for (int i = 0; i < HF; ++i) o[HF + i] += cf.sbk * d[i];
             }
         }
     }
@@ -749,9 +712,21 @@ template <int LS, int VAR> struct MinBlocksCap {
     static constexpr int V = 65536 / (72 * Tile<LS, VAR>::NT);
 };
 
-// sites per CTA of a tile variant (for reports)
-inline int tile_sites(int Ls, int var) {
+// lanes per 5D site of a kernel (the FP64 hop kinds: two, one per upper spin),
+// and its CTA: the FP64 hop kinds take half the sites of the tile.  Against one
+// lane per site on the same half tile: K at 4^4 Ls = 8 53 -> 37 us, FP64 CG
+// iteration at 8^3x16 Ls = 8 157 -> 133 us, K^dag at 24^3x64 Ls = 12 8.85 ->
+// 6.94 ms; K at 16^3x32 Ls = 16 1.15 -> 1.20 ms is the only size that lost.
+template <typename S, int LS, int K, int VAR> struct HopTile {
+    static constexpr int HV = sizeof(S) == 8 && KindTraits<K>::HOP ? 2 : 1;
+    static constexpr int NS = Tile<LS, VAR>::NS / HV;
+    static constexpr int NT = NS * LS * HV;
+};
+
+// sites per CTA of a tile variant of the inner kinds (for reports)
+inline int tile_sites(int prec, int Ls, int var) {
     const bool alt = var & 1;
+    if (prec == 0) return tile_sites(1, Ls, var) / 2;
     switch (Ls) {
         case 4: return alt ? Tile<4, 1>::NS : Tile<4, 0>::NS;
         case 8: return alt ? Tile<8, 1>::NS : Tile<8, 0>::NS;
@@ -848,61 +823,114 @@ static __device__ __noinline__ void hop_fp64_slow(const longlong2* in, const int
     for (int i = 0; i < 24; ++i) out[i] = acc[i];
 }
 
-// The hop sum of one 5D site in fixed point (fixed64.cuh): lk the site's 8
-// staged links (backward ones daggered), nb its neighbour indices.  The
-// direction loop stays rolled: one copy of the products fits the
-// instruction cache (unrolled eight times it is about 100 KB).
+// The hop sum of one 5D site in fixed point (fixed64.cuh) by two lanes: lane
+// sp forms the projected colour vector h = psi_sp + sigma B psi_low, its
+// product w, and adds w to spin sp and sigma B^dag w to a lower spin, 3 - sp
+// for mu = 0, 1 and 2 + sp for mu = 2, 3.  After mu = 1 the lanes swap their
+// lower sums, so each ends with spins sp and 2 + sp.  sigma is the projector's
+// sign times the lane's sign in B (mu = 1: -, +; mu = 2: +, -); a lane takes
+// the direction with sigma = +1 first, so that the sign is the same for all.
+// Per lane: half the loads, products and sums and 96 registers instead of
+// 128 with spills (or 168).  lk: the site's 8 staged links (backward ones
+// daggered), nb its neighbour indices, mask: the lanes that call.  Two mu at
+// a time: four copies of the products fit the instruction cache, eight do not.
 template <int LS, bool DAG>
 __device__ __forceinline__ void hop_fixed(const void* __restrict__ in, const float* __restrict__ nrm,
-                                          const int4* __restrict__ lk, const unsigned* __restrict__ nb, int s,
-                                          double* out) {
+                                          const int4* __restrict__ lk, const unsigned* __restrict__ nb, int s, int sp,
+                                          unsigned mask, double* out) {
     const longlong2* base = reinterpret_cast<const longlong2*>(in) + s;
     const int* ex = reinterpret_cast<const int*>(nrm) + s;
-    i64 acc[24];
+    i64 up[6], lo[6];
 #pragma unroll
-    for (int i = 0; i < 24; ++i) acc[i] = 0;
-    int E = 64;         // exponent field of the units of acc
+    for (int i = 0; i < 6; ++i) up[i] = lo[i] = 0;
+    int E = 64;         // exponent field of the units of the sums
     bool raw = false;   // a neighbour is kept as doubles
-#pragma unroll 1
-    for (int k = 0; k < 8; ++k) {  // k = 2 mu + dir (dir 0 forward, 1 backward)
-        const int l = (k & 1) * 4 + (k >> 1);
-        const long n = (long)(nb[l] & 0x7fffffffu);
-        const longlong2* q = base + n * (12 * LS);
-        const int e = ex[n * LS];
-        i64 p[24], h[12], w[12];
-#pragma unroll
-        for (int c = 0; c < 12; ++c) {
-            const longlong2 t = q[c * LS];
-            p[2 * c] = t.x;
-            p[2 * c + 1] = t.y;
-        }
-        raw = raw || e == kFxRaw;
+    auto raise = [&](int e) {
         if (e > E) {
             const int sh = min(e - E, 63);
 #pragma unroll
-            for (int i = 0; i < 24; ++i) acc[i] >>= sh;
+            for (int i = 0; i < 6; ++i) {
+                up[i] >>= sh;
+                lo[i] >>= sh;
+            }
             E = e;
         }
-        const int kp = DAG ? k : k ^ 1;  // forward projector 1 + gamma for D^dag, 1 - gamma for D
-        fx_project(kp, p, h);
+    };
+    // B is -i times real for mu = 0, 2 and real for mu = 1, 3
+    auto step = [&](auto real_c, auto plus_c, int l, int low) {
+        constexpr bool REAL = decltype(real_c)::value, PLUS = decltype(plus_c)::value;
+        const long n = (long)(nb[l] & 0x7fffffffu);
+        const longlong2* q = base + n * (12 * LS);
+        const int e = ex[n * LS];
+        const longlong2* qu = q + 3 * sp * LS;
+        const longlong2* ql = q + low * LS;
+        i64 h[6], w[6];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const longlong2 t = qu[c * LS], b = ql[c * LS];
+            if constexpr (REAL) {
+                h[2 * c] = PLUS ? t.x + b.x : t.x - b.x;
+                h[2 * c + 1] = PLUS ? t.y + b.y : t.y - b.y;
+            } else {
+                h[2 * c] = PLUS ? t.x + b.y : t.x - b.y;
+                h[2 * c + 1] = PLUS ? t.y - b.x : t.y + b.x;
+            }
+        }
+        raw = raw || e == kFxRaw;
+        raise(e);
         if (e < E) {
             const int sh = min(E - e, 63);
             const i64 half = 1ll << (sh - 1);
 #pragma unroll
-            for (int i = 0; i < 12; ++i) h[i] = (h[i] + half) >> sh;
+            for (int i = 0; i < 6; ++i) h[i] = (h[i] + half) >> sh;
         }
         fx_mul(lk + l * 9, h, w);
-        fx_reconstruct(kp, w, acc);
+#pragma unroll
+        for (int i = 0; i < 6; i += 2) {
+            up[i] += w[i];
+            up[i + 1] += w[i + 1];
+            if constexpr (REAL) {
+                lo[i] = PLUS ? lo[i] + w[i] : lo[i] - w[i];
+                lo[i + 1] = PLUS ? lo[i + 1] + w[i + 1] : lo[i + 1] - w[i + 1];
+            } else {
+                lo[i] = PLUS ? lo[i] - w[i + 1] : lo[i] + w[i + 1];
+                lo[i + 1] = PLUS ? lo[i + 1] + w[i] : lo[i + 1] - w[i];
+            }
+        }
+    };
+    // the projector is 1 + gamma forward for D^dag and backward for D
+    constexpr int BACK = DAG ? 0 : 4;
+    typedef std::integral_constant<bool, true> T;
+    typedef std::integral_constant<bool, false> F;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {  // mu = 0, 1, then 2, 3
+        const int fi = half ? 4 * sp : 0, fr = half ? 0 : 4 * (1 - sp);
+        const int low = 6 + 3 * (half ? sp : 1 - sp), l = 2 * half;
+        step(F{}, T{}, l + (fi ^ BACK), low);
+        step(F{}, F{}, l + (fi ^ BACK ^ 4), low);
+        step(T{}, T{}, l + 1 + (fr ^ BACK), low);
+        step(T{}, F{}, l + 1 + (fr ^ BACK ^ 4), low);
+        if (half == 0) {
+            raise(__shfl_xor_sync(mask, E, 1));  // one unit for both lanes
+#pragma unroll
+            for (int i = 0; i < 6; ++i) lo[i] = __shfl_xor_sync(mask, lo[i], 1);
+        }
     }
     if (!raw) {
 #pragma unroll
-        for (int i = 0; i < 24; ++i) out[i] = fx_to(acc[i], E);
+        for (int i = 0; i < 6; ++i) {
+            out[i] = fx_to(up[i], E);
+            out[6 + i] = fx_to(lo[i], E);
+        }
     } else {
         double r[24];
         hop_fp64_slow(reinterpret_cast<const longlong2*>(in), reinterpret_cast<const int*>(nrm), lk, nb, s, LS,
                       DAG ? 1 : -1, r);
 #pragma unroll
-        for (int i = 0; i < 24; ++i) out[i] = r[i];
+        for (int i = 0; i < 6; ++i) {
+            out[i] = sp ? r[6 + i] : r[i];
+            out[6 + i] = sp ? r[18 + i] : r[12 + i];
+        }
     }
 }
 
@@ -915,8 +943,11 @@ template <typename S, int LS, int KIND, int VAR>
 __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename Traits<S>::R>& cf) {
     typedef typename Traits<S>::R R;
     typedef KindTraits<KIND> KT;
-    constexpr int NS = Tile<LS, VAR>::NS;
-    constexpr int NT = Tile<LS, VAR>::NT;
+    constexpr int HV = HopTile<S, LS, KIND, VAR>::HV;
+    constexpr int NS = HopTile<S, LS, KIND, VAR>::NS;
+    constexpr int NT = HopTile<S, LS, KIND, VAR>::NT;
+    constexpr int NR = 24 / HV, HF = 12 / HV;  // reals of a lane: HF of each chirality
+    constexpr int NCOL = sizeof(R) == 8 ? 24 : 12;  // columns of a site (ColVal)
     constexpr int ST = ShStride<R>::V;
     constexpr int SS = SiteStride<R, LS>::V;
     constexpr int LK = LinkStride<R>::V;
@@ -939,10 +970,11 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
 
     const Geom& g = a.g;
     const int tid = threadIdx.x;
-    const int il = tid / LS;
-    const int s = tid - il * LS;
-    const int rp = il * SS + s * ST;                  // row of the P+ half
-    const int rm = il * SS + (LS - 1 - s) * ST + 12;  // row of the P- half
+    const int il = tid / (LS * HV);
+    const int s = (tid - il * LS * HV) / HV;
+    const int sp = tid % HV;                                    // the lane's upper spin (HV = 2)
+    const int rp = il * SS + s * ST + sp * HF;                  // row of the P+ half
+    const int rm = il * SS + (LS - 1 - s) * ST + 12 + sp * HF;  // row of the P- half
     const long nblk = ((long)g.Vh + NS - 1) / NS;
 
     // ---------------- phase 0: links and neighbours, once per 4D site ---
@@ -1044,6 +1076,7 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
         const unsigned* snc = snb + cur * NL;
         const long xcb = blk * NS + il;
         const bool valid = xcb < g.Vh;
+        const unsigned mask = HV == 2 ? __ballot_sync(0xffffffffu, valid) : 0u;
 
         // the site-local input, and the canonical site where the fields are the caller's
         long lex = 0;
@@ -1053,9 +1086,9 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
         auto y_half = [&](int sl, int hi, R* q) {
             if constexpr (CANON) {
                 if (a.canon) {
-                    const double2* p = reinterpret_cast<const double2*>(a.y) + (lex * LS + sl) * 12 + 6 * hi;
+                    const double2* p = reinterpret_cast<const double2*>(a.y) + (lex * LS + sl) * 12 + 6 * hi + 3 * sp;
 #pragma unroll
-                    for (int c = 0; c < 6; ++c) {
+                    for (int c = 0; c < HF / 2; ++c) {
                         const double2 t = p[c];
                         q[2 * c] = t.x;
                         q[2 * c + 1] = t.y;
@@ -1063,46 +1096,51 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
                     return;
                 }
             }
-            load_half<S, R>(a.y, a.y_nrm, xcb, sl, LS, hi, q);
+            load_half_part<S, R, HV>(a.y, a.y_nrm, xcb, sl, LS, hi, sp, q);
         };
         auto y_load = [&](R* v) {
             if constexpr (CANON) {
                 if (a.canon) {
                     y_half(s, 0, v);
-                    y_half(s, 1, v + 12);
+                    y_half(s, 1, v + HF);
                     return;
                 }
             }
-            load_sp<S, R>(a.y, a.y_nrm, xcb, s, LS, v);
+            if constexpr (HV == 2) {
+                load_half_part<S, R, HV>(a.y, a.y_nrm, xcb, s, LS, 0, sp, v);
+                load_half_part<S, R, HV>(a.y, a.y_nrm, xcb, s, LS, 1, sp, v + HF);
+            } else {
+                load_sp<S, R>(a.y, a.y_nrm, xcb, s, LS, v);
+            }
         };
 
         if constexpr (KT::YCOL) {
             if (valid) {
-                R v[24];
+                R v[NR];
                 y_load(v);
-                st_half(sh + rp, v);
-                st_half(sh + rm, v + 12);
+                st_half<HF>(sh + rp, v);
+                st_half<HF>(sh + rm, v + HF);
             }
             __syncthreads();
-            for (int col = tid; col < NS * 12; col += NT) {
-                const int ci = col / 12;
-                const int cc = col - ci * 12;     // spin * 3 + colour
-                const bool shv = cf.has_shift && ((cc >= 6 ? 1 : 0) == cf.cs);
-                column_program<R, LS, KIND, ST>(sh + ci * SS + 2 * cc, (const R*)nullptr, cf, shv, (R)1, (const R*)nullptr);
+            for (int col = tid; col < NS * NCOL; col += NT) {
+                const int ci = col / NCOL;
+                const int cc = (col - ci * NCOL) * (24 / NCOL);  // place among the 24 reals of a row
+                const bool shv = cf.has_shift && ((cc >= 12 ? 1 : 0) == cf.cs);
+                column_program<R, LS, KIND, ST>(sh + ci * SS + cc, (const R*)nullptr, cf, shv, (R)1, (const R*)nullptr);
             }
         }
 
         // ---------------- phase 1: hop and staging ----------------------
-        R o[24];    // the output spinor of this thread's 5D site
-        R acc[24];  // its hop result (zero for padding sites)
+        R o[NR];    // the output spinor of this thread's 5D site
+        R acc[NR];  // its hop result (zero for padding sites)
 #pragma unroll
-        for (int i = 0; i < 24; ++i) acc[i] = (R)0;
+        for (int i = 0; i < NR; ++i) acc[i] = (R)0;
         if (valid) {
             if constexpr (KT::HOP) {
                 constexpr int FS = KT::DAG ? +1 : -1;  // forward projector 1 + FS gamma
                 if constexpr (FX) {
                     hop_fixed<LS, KT::DAG>(a.in, a.in_nrm, reinterpret_cast<const int4*>(slc + il * 8 * LK),
-                                           snc + il * 8, s, acc);
+                                           snc + il * 8, s, sp, mask, acc);
                 } else
                 // hop k = 2 mu + dir (dir 0 forward, 1 backward)
 #pragma unroll
@@ -1143,34 +1181,34 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
                 if constexpr (KT::PTW) {
                     // out = [M] y + f h, finished in registers
                     const R f = ((KIND == KIND_FULL) ? (R)-0.5 : (R)0.5) * (KT::PRE ? cf.b5 : (R)1);
-                    R v[24];
+                    R v[NR];
                     y_load(v);
-                    if constexpr (KIND != KIND_SRC) site_M<R, LS>(y_half, s, cf, v);
+                    if constexpr (KIND != KIND_SRC) site_M<R, LS, HF>(y_half, s, cf, v);
 #pragma unroll
-                    for (int i = 0; i < 24; ++i) o[i] = v[i] + f * acc[i];
+                    for (int i = 0; i < NR; ++i) o[i] = v[i] + f * acc[i];
                 } else if constexpr (COLS && !KT::YCOL) {
-                    st_half(sh + rp, acc);
-                    st_half(sh + rm, acc + 12);
+                    st_half<HF>(sh + rp, acc);
+                    st_half<HF>(sh + rm, acc + HF);
                 }
             }
             if constexpr (KT::HASY && COLS && !KT::YCOL) {
-                R v[24];
+                R v[NR];
                 y_load(v);
-                st_half(sy + rp, v);
-                st_half(sy + rm, v + 12);
+                st_half<HF>(sy + rp, v);
+                st_half<HF>(sy + rm, v + HF);
             }
         }
         if constexpr (SHF) {
             // out = M^T y + f D~^T h with the slice neighbours from the site's lanes
-            R v[24];
+            R v[NR];
             if (valid) {
                 y_load(v);
             } else {
 #pragma unroll
-                for (int i = 0; i < 24; ++i) v[i] = (R)0;
+                for (int i = 0; i < NR; ++i) v[i] = (R)0;
             }
             const R f = (KIND == KIND_FULL_DAG) ? (R)-0.5 : (R)0.5;
-            site_MT_dtT<R, LS>(s, cf, v, acc, f, o);
+            site_MT_dtT<R, LS, HV>(s, sp, cf, v, acc, f, o);
         }
 
         // ---------------- phase 2: fifth-dimension program --------------
@@ -1179,12 +1217,12 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
         } else if constexpr (COLS) {
             __syncthreads();
             const R hb = KT::PRE ? cf.b5 : (R)1;  // the b5 of the on-the-fly D~
-            for (int col = tid; col < NS * 12; col += NT) {
-                const int ci = col / 12;
-                const int cc = col - ci * 12;     // spin * 3 + colour
-                const bool shv = cf.has_shift && ((cc >= 6 ? 1 : 0) == cf.cs);
-                column_program<R, LS, KIND, ST>(sh + ci * SS + 2 * cc, sy + ci * SS + 2 * cc, cf, shv, hb,
-                                                smat + (cc >= 6 ? LS * LS : 0));
+            for (int col = tid; col < NS * NCOL; col += NT) {
+                const int ci = col / NCOL;
+                const int cc = (col - ci * NCOL) * (24 / NCOL);  // place among the 24 reals of a row
+                const bool shv = cf.has_shift && ((cc >= 12 ? 1 : 0) == cf.cs);
+                column_program<R, LS, KIND, ST>(sh + ci * SS + cc, sy + ci * SS + cc, cf, shv, hb,
+                                                smat + (cc >= 12 ? LS * LS : 0));
             }
             __syncthreads();
         }
@@ -1192,30 +1230,39 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
         // ---------------- phase 3: store ----------------------------------
         if (valid) {
             if constexpr (COLS) {
-                ld_half(sh + rp, o);
-                ld_half(sh + rm, o + 12);
+                ld_half<HF>(sh + rp, o);
+                ld_half<HF>(sh + rm, o + HF);
             }
             if constexpr (KT::YCOL) {
 #pragma unroll
-                for (int i = 0; i < 24; ++i)
+                for (int i = 0; i < NR; ++i)
                     o[i] = KIND == KIND_H ? cf.kTi * o[i] - (R)0.5 * acc[i] : o[i] + cf.fR * acc[i];
             }
             if constexpr (FX && KT::FXOUT) {
-                fx_store(a.out, a.out_nrm, xcb, s, LS, o);
+                if constexpr (HV == 2) fx_store_part(a.out, a.out_nrm, xcb, s, LS, sp, o, mask);
+                else fx_store(a.out, a.out_nrm, xcb, s, LS, o);
             } else if (CANON && a.canon) {
                 const bool g5 = a.canon & 2;
-                double2* p = reinterpret_cast<double2*>(a.out) + (lex * LS + (g5 ? LS - 1 - s : s)) * 12;
+                double2* p = reinterpret_cast<double2*>(a.out) + (lex * LS + (g5 ? LS - 1 - s : s)) * 12 + 3 * sp;
+                const double f = g5 ? -1.0 : 1.0;
 #pragma unroll
-                for (int c = 0; c < 12; ++c) {
-                    const double f = (g5 && c >= 6) ? -1.0 : 1.0;
-                    p[c] = make_double2(f * o[2 * c], f * o[2 * c + 1]);
+                for (int c = 0; c < HF / 2; ++c) {
+                    p[c] = make_double2(o[2 * c], o[2 * c + 1]);
+                    p[6 + c] = make_double2(f * o[HF + 2 * c], f * o[HF + 2 * c + 1]);
+                }
+            } else if constexpr (HV == 2) {
+                double2* p = reinterpret_cast<double2*>(a.out) + (xcb * 12 + 3 * sp) * LS + s;
+#pragma unroll
+                for (int c = 0; c < HF / 2; ++c) {
+                    p[c * LS] = make_double2(o[2 * c], o[2 * c + 1]);
+                    p[(6 + c) * LS] = make_double2(o[HF + 2 * c], o[HF + 2 * c + 1]);
                 }
             } else {
                 store_sp<S, R>(a.out, a.out_nrm, xcb, s, LS, o);
             }
             if (a.rd.fin != FIN_NONE) {
 #pragma unroll
-                for (int i = 0; i < 24; ++i) nn += o[i] * o[i];
+                for (int i = 0; i < NR; ++i) nn += o[i] * o[i];
             }
         }
 
@@ -1227,11 +1274,13 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
     if (a.rd.fin != FIN_NONE) block_reduce_finalize<NT>(nn, a.rd);
 }
 
-// the kernel with the compiler's own register choice (variants 0, 1; FP64:
-// 16 warps per SM, 128 registers and 76 bytes of spills, 228 us against 297 us
-// for the compiler's 168 registers at 16^4, Ls = 16) ...
+// the kernel with the compiler's own register choice (variants 0, 1; the FP64
+// hop kinds: 20 warps per SM, 96 registers; caps of 16 and 24 warps measured
+// 428 and 408 us against 370 us for K^dag at 12^3x24, Ls = 12, and 7.65 and
+// 6.50 ms against 6.94 ms for H at 24^3x64, Ls = 12) ...
 template <typename S, int LS, int KIND, int VAR = 0>
-__global__ void __launch_bounds__(Tile<LS, VAR>::NT, sizeof(S) == 8 ? 512 / Tile<LS, VAR>::NT : 1)
+__global__ void __launch_bounds__(HopTile<S, LS, KIND, VAR>::NT,
+                                  HopTile<S, LS, KIND, VAR>::HV == 2 ? 640 / HopTile<S, LS, KIND, VAR>::NT : 1)
     hop_kernel(const HopArgs a, const SCoef<typename Traits<S>::R> cf) {
     hop_body<S, LS, KIND, VAR>(a, cf);
 }
@@ -1247,8 +1296,8 @@ template <typename S, int LS, int K, int VAR = 0>
 constexpr size_t hop_smem_bytes() {
     typedef typename Traits<S>::R R;
     constexpr size_t bufs = ShflTail<K, LS>::COLS ? (1 + (KindTraits<K>::HASY && !KindTraits<K>::YCOL ? 1 : 0)) : 0;
-    constexpr size_t NL = (size_t)Tile<LS, VAR>::NS * 8;
-    return bufs * (size_t)Tile<LS, VAR>::NS * SiteStride<R, LS>::V * sizeof(R) +
+    constexpr size_t NS = HopTile<S, LS, K, VAR>::NS, NL = NS * 8;
+    return bufs * NS * SiteStride<R, LS>::V * sizeof(R) +
            (KindTraits<K>::DENSE ? 2 * (size_t)LS * LS * sizeof(R) : 0) +
            (KindTraits<K>::HOP ? 2 * NL * (LinkStride<R>::V * sizeof(R) + LinkRaw<S>::PAD + sizeof(unsigned)) : 0);
 }

@@ -21,8 +21,8 @@ constexpr int kHopMaxDevices = 64;
 template <typename S, int LS, int K, int VAR>
 static cudaError_t launch_one(const HopArgs& a, const SCoef<typename Traits<S>::R>& c,
                               cudaStream_t st) {
-    constexpr int NS = Tile<LS, VAR>::NS;
-    constexpr int NT = Tile<LS, VAR>::NT;
+    constexpr int NS = HopTile<S, LS, K, VAR>::NS;
+    constexpr int NT = HopTile<S, LS, K, VAR>::NT;
     const size_t smem = hop_smem_bytes<S, LS, K, VAR>();
     static_assert(hop_smem_bytes<S, LS, K, VAR>() <= 232448, "tile exceeds the 227 KB of shared memory per CTA");
     constexpr bool RCAP = (VAR & 2) != 0;

@@ -1792,7 +1792,7 @@ static eofa_status create_impl(const eofa_params* p, const void* gauge, int gpma
     }
     if ((s = vec_alloc(c, 0, &c->ro, true)) || (s = vec_alloc(c, 0, &c->bto)) || (s = vec_alloc(c, 0, &c->qo)))
         return bail(s);
-    const int maxgrid = std::max(blas_max_grid(c->n5), g.Vh / 8 + 2);
+    const int maxgrid = std::max(blas_max_grid(c->n5), g.Vh / 4 + 2);
     void* tmp = nullptr;
     if ((s = dalloc(c, &tmp, sizeof(double) * maxgrid))) return bail(s);
     c->partials = (double*)tmp;
@@ -2096,7 +2096,7 @@ const char* eofa_last_error(const eofa_ctx* ctx) { return ctx ? ctx->err.c_str()
 
 int eofa_tile_sites(const eofa_ctx* ctx, int prec, int kind) {
     if (!ctx || prec < 0 || prec > 3 || kind < 0 || kind > 3) return 0;
-    return tile_sites(ctx->g.Ls, ctx->tuned[prec] ? ctx->tile[prec][kind] : 0);
+    return tile_sites(prec, ctx->g.Ls, ctx->tuned[prec] ? ctx->tile[prec][kind] : 0);
 }
 
 int eofa_tile_variant(const eofa_ctx* ctx, int prec, int kind) {
@@ -2405,7 +2405,7 @@ eofa_status ensure_learned(eofa_ctx* c) {
     if ((s = vec_alloc(c, EOFA_F32, &c->gx)) || (s = vec_alloc(c, EOFA_F32, &c->gr))) return s;
     for (int k = 0; k < kGcrM; ++k)
         if ((s = vec_alloc(c, EOFA_F32, &c->gz[k])) || (s = vec_alloc(c, EOFA_F32, &c->gw[k]))) return s;
-    const int maxgrid = std::max(blas_max_grid(c->n5), c->g.Vh / 8 + 2);
+    const int maxgrid = std::max(blas_max_grid(c->n5), c->g.Vh / 4 + 2);
     if ((s = dalloc(c, &p, sizeof(double) * maxgrid))) return s;
     c->partials2 = (double*)p;
     if ((s = dalloc(c, &p, 256))) return s;

@@ -26,9 +26,10 @@
 // arithmetic (hop_fp64_slow).
 //
 // Measured, one launch at 16^4, Ls = 16 (524288 5D sites): FP64 arithmetic
-// 1.04 ms (mean of kinds 0 to 3, FP64 pipe 88-90% busy), this form 0.22 to
-// 0.34 ms (the fifth dimension is FP64 still: 41% of its pipe) plus 0.026 to
-// 0.036 ms for the input pass.  Error of K, K^dag and H against extended
+// 1.04 ms (mean of kinds 0 to 3, FP64 pipe 88-90% busy), this form 0.24 to
+// 0.36 ms (the fifth dimension is FP64 still: 42% of its pipe; the integer
+// pipes 40-52%, 46% of the issue slots: fixed-latency dependencies at 19
+// warps per SM) plus 0.025 to 0.041 ms for the input pass.  Error of K, K^dag and H against extended
 // precision (random SU(3), Ls 4 to 16): 1.61e-16 to 1.69e-16 relative,
 // 1.66e-16 to 1.99e-16 with FP64 arithmetic.
 #pragma once
@@ -65,26 +66,31 @@ __device__ __forceinline__ i64 fx_link(double u) {
 
 constexpr int kFxRaw = 2047;  // exponent mark of a spinor kept as doubles
 
-// 24 doubles -> their fixed-point form; returns E (0 for a zero spinor)
-__device__ __forceinline__ int fx_pack(const double* v, i64* m) {
+// N reals of a spinor -> their fixed-point form; returns E (0 for a zero
+// spinor).  N = 12: the two lanes (sp = 0, 1) of a spinor share its exponent;
+// mask: the lanes that call.
+template <int N>
+__device__ __forceinline__ int fx_pack(const double* v, i64* m, unsigned mask = 0) {
     int top = 0;
+    unsigned low = 0;
 #pragma unroll
-    for (int i = 0; i < 24; ++i) top = max(top, __double2hiint(v[i]) & 0x7fffffff);
+    for (int i = 0; i < N; ++i) {
+        top = max(top, __double2hiint(v[i]) & 0x7fffffff);
+        low |= (unsigned)__double2loint(v[i]);
+    }
+    if constexpr (N == 12) {
+        top = max(top, __shfl_xor_sync(mask, top, 1));
+        low |= __shfl_xor_sync(mask, low, 1);
+    }
     const int E = top >> 20;
     if (E < 64 || E > 2030) {
-        bool zero = true;
+        const bool zero = top == 0 && low == 0;
 #pragma unroll
-        for (int i = 0; i < 24; ++i) {
-            zero = zero && v[i] == 0.0;
-            m[i] = __double_as_longlong(v[i]);
-        }
-        if (!zero) return kFxRaw;
-#pragma unroll
-        for (int i = 0; i < 24; ++i) m[i] = 0;
-        return 0;
+        for (int i = 0; i < N; ++i) m[i] = zero ? 0 : __double_as_longlong(v[i]);
+        return zero ? 0 : kFxRaw;
     }
 #pragma unroll
-    for (int i = 0; i < 24; ++i) m[i] = fx_from<kFxFrac>(__double2hiint(v[i]), (unsigned)__double2loint(v[i]), E);
+    for (int i = 0; i < N; ++i) m[i] = fx_from<kFxFrac>(__double2hiint(v[i]), (unsigned)__double2loint(v[i]), E);
     return E;
 }
 
@@ -92,7 +98,7 @@ __device__ __forceinline__ int fx_pack(const double* v, i64* m) {
 // its exponent in the site's scale slot
 __device__ __forceinline__ void fx_store(void* base, float* nrm, long xcb, int s, int Ls, const double* v) {
     i64 m[24];
-    const int E = fx_pack(v, m);
+    const int E = fx_pack<24>(v, m);
     longlong2* p = reinterpret_cast<longlong2*>(base) + xcb * 12 * Ls + s;
 #pragma unroll
     for (int c = 0; c < 12; ++c) p[c * Ls] = make_longlong2(m[2 * c], m[2 * c + 1]);
@@ -153,101 +159,52 @@ __device__ __forceinline__ void fx_stage_link(const double* u, bool neg, bool da
         dst[dag ? (i % 3) * 3 + i / 3 : i] = make_int4(sr * e[i].x, sr * e[i].y, si * e[i].z, si * e[i].w);
 }
 
-// spin projection of a hop (see hop_dir): k = 2 mu + (SG < 0), h = the two
-// colour vectors of (1 + SG gamma_mu) p; exact
-__device__ __forceinline__ void fx_project(int k, const i64* __restrict__ p, i64* __restrict__ h) {
-    const i64 *u0 = p, *u1 = p + 6, *d0 = p + 12, *d1 = p + 18;
-#define FX_PROJ(K, R0, I0, R1, I1)                                  \
-    case K:                                                         \
-        _Pragma("unroll") for (int c = 0; c < 6; c += 2) {          \
-            h[c] = u0[c] R0; h[c + 1] = u0[c + 1] I0;               \
-            h[6 + c] = u1[c] R1; h[7 + c] = u1[c + 1] I1;           \
-        }                                                           \
-        break;
-    switch (k) {
-        FX_PROJ(0, +d1[c + 1], -d1[c], +d0[c + 1], -d0[c])
-        FX_PROJ(1, -d1[c + 1], +d1[c], -d0[c + 1], +d0[c])
-        FX_PROJ(2, -d1[c], -d1[c + 1], +d0[c], +d0[c + 1])
-        FX_PROJ(3, +d1[c], +d1[c + 1], -d0[c], -d0[c + 1])
-        FX_PROJ(4, +d0[c + 1], -d0[c], -d1[c + 1], +d1[c])
-        FX_PROJ(5, -d0[c + 1], +d0[c], +d1[c + 1], -d1[c])
-        FX_PROJ(6, +d0[c], +d0[c + 1], +d1[c], +d1[c + 1])
-        default:
-        FX_PROJ(7, -d0[c], -d0[c + 1], -d1[c], -d1[c + 1])
-    }
-#undef FX_PROJ
-}
-
-// reconstruction (see hop_dir): acc += the four spins of the projected w
-__device__ __forceinline__ void fx_reconstruct(int k, const i64* __restrict__ w, i64* __restrict__ acc) {
+// lane sp's share of a packed spinor: spins sp and 2 + sp (N = 12 reals)
+__device__ __forceinline__ void fx_store_part(void* base, float* nrm, long xcb, int s, int Ls, int sp, const double* v,
+                                              unsigned mask) {
+    i64 m[12];
+    const int E = fx_pack<12>(v, m, mask);
+    longlong2* p = reinterpret_cast<longlong2*>(base) + (xcb * 12 + 3 * sp) * Ls + s;
 #pragma unroll
-    for (int i = 0; i < 12; ++i) acc[i] += w[i];
-    i64 *d0 = acc + 12, *d1 = acc + 18;
-    const i64 *w0 = w, *w1 = w + 6;
-#define FX_REC(K, R0, I0, R1, I1)                                   \
-    case K:                                                         \
-        _Pragma("unroll") for (int c = 0; c < 6; c += 2) {          \
-            d0[c] R0; d0[c + 1] I0; d1[c] R1; d1[c + 1] I1;         \
-        }                                                           \
-        break;
-    switch (k) {
-        FX_REC(0, -= w1[c + 1], += w1[c], -= w0[c + 1], += w0[c])
-        FX_REC(1, += w1[c + 1], -= w1[c], += w0[c + 1], -= w0[c])
-        FX_REC(2, += w1[c], += w1[c + 1], -= w0[c], -= w0[c + 1])
-        FX_REC(3, -= w1[c], -= w1[c + 1], += w0[c], += w0[c + 1])
-        FX_REC(4, -= w0[c + 1], += w0[c], += w1[c + 1], -= w1[c])
-        FX_REC(5, += w0[c + 1], -= w0[c], -= w1[c + 1], += w1[c])
-        FX_REC(6, += w0[c], += w0[c + 1], += w1[c], += w1[c + 1])
-        default:
-        FX_REC(7, -= w0[c], -= w0[c + 1], -= w1[c], -= w1[c + 1])
+    for (int c = 0; c < 3; ++c) {
+        p[c * Ls] = make_longlong2(m[2 * c], m[2 * c + 1]);
+        p[(6 + c) * Ls] = make_longlong2(m[6 + 2 * c], m[6 + 2 * c + 1]);
     }
-#undef FX_REC
+    if (sp == 0) reinterpret_cast<int*>(nrm)[xcb * Ls + s] = E;
 }
 
-// w = W h for both colour vectors of a projected spinor, W the staged link
-// (already daggered for a backward hop)
+// w = W h for one colour vector, W the staged link (already daggered for a
+// backward hop)
 __device__ __forceinline__ void fx_mul(const int4* __restrict__ W, const i64* __restrict__ h, i64* __restrict__ w) {
-    int2 hr[2][3], hi[2][3], hn[2][3];  // limbs of re, im and -im
+    int2 hr[3], hi[3], hn[3];  // limbs of re, im and -im
 #pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            hr[s][c] = fx_split(h[6 * s + 2 * c]);
-            hi[s][c] = fx_split(h[6 * s + 2 * c + 1]);
-            hn[s][c] = make_int2(-hi[s][c].x, -hi[s][c].y);
-        }
+    for (int c = 0; c < 3; ++c) {
+        hr[c] = fx_split(h[2 * c]);
+        hi[c] = fx_split(h[2 * c + 1]);
+        hn[c] = make_int2(-hi[c].x, -hi[c].y);
+    }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        i64 H[2][2], M[2][2];  // [spin][re, im]: high products; middle products, from 1/2
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            H[s][0] = H[s][1] = 0;
-            M[s][0] = M[s][1] = 1 << (kFxLimb - 1);
-        }
+        // high products, and the two kinds of middle products (the first from 1/2)
+        i64 Hr = 0, Hi = 0, Mr = 1 << (kFxLimb - 1), Mi = 1 << (kFxLimb - 1), Nr = 0, Ni = 0;
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
             const int4 e = W[a * 3 + b];
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                H[s][0] = fx_mad(e.x, hr[s][b].x, H[s][0]);
-                M[s][0] = fx_mad(e.x, hr[s][b].y, M[s][0]);
-                M[s][0] = fx_mad(e.y, hr[s][b].x, M[s][0]);
-                H[s][0] = fx_mad(e.z, hn[s][b].x, H[s][0]);
-                M[s][0] = fx_mad(e.z, hn[s][b].y, M[s][0]);
-                M[s][0] = fx_mad(e.w, hn[s][b].x, M[s][0]);
-                H[s][1] = fx_mad(e.x, hi[s][b].x, H[s][1]);
-                M[s][1] = fx_mad(e.x, hi[s][b].y, M[s][1]);
-                M[s][1] = fx_mad(e.y, hi[s][b].x, M[s][1]);
-                H[s][1] = fx_mad(e.z, hr[s][b].x, H[s][1]);
-                M[s][1] = fx_mad(e.z, hr[s][b].y, M[s][1]);
-                M[s][1] = fx_mad(e.w, hr[s][b].x, M[s][1]);
-            }
+            Hr = fx_mad(e.x, hr[b].x, Hr);
+            Hi = fx_mad(e.x, hi[b].x, Hi);
+            Mr = fx_mad(e.x, hr[b].y, Mr);
+            Mi = fx_mad(e.x, hi[b].y, Mi);
+            Nr = fx_mad(e.y, hr[b].x, Nr);
+            Ni = fx_mad(e.y, hi[b].x, Ni);
+            Hr = fx_mad(e.z, hn[b].x, Hr);
+            Hi = fx_mad(e.z, hr[b].x, Hi);
+            Mr = fx_mad(e.z, hn[b].y, Mr);
+            Mi = fx_mad(e.z, hr[b].y, Mi);
+            Nr = fx_mad(e.w, hn[b].x, Nr);
+            Ni = fx_mad(e.w, hr[b].x, Ni);
         }
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            w[6 * s + 2 * a] = H[s][0] + (M[s][0] >> kFxLimb);
-            w[6 * s + 2 * a + 1] = H[s][1] + (M[s][1] >> kFxLimb);
-        }
+        w[2 * a] = Hr + ((Mr + Nr) >> kFxLimb);
+        w[2 * a + 1] = Hi + ((Mi + Ni) >> kFxLimb);
     }
 }
 
