@@ -419,15 +419,15 @@ __global__ void __launch_bounds__(kCvThreads, 1)
 // the same haloed numbering and segments as the convolution.  A CTA belongs to
 // one dt and takes an equal share of the (column, t) steps; a step holds the
 // 128 rows of dy (zero in the halo) and the three dz segments of in at t + dt
-// in shared memory, and its nine warps, one per (dz, dy), form the three dx
-// taps with mma.sync, rows along K.  Every element loaded serves nine taps
+// in shared memory, and its 18 warps, two per (dz, dy) with 16 input channels
+// each, form the three dx taps with mma.sync, rows along K.  Every element loaded serves nine taps
 // (before: one, each tap re-reading both fields through L1; 16^3 x 32, 8
 // slices: 1.6 -> 0.93 ms a layer).  Sums: 64
 // k16 products in the tensor cores, then FP32 registers over the CTA's share,
 // one atomic per element and CTA.  Bound by the ldmatrix reads of shared
 // memory (36 KB per 16 rows, 288 clocks).
 // ---------------------------------------------------------------------------
-constexpr int kWgThreads = 288;
+constexpr int kWgThreads = 576;
 constexpr int kWgStages = 3;
 constexpr int kWgFlush = 8;  // steps (of 8 k16 products) between sums into the FP32 registers
 
@@ -485,12 +485,12 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         }
     };
 
-    float acc[3][2][4][4], sum[3][2][4][4];
+    float acc[3][2][2][4], sum[3][2][2][4];
 #pragma unroll
-    for (int i = 0; i < 96; ++i) (&acc[0][0][0][0])[i] = (&sum[0][0][0][0])[i] = 0.f;
+    for (int i = 0; i < 48; ++i) (&acc[0][0][0][0])[i] = (&sum[0][0][0][0])[i] = 0.f;
     auto flush = [&]() {
 #pragma unroll
-        for (int i = 0; i < 96; ++i) {
+        for (int i = 0; i < 48; ++i) {
             (&sum[0][0][0][0])[i] += (&acc[0][0][0][0])[i];
             (&acc[0][0][0][0])[i] = 0.f;
         }
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         cp_commit();
         __syncthreads();  // the table may be rewritten by the next issue
     }
-    const int dz = warp / 3, dyy = warp % 3;
+    const int dz = warp % 9 / 3, dyy = warp % 3, nh = warp / 9;
     const int i8 = lane >> 3;
     int buf = 0;
     for (long s = s0; s < s1; ++s) {
@@ -515,22 +515,20 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         const int off = dyy * pl.line;
 #pragma unroll 2
         for (int kb = 0; kb < kCvRows / 16; ++kb) {
-            unsigned af[2][4];
+            unsigned af[2][4], bfr[3][4];
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt)   // A = dy^T: (co, k) from rows k, columns co
                 ldsm_x4_t(af[mt], D + swz(kb * 16 + (lane & 7) + (i8 >> 1) * 8, mt * 2 + (i8 & 1)));
 #pragma unroll
-            for (int dx = 0; dx < 3; ++dx) {
-                unsigned bfr[2][4];
+            for (int dx = 0; dx < 3; ++dx)   // B = in_shift: (k, ci) rows k
+                ldsm_x4_t(bfr[dx], In + swz(off + dx + kb * 16 + (lane & 7) + (i8 & 1) * 8, nh * 2 + (i8 >> 1)));
 #pragma unroll
-                for (int n2 = 0; n2 < 2; ++n2)  // B = in_shift: (k, ci) rows k
-                    ldsm_x4_t(bfr[n2], In + swz(off + dx + kb * 16 + (lane & 7) + (i8 & 1) * 8, n2 * 2 + (i8 >> 1)));
+            for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
                 for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-                    for (int nt = 0; nt < 4; ++nt)
-                        mma16816(acc[dx][mt][nt], af[mt], bfr[nt >> 1][(nt & 1) * 2], bfr[nt >> 1][(nt & 1) * 2 + 1]);
-            }
+                    for (int nt = 0; nt < 2; ++nt)
+                        mma16816(acc[dx][mt][nt], af[mt], bfr[dx][nt * 2], bfr[dx][nt * 2 + 1]);
         }
         if ((s - s0) % kWgFlush == kWgFlush - 1) flush();
         buf = buf + 1 == kWgStages ? 0 : buf + 1;
@@ -544,11 +542,11 @@ __global__ void __launch_bounds__(kWgThreads, 1)
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt)
+            for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int co = mt * 16 + (lane >> 2) + (e >> 1) * 8;
-                    const int ci = nt * 8 + (lane & 3) * 2 + (e & 1);
+                    const int ci = (nh * 2 + nt) * 8 + (lane & 3) * 2 + (e & 1);
                     if (co < cout && ci < cin) atomicAdd(dst + (long)co * cin + ci, sum[dx][mt][nt][e]);
                 }
     }
