@@ -220,8 +220,9 @@ cudaError_t outer_cond(cudaGraphConditionalHandle h, const ScalList& L, cudaStre
 template <typename S>
 __global__ void __launch_bounds__(BT) k_cg_r(VecRef q, VecRef r, long n5, int Ls, Reduce rd, const int* done) {
     typedef typename Traits<S>::R R;
-    if (*done) return;
+    const int dn = *done;
     const R al = (R)rd.scal->alpha;
+    if (dn) return;
     R nn = (R)0;
     for (long t = (long)blockIdx.x * BT + threadIdx.x; t < n5; t += (long)gridDim.x * BT) {
         const long xcb = t / Ls;
@@ -241,27 +242,31 @@ __global__ void __launch_bounds__(BT) k_cg_r(VecRef q, VecRef r, long n5, int Ls
 
 // x += alpha p, then p = z + beta p, sharing the read of p.  The update of
 // x belongs to the iteration whose residual update ran, so it still runs in
-// the iteration that set the done flag; the last block then sets stop
-// (FIN_STOP), which ends this kernel in the iterations that follow.
+// the iteration that set the done flag; the next iteration's first kernel
+// finds the flag and sets stop, which ends this kernel from then on: no
+// grid-wide reduction here for that alone (with the scalars read at once and
+// the hops' done flag read beside their link staging, an FP32 CG iteration
+// takes 37.9 -> 35.0 us at 4^4 Ls = 8, 76.6 -> 72.1 us with G-parity at
+// 12x10x8x14 Ls = 8, 243.9 -> 238.6 us at 16^4 Ls = 16).
 template <typename S, typename SX>
-__global__ void __launch_bounds__(BT) k_cg_px(VecRef x, VecRef p, VecRef z, long n5, int Ls, Reduce rd) {
+__global__ void __launch_bounds__(BT) k_cg_px(VecRef x, VecRef p, VecRef z, long n5, int Ls, const DevScal* sc) {
     typedef typename Traits<S>::R R;
     typedef typename Traits<SX>::R RX;
-    const DevScal* sc = rd.scal;
-    if (sc->stop) return;
+    const int stop = sc->stop, done = sc->done;
+    const RX al = (RX)sc->alpha;
+    const R be = (R)sc->beta;
+    if (stop) return;
     for (long t = (long)blockIdx.x * BT + threadIdx.x; t < n5; t += (long)gridDim.x * BT) {
         const long xcb = t / Ls;
         const int s = (int)(t - xcb * Ls);
-        const double al = sc->alpha;
         R pv[24];
         RX xv[24];
         load_sp<S, R>(p.d, p.n, xcb, s, Ls, pv);
         load_sp<SX, RX>(x.d, x.n, xcb, s, Ls, xv);
 #pragma unroll
-        for (int i = 0; i < 24; ++i) xv[i] += (RX)al * (RX)pv[i];
+        for (int i = 0; i < 24; ++i) xv[i] += al * (RX)pv[i];
         store_sp<SX, RX>(x.d, x.n, xcb, s, Ls, xv);
-        if (!sc->done) {
-            const R be = (R)sc->beta;
+        if (!done) {
             R zv[24];
             load_sp<S, R>(z.d, z.n, xcb, s, Ls, zv);
 #pragma unroll
@@ -269,7 +274,6 @@ __global__ void __launch_bounds__(BT) k_cg_px(VecRef x, VecRef p, VecRef z, long
             store_sp<S, R>(p.d, p.n, xcb, s, Ls, pv);
         }
     }
-    block_reduce_finalize<BT>((R)0, rd);
 }
 
 // dst = a * src (types may differ); optional |dst|^2 reduction.
@@ -562,12 +566,12 @@ cudaError_t blas_cg_r(int prec, VecRef q, VecRef r, long n5, int Ls, Reduce rd, 
     });
 }
 
-cudaError_t blas_cg_px(int prec, int xprec, VecRef x, VecRef p, VecRef z, long n5, int Ls, Reduce rd,
+cudaError_t blas_cg_px(int prec, int xprec, VecRef x, VecRef p, VecRef z, long n5, int Ls, const DevScal* sc,
                        cudaStream_t st) {
     return dispatch_prec(prec, [&](auto* tag) -> cudaError_t {
         typedef std::remove_pointer_t<decltype(tag)> S;
-        if (xprec == 0) k_cg_px<S, double><<<grid_capped(n5), BT, 0, st>>>(x, p, z, n5, Ls, rd);
-        else k_cg_px<S, float><<<grid_capped(n5), BT, 0, st>>>(x, p, z, n5, Ls, rd);
+        if (xprec == 0) k_cg_px<S, double><<<grid_capped(n5), BT, 0, st>>>(x, p, z, n5, Ls, sc);
+        else k_cg_px<S, float><<<grid_capped(n5), BT, 0, st>>>(x, p, z, n5, Ls, sc);
         return cudaGetLastError();
     });
 }

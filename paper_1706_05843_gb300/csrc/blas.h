@@ -36,8 +36,8 @@ cudaError_t outer_cond(cudaGraphConditionalHandle h, const ScalList& L, cudaStre
 // r -= alpha q with |r|^2 (rd: FIN_RR); returns at once when *done
 cudaError_t blas_cg_r(int prec, VecRef q, VecRef r, long n5, int Ls, Reduce rd, const int* done,
                       cudaStream_t st);
-// x += alpha p; p = z + beta p unless done (rd: FIN_STOP on the same scalars)
-cudaError_t blas_cg_px(int prec, int xprec, VecRef x, VecRef p, VecRef z, long n5, int Ls, Reduce rd,
+// x += alpha p; p = z + beta p unless done; returns at once when stop is set
+cudaError_t blas_cg_px(int prec, int xprec, VecRef x, VecRef p, VecRef z, long n5, int Ls, const DevScal* sc,
                        cudaStream_t st);
 // skip (may be NULL): the kernel returns at once while *skip is nonzero
 cudaError_t blas_copy(int dprec, VecRef dst, int sprec, VecRef src, long n5, int Ls, double scale,

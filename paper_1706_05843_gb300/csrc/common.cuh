@@ -87,7 +87,7 @@ struct DevScal {
     unsigned long long t0_ns;      // %globaltimer at the start of the solve
     unsigned long long timeout_ns; // 0: none
     int timed_out;
-    int stop;                      // the CG update of x and p has run after done was set
+    int stop;                      // set by the first iteration after done: the last CG update of x has run
     // device-driven defect correction of a batched solve (one graph launch):
     // every flag below is read by the kernels of one phase, which return at
     // once while it is nonzero
@@ -111,7 +111,7 @@ struct ScalList {
     int n;
 };
 
-enum Fin { FIN_NONE = 0, FIN_STORE = 1, FIN_ALPHA = 2, FIN_BETA = 3, FIN_RR = 4, FIN_ZZ = 5, FIN_STOP = 6 };
+enum Fin { FIN_NONE = 0, FIN_STORE = 1, FIN_ALPHA = 2, FIN_BETA = 3, FIN_RR = 4, FIN_ZZ = 5 };
 
 struct Reduce {
     double* partials;   // one per block
@@ -398,7 +398,6 @@ __device__ __forceinline__ void finalize(const Reduce& rd, double total) {
             sc->zz = total;
             break;
         case FIN_ZZ: sc->zz = total; break;
-        case FIN_STOP: sc->stop = sc->done; break;
         case FIN_RR:
             sc->rr = total;
             sc->iters += 1;

@@ -99,6 +99,7 @@ struct HopArgs {
     const void* lk_in;                       // links of parity 1 - out_par
     Reduce rd;                               // rd.fin == FIN_NONE: no reduction
     const int* done;                         // early exit when *done != 0 (may be NULL)
+    int* stop;                               // set by a launch that finds *done set (may be NULL)
     int canon;                               // KT::APPLY kinds, bit 0: y and out are canonical complex128 fields
                                              // of the whole lattice; bit 1: out takes gamma_5 R_5
     // dense kinds: the Ls x Ls s-space matrix of each chirality in compute
@@ -956,7 +957,13 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
     constexpr bool FX = sizeof(S) == 8;  // the hop in fixed point (fixed64.cuh)
     constexpr bool CANON = FX && KT::APPLY;
 
-    if (a.done && *a.done) return;
+    // issued now, used after the first links are staged; a launch of several
+    // blocks per CTA, whose first stage is a small part, leaves at once
+    const int dn = a.done ? *reinterpret_cast<const volatile int*>(a.done) : 0;
+    auto leave = [&]() {
+        if (a.stop && blockIdx.x == 0 && threadIdx.x == 0) *a.stop = 1;
+    };
+    if ((long)gridDim.x * NS < a.g.Vh && dn) return leave();
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr bool SHF = ShflTail<KIND, LS>::ON;
@@ -1064,6 +1071,7 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
         }
         __syncthreads();
     }
+    if (dn) return leave();
 
     R nn = (R)0;
     for (int it = 0; blk < nblk; ++it, blk += gridDim.x) {

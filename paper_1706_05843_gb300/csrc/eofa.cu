@@ -318,7 +318,7 @@ int hop_input_pass(int kind) {
 }
 
 eofa_status hop(eofa_ctx* c, int prec, int kind, int out_par, VecRef in, VecRef y, VecRef out, Reduce rd,
-                const int* done, cudaStream_t st, bool timed = false) {
+                const int* done, cudaStream_t st, bool timed = false, int* stop = nullptr) {
     if (const int pass = prec == EOFA_F64 ? hop_input_pass(kind) : 0) {
         // into c->ro, which holds nothing live at any of these launches
         // (outer_residual writes it last)
@@ -337,6 +337,7 @@ eofa_status hop(eofa_ctx* c, int prec, int kind, int out_par, VecRef in, VecRef 
     a.rd = rd;
     a.tile_var = (kind >= KIND_R_EO && kind <= KIND_R_OE_DAG && c->tuned[prec]) ? c->tile[prec][kind - KIND_R_EO] : 0;
     a.done = done;
+    a.stop = stop;
     if (kind >= KIND_D_EO && kind <= KIND_D_OE_DAG && prec <= EOFA_F32)
         a.dense = c->dense[prec][(kind == KIND_D_OE || kind == KIND_D_OE_DAG) ? 1 : 0];
     const void* coef = prec == EOFA_F64 ? (const void*)&c->c64 : (const void*)&c->c32;
@@ -567,7 +568,7 @@ eofa_status cg_iteration(eofa_ctx* c, int P, cudaStream_t st, bool timed, cudaEv
         if (ev) CK(cudaEventRecordWithFlags(ev[i], st, cudaEventRecordExternal), "cudaEventRecordWithFlags");
         return EOFA_OK;
     };
-    if ((s = mark(0)) || (s = hop(c, P, k0, 0, in.p, none, in.t, red(c, FIN_NONE), done, st, timed)) ||
+    if ((s = mark(0)) || (s = hop(c, P, k0, 0, in.p, none, in.t, red(c, FIN_NONE), done, st, timed, &c->scal->stop)) ||
         (s = mark(1)))
         return s;
     if ((s = mark(2)) || (s = hop(c, P, k1, 1, in.t, in.p, in.q, red(c, FIN_ALPHA), done, st, timed)) ||
@@ -580,7 +581,7 @@ eofa_status cg_iteration(eofa_ctx* c, int P, cudaStream_t st, bool timed, cudaEv
     if ((s = mark(6)) || (s = hop(c, P, k3, 1, in.t, in.r, in.z, red(c, FIN_BETA), done, st, timed)) ||
         (s = mark(7)))
         return s;
-    CKL(blas_cg_px(P, xp, in.x, in.p, in.z, c->n5, c->g.Ls, red(c, FIN_STOP), st), "cg_px");
+    CKL(blas_cg_px(P, xp, in.x, in.p, in.z, c->n5, c->g.Ls, c->scal, st), "cg_px");
     return EOFA_OK;
 }
 

@@ -422,10 +422,10 @@ __global__ void __launch_bounds__(kCvThreads, 1)
 // in shared memory, and its 18 warps, two per (dz, dy) with 16 input channels
 // each, form the three dx taps with mma.sync, rows along K.  Every element loaded serves nine taps
 // (before: one, each tap re-reading both fields through L1; 16^3 x 32, 8
-// slices: 1.6 -> 0.93 ms a layer).  Sums: 64
+// slices: 1.6 -> 0.82 ms a layer).  Sums: 64
 // k16 products in the tensor cores, then FP32 registers over the CTA's share,
-// one atomic per element and CTA.  Bound by the ldmatrix reads of shared
-// memory (36 KB per 16 rows, 288 clocks).
+// one atomic per element and CTA.  Bound by the mma.sync rate (math pipe
+// throttle leads the stalls; nine warps of 32 channels: 0.93 ms).
 // ---------------------------------------------------------------------------
 constexpr int kWgThreads = 576;
 constexpr int kWgStages = 3;
