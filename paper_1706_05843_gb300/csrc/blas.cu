@@ -176,7 +176,7 @@ __global__ void k_outer_decide(DevScal* sc, int first) {
         outer_end(sc, EOFA_ERR_TIMEOUT);
         return;
     }
-    const double t = fmax(sc->tol / rel, sc->floor_tol);
+    const double t = fmax(kInnerMargin * sc->tol / rel, sc->floor_tol);
     sc->target_rr = t * t;
     sc->qq = sc->zz = sc->rr = sc->alpha = sc->beta = 0.0;
     sc->iters = 0;

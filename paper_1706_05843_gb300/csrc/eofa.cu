@@ -1087,7 +1087,7 @@ eofa_status solve_impl(eofa_ctx* c, const double* rhs, double* sol, const eofa_s
         if ((s = outer_residual(c, ss, st))) return s;
         CK(cudaStreamSynchronize(st), "sync");
         if (!outer_decide(c, o, ss)) break;
-        const double itol = std::max(o.tol / ss.rel, inner_tol_floor(o, ss.P));
+        const double itol = std::max(kInnerMargin * o.tol / ss.rel, inner_tol_floor(o, ss.P));
         // inner source r / |r| in precision P
         CKL(blas_copy(ss.P, c->inner[ss.P].r, 0, c->ro, c->n5, Ls, 1.0, 0, red(c, FIN_NONE), st), "copy");
         int its = 0;
