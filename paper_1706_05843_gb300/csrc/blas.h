@@ -14,12 +14,15 @@ struct VecRef {
 };
 
 struct HopArgs;
+struct HopPair;
 
 // precision codes: 0 F64, 1 F32, 2 F16, 3 BF16 (the eofa_prec values)
 cudaError_t launch_hop_f64(int kind, const HopArgs& a, const void* coef, cudaStream_t st);
 cudaError_t launch_hop_f32(int kind, const HopArgs& a, const void* coef, cudaStream_t st);
 cudaError_t launch_hop_f16(int kind, const HopArgs& a, const void* coef, cudaStream_t st);
 cudaError_t launch_hop_bf16(int kind, const HopArgs& a, const void* coef, cudaStream_t st);
+// KIND_FULL, KIND_FULL_DAG or KIND_H over both parities, on canonical fields
+cudaError_t launch_apply_f64(int kind, const HopPair& p, const SCoef<double>& c, cudaStream_t st);
 // kinds >= 4 (FP64 and FP32 storage only)
 cudaError_t launch_hop_f64_outer(int kind, const HopArgs& a, const void* coef, cudaStream_t st);
 cudaError_t launch_hop_f32_outer(int kind, const HopArgs& a, const void* coef, cudaStream_t st);

@@ -983,7 +983,6 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
     const int rp = il * SS + s * ST + sp * HF;                  // row of the P+ half
     const int rm = il * SS + (LS - 1 - s) * ST + 12 + sp * HF;  // row of the P- half
     const long nblk = ((long)g.Vh + NS - 1) / NS;
-
     // ---------------- phase 0: links and neighbours, once per 4D site ---
     // The 8 links of each site (4 forward from this parity, 4 backward from
     // the neighbours) and the 8 neighbour indices (bit 31: the hop carries a
@@ -1291,6 +1290,16 @@ __global__ void __launch_bounds__(HopTile<S, LS, KIND, VAR>::NT,
                                   HopTile<S, LS, KIND, VAR>::HV == 2 ? 640 / HopTile<S, LS, KIND, VAR>::NT : 1)
     hop_kernel(const HopArgs a, const SCoef<typename Traits<S>::R> cf) {
     hop_body<S, LS, KIND, VAR>(a, cf);
+}
+
+// ... an application's two parities in one grid (blockIdx.y) ...
+struct HopPair {
+    HopArgs a[2];
+};
+template <typename S, int LS, int KIND>
+__global__ void __launch_bounds__(HopTile<S, LS, KIND, 0>::NT, 640 / HopTile<S, LS, KIND, 0>::NT)
+    hop_kernel_pair(const __grid_constant__ HopPair p, const SCoef<typename Traits<S>::R> cf) {
+    hop_body<S, LS, KIND, 0>(p.a[blockIdx.y], cf);
 }
 
 // ... and with capped registers (variants 2, 3; FP32 arithmetic)

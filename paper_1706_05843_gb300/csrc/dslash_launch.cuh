@@ -74,6 +74,55 @@ static cudaError_t launch_one(const HopArgs& a, const SCoef<typename Traits<S>::
     return cudaGetLastError();
 }
 
+// An application's two hops (p.a[0], p.a[1]; FP64).  Up to 8 rounds of
+// resident CTAs they share one grid (K at 4^4, Ls = 8: 26-31 us against 36 us
+// for a grid each; 8^3x16, Ls = 8: 52 against 62.5 us; 12^3x24, Ls = 12, six
+// rounds: 306 against 318 us); larger lattices fill the SMs with a grid each
+// (16^4, Ls = 16, eleven rounds: 609 us in one grid, 599 us in two).
+template <typename S, int LS, int K>
+static cudaError_t launch_pair(const HopPair& p, const SCoef<typename Traits<S>::R>& c, cudaStream_t st) {
+    constexpr int NS = HopTile<S, LS, K, 0>::NS;
+    constexpr int NT = HopTile<S, LS, K, 0>::NT;
+    const size_t smem = hop_smem_bytes<S, LS, K, 0>();
+    static std::atomic<int> resident_of[kHopMaxDevices];
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kHopMaxDevices) return cudaErrorInvalidDevice;
+    int resident = resident_of[dev].load(std::memory_order_acquire);
+    if (resident == 0) {  // several threads may do this at once, with the same result
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
+            return cudaErrorStreamCaptureUnsupported;
+        e = cudaFuncSetAttribute(hop_kernel_pair<S, LS, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, hop_kernel_pair<S, LS, K>, NT, smem);
+        if (e != cudaSuccess) return e;
+        resident = std::max(resident, 1);
+        resident_of[dev].store(resident, std::memory_order_release);
+    }
+    const long nblk = ((long)p.a[0].g.Vh + NS - 1) / NS, full = (long)resident * sms;
+    if (nblk > 8 * full) {
+        e = launch_one<S, LS, K, 0>(p.a[0], c, st);
+        return e != cudaSuccess ? e : launch_one<S, LS, K, 0>(p.a[1], c, st);
+    }
+    const dim3 grid((unsigned)std::min<long>(nblk, std::max<long>(1, full / 2)), 2);
+    hop_kernel_pair<S, LS, K><<<grid, NT, smem, st>>>(p, c);
+    return cudaGetLastError();
+}
+
+// the FP64 applications: kinds KIND_FULL, KIND_FULL_DAG, KIND_H
+template <int LS>
+static cudaError_t launch_pair_ls(int kind, const HopPair& p, const SCoef<double>& c, cudaStream_t st) {
+    switch (kind) {
+        case KIND_FULL: return launch_pair<double, LS, KIND_FULL>(p, c, st);
+        case KIND_FULL_DAG: return launch_pair<double, LS, KIND_FULL_DAG>(p, c, st);
+        case KIND_H: return launch_pair<double, LS, KIND_H>(p, c, st);
+        default: return cudaErrorNotSupported;
+    }
+}
+
 template <typename S, int LS, int K>
 static cudaError_t launch_var(const HopArgs& a, const SCoef<typename Traits<S>::R>& c, cudaStream_t st) {
     if constexpr (kTileVariants<S> == 4) {
@@ -111,7 +160,6 @@ static cudaError_t launch_outer_ls(int kind, const HopArgs& a, const SCoef<typen
             case KIND_SRC: return launch_one<S, LS, KIND_SRC, 0>(a, c, st);
             case KIND_FULL: return launch_one<S, LS, KIND_FULL, 0>(a, c, st);
             case KIND_FULL_DAG: return launch_one<S, LS, KIND_FULL_DAG, 0>(a, c, st);
-            case KIND_H: return launch_one<S, LS, KIND_H, 0>(a, c, st);
             case KIND_LOC_DTMINV: return launch_one<S, LS, KIND_LOC_DTMINV, 0>(a, c, st);
             case KIND_LOC_DT: return launch_one<S, LS, KIND_LOC_DT, 0>(a, c, st);
             default: break;

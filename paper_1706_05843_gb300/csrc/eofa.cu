@@ -1391,15 +1391,16 @@ eofa_status solve_batched_impl(eofa_ctx* const* cs, int n, const void* const* rh
 double* act_buf(eofa_ctx* c, size_t i);
 
 // The operator applications: one pass makes both parities' hop inputs, then
-// one hop kernel per parity reads its site-local part from the caller's field
-// and writes the caller's result: three launches and 970 bytes of traffic per
+// the hops (one launch for both where that fills the SMs better) read their
+// site-local part from the caller's field and write the caller's result: two
+// or three launches and 970 bytes of traffic per
 // 5D site, where import, D~ passes, hops and export took six to eight and up
 // to 1900 (H at 24^3x64, Ls = 12: 8.8 -> 7.0 ms; K at 4^4, Ls = 8: 78 -> 51
-// us).  H = g5 R5 K D~^-1 needs no D~: K D~^-1 = T^-1 - 1/2 D_h.
+// us with a hop launch per parity).  H = g5 R5 K D~^-1 needs no D~: K D~^-1 = T^-1 - 1/2 D_h.
 eofa_status apply_impl(eofa_ctx* c, const void* in, void* out, int which, cudaStream_t st) {
     // which: 0 = K, 1 = K^dag, 2 = H + beta Delta P = g5 R5 K D~^-1
-    // the second hop reads the input after the first has written: fields that
-    // overlap need the input's copy
+    // the hop reads the input while it writes the output: fields that overlap
+    // need the input's copy
     const size_t bytes = (size_t)c->n5 * 2 * 24 * sizeof(double);
     if ((const char*)in < (const char*)out + bytes && (const char*)out < (const char*)in + bytes) {
         double* copy = act_buf(c, 2);
@@ -1408,9 +1409,10 @@ eofa_status apply_impl(eofa_ctx* c, const void* in, void* out, int which, cudaSt
         in = copy;
     }
     CKL(import_hop(c->t[0], c->t[1], (const double*)in, c->g, which == 0, c->c64.zb, c->c64.mzb, st), "import");
+    HopPair p;
+    std::memset(&p, 0, sizeof(p));
     for (int par = 0; par < 2; ++par) {
-        HopArgs a;
-        std::memset(&a, 0, sizeof(a));
+        HopArgs& a = p.a[par];
         a.g = c->g;
         a.out_par = par;
         a.in = c->t[1 - par].d;
@@ -1420,8 +1422,8 @@ eofa_status apply_impl(eofa_ctx* c, const void* in, void* out, int which, cudaSt
         a.lk_out = c->links[EOFA_F64][par];
         a.lk_in = c->links[EOFA_F64][1 - par];
         a.canon = which == 2 ? 3 : 1;
-        CKL(launch_hop_f64(which == 2 ? KIND_H : which == 0 ? KIND_FULL : KIND_FULL_DAG, a, &c->c64, st), "apply");
     }
+    CKL(launch_apply_f64(which == 2 ? KIND_H : which == 0 ? KIND_FULL : KIND_FULL_DAG, p, c->c64, st), "apply");
     return EOFA_OK;
 }
 
