@@ -11,6 +11,9 @@
 //            "L acts first" order of Eq. (Ddwf).  Spin projection to half
 //            spinors, two-row links rebuilt in registers; h goes to shared
 //            memory.  An optional site-local input y is staged beside it.
+//            FP64: the products run in 64-bit fixed point on inputs prepared
+//            for it (fixed64.cuh), two lanes to a 5D site, and a pass over
+//            the input applies D~ where a kind wants it.
 //  2. fifth dimension: each thread takes complex columns (x_i, spin, colour)
 //            and applies an O(Ls) program: the cyclic bidiagonal
 //            A = alpha + gamma L (the site-diagonal block of D_DWF, App. B),
@@ -25,7 +28,8 @@
 //            chunks) and contributes |out|^2 to a deterministic reduction.
 //
 // The kernel kinds below are the even-odd blocks of K (App. B):
-//   K_ee = K_oo = M (site-local), K_eo = K_oe = -1/2 D_h D~.
+//   K_ee = K_oo = M (site-local), K_eo = K_oe = -1/2 D_h D~,
+// and of K D~^-1, which the inner CG inverts.
 #pragma once
 
 #include <type_traits>

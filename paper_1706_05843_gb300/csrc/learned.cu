@@ -69,9 +69,13 @@ enum Epi { EPI_LEAKY_BF16 = 0, EPI_F32 = 1, EPI_DMASK_BF16 = 2 };
 // g_tc_fault, every role leaves its loop, the copies and MMAs in flight are
 // waited for and the tensor memory is freed.
 //
-// What bounds it: shared-memory reads of the operands, 93 clocks an MMA
-// measured (4 KB of A rows that mostly straddle 128-byte lines, 3 KB of B)
-// against 48 clocks of tensor work; tensor pipe 44%.  16^3 x 32, 16 slices:
+// What bounds it: shared-memory reads of the operands (4 KB of A and 3 KB of B
+// an MMA beside the segments' own 10 KB per 18 MMAs): 93 clocks an MMA measured,
+// 19% of them spent waiting for a segment, against 48 clocks of tensor work;
+// tensor pipe 44%.  Lines without a halo and a copy of each segment per dx, so
+// that every A view starts at a 128-byte line, took 1.65 against 1.68 ms for the
+// network at 16^3 x 32 and 0.56 against 0.54 ms at 40 x 8 x 8 x 16: the
+// alignment of the views is not what costs.  16^3 x 32, 16 slices:
 // 0.417 ms a layer, 2.2 ms for the kernel it replaces, which gathered the 128
 // neighbour rows of every tap through L1 (97% of its peak, tensor pipe 7%).
 // ---------------------------------------------------------------------------
