@@ -23,6 +23,7 @@ cudaError_t launch_hop_f16(int kind, const HopArgs& a, const void* coef, cudaStr
 cudaError_t launch_hop_bf16(int kind, const HopArgs& a, const void* coef, cudaStream_t st);
 // KIND_FULL, KIND_FULL_DAG or KIND_H over both parities, on canonical fields
 cudaError_t launch_apply_f64(int kind, const HopPair& p, const SCoef<double>& c, cudaStream_t st);
+cudaError_t setup_apply_f64(int Ls, cudaStream_t st);
 // kinds >= 4 (FP64 and FP32 storage only)
 cudaError_t launch_hop_f64_outer(int kind, const HopArgs& a, const void* coef, cudaStream_t st);
 cudaError_t launch_hop_f32_outer(int kind, const HopArgs& a, const void* coef, cudaStream_t st);

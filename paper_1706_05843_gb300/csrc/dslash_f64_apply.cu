@@ -13,4 +13,14 @@ cudaError_t launch_apply_f64(int kind, const HopPair& p, const SCoef<double>& c,
         default: return cudaErrorNotSupported;
     }
 }
+// once per device, so that an application can be captured whatever ran before
+cudaError_t setup_apply_f64(int Ls, cudaStream_t st) {
+    switch (Ls) {
+        case 4: return setup_apply_ls<4>(st);
+        case 8: return setup_apply_ls<8>(st);
+        case 12: return setup_apply_ls<12>(st);
+        case 16: return setup_apply_ls<16>(st);
+        default: return cudaErrorNotSupported;
+    }
+}
 }  // namespace eofa

@@ -18,51 +18,57 @@ namespace eofa {
 // devices a process may use the hop kernels on
 constexpr int kHopMaxDevices = 64;
 
+// The CTAs of one kernel that one SM holds, on the current device (the
+// persistent grids are that many per SM).  Once per kernel and device, before
+// its first launch there: the shared-memory limit, an attribute of the current
+// device; not inside a stream capture (the drivers launch every kernel once
+// before they capture it, and a context sets up its applications' kernels).
+struct HopResident {
+    std::atomic<int> of[kHopMaxDevices] = {};
+    std::mutex mu;
+};
+template <typename F>
+static cudaError_t hop_resident(HopResident& r, F* kernel, int nt, size_t smem, cudaStream_t st, int* dev,
+                                int* resident) {
+    cudaError_t e = cudaGetDevice(dev);
+    if (e != cudaSuccess) return e;
+    if (*dev < 0 || *dev >= kHopMaxDevices) return cudaErrorInvalidDevice;
+    *resident = r.of[*dev].load(std::memory_order_acquire);
+    if (*resident) return cudaSuccess;
+    std::lock_guard<std::mutex> lock(r.mu);
+    *resident = r.of[*dev].load(std::memory_order_relaxed);
+    if (*resident) return cudaSuccess;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
+        return cudaErrorStreamCaptureUnsupported;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, kernel, nt, smem);
+    if (e != cudaSuccess) return e;
+    *resident = std::max(*resident, 1);
+    r.of[*dev].store(*resident, std::memory_order_release);
+    return cudaSuccess;
+}
+
+template <typename S, int LS, int K, int VAR>
+static cudaError_t resident_one(cudaStream_t st, int* dev, int* resident) {
+    static HopResident r;
+    constexpr int NT = HopTile<S, LS, K, VAR>::NT;
+    const size_t smem = hop_smem_bytes<S, LS, K, VAR>();
+    static_assert(hop_smem_bytes<S, LS, K, VAR>() <= 232448, "tile exceeds the 227 KB of shared memory per CTA");
+    if constexpr ((VAR & 2) != 0) return hop_resident(r, hop_kernel_rc<S, LS, K, VAR>, NT, smem, st, dev, resident);
+    else return hop_resident(r, hop_kernel<S, LS, K, VAR>, NT, smem, st, dev, resident);
+}
+
 template <typename S, int LS, int K, int VAR>
 static cudaError_t launch_one(const HopArgs& a, const SCoef<typename Traits<S>::R>& c,
                               cudaStream_t st) {
     constexpr int NS = HopTile<S, LS, K, VAR>::NS;
     constexpr int NT = HopTile<S, LS, K, VAR>::NT;
     const size_t smem = hop_smem_bytes<S, LS, K, VAR>();
-    static_assert(hop_smem_bytes<S, LS, K, VAR>() <= 232448, "tile exceeds the 227 KB of shared memory per CTA");
     constexpr bool RCAP = (VAR & 2) != 0;
-    // per instantiation and device, before its first launch there: the
-    // shared-memory limit (an attribute of the current device) and the
-    // number of CTAs one SM holds (the persistent grid is that many per SM)
-    static std::atomic<int> resident_of[kHopMaxDevices];
-    static std::mutex setup_mu;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    int dev = 0, resident = 0;
+    cudaError_t e = resident_one<S, LS, K, VAR>(st, &dev, &resident);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kHopMaxDevices) return cudaErrorInvalidDevice;
-    int resident = resident_of[dev].load(std::memory_order_acquire);
-    if (resident == 0) {
-        std::lock_guard<std::mutex> lock(setup_mu);
-        resident = resident_of[dev].load(std::memory_order_relaxed);
-        if (resident == 0) {
-            // the one-time set-up must not run inside a stream capture (the
-            // drivers launch every kernel once before they capture it)
-            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-            if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
-                return cudaErrorStreamCaptureUnsupported;
-            if constexpr (RCAP) {
-                e = cudaFuncSetAttribute(hop_kernel_rc<S, LS, K, VAR>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e == cudaSuccess)
-                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, hop_kernel_rc<S, LS, K, VAR>,
-                                                                      NT, smem);
-            } else {
-                e = cudaFuncSetAttribute(hop_kernel<S, LS, K, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-                if (e == cudaSuccess)
-                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, hop_kernel<S, LS, K, VAR>, NT,
-                                                                      smem);
-            }
-            if (e != cudaSuccess) return e;
-            if (resident < 1) resident = 1;
-            resident_of[dev].store(resident, std::memory_order_release);
-        }
-    }
     const long nblk = ((long)a.g.Vh + NS - 1) / NS;
     if (nblk == 0) return cudaSuccess;
     int sms = 0;
@@ -72,6 +78,13 @@ static cudaError_t launch_one(const HopArgs& a, const SCoef<typename Traits<S>::
     if constexpr (RCAP) hop_kernel_rc<S, LS, K, VAR><<<grid, NT, smem, st>>>(a, c);
     else hop_kernel<S, LS, K, VAR><<<grid, NT, smem, st>>>(a, c);
     return cudaGetLastError();
+}
+
+template <typename S, int LS, int K>
+static cudaError_t resident_pair(cudaStream_t st, int* dev, int* resident) {
+    static HopResident r;
+    return hop_resident(r, hop_kernel_pair<S, LS, K>, HopTile<S, LS, K, 0>::NT, hop_smem_bytes<S, LS, K, 0>(), st, dev,
+                        resident);
 }
 
 // An application's two hops (p.a[0], p.a[1]; FP64).  Up to 8 rounds of
@@ -84,24 +97,10 @@ static cudaError_t launch_pair(const HopPair& p, const SCoef<typename Traits<S>:
     constexpr int NS = HopTile<S, LS, K, 0>::NS;
     constexpr int NT = HopTile<S, LS, K, 0>::NT;
     const size_t smem = hop_smem_bytes<S, LS, K, 0>();
-    static std::atomic<int> resident_of[kHopMaxDevices];
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    int dev = 0, resident = 0, sms = 0;
+    cudaError_t e = resident_pair<S, LS, K>(st, &dev, &resident);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kHopMaxDevices) return cudaErrorInvalidDevice;
-    int resident = resident_of[dev].load(std::memory_order_acquire);
-    if (resident == 0) {  // several threads may do this at once, with the same result
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
-            return cudaErrorStreamCaptureUnsupported;
-        e = cudaFuncSetAttribute(hop_kernel_pair<S, LS, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, hop_kernel_pair<S, LS, K>, NT, smem);
-        if (e != cudaSuccess) return e;
-        resident = std::max(resident, 1);
-        resident_of[dev].store(resident, std::memory_order_release);
-    }
     const long nblk = ((long)p.a[0].g.Vh + NS - 1) / NS, full = (long)resident * sms;
     if (nblk > 8 * full) {
         e = launch_one<S, LS, K, 0>(p.a[0], c, st);
@@ -121,6 +120,21 @@ static cudaError_t launch_pair_ls(int kind, const HopPair& p, const SCoef<double
         case KIND_H: return launch_pair<double, LS, KIND_H>(p, c, st);
         default: return cudaErrorNotSupported;
     }
+}
+
+// both forms of every application's kernel
+template <int LS>
+static cudaError_t setup_apply_ls(cudaStream_t st) {
+    int dev, n;
+    cudaError_t e = cudaSuccess;
+    auto one = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
+    one(resident_pair<double, LS, KIND_FULL>(st, &dev, &n));
+    one(resident_pair<double, LS, KIND_FULL_DAG>(st, &dev, &n));
+    one(resident_pair<double, LS, KIND_H>(st, &dev, &n));
+    one(resident_one<double, LS, KIND_FULL, 0>(st, &dev, &n));
+    one(resident_one<double, LS, KIND_FULL_DAG, 0>(st, &dev, &n));
+    one(resident_one<double, LS, KIND_H, 0>(st, &dev, &n));
+    return e;
 }
 
 template <typename S, int LS, int K>

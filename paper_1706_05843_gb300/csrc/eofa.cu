@@ -3,10 +3,10 @@
 // Solve path (App. B of arXiv:1706.05843):
 //   b   = g5 R5 phi (H form) or b (K form), imported into the even-odd layout
 //   b~o = b_o - K_oe K_ee^-1 b_e                       even-odd source
-//   CGNR on S = K_oo - K_oe K_ee^-1 K_eo:  S^dag S x_o = S^dag b~o
-//     inside a restarted defect-correction loop (Sec. V.A): the FP64 outer
-//     loop forms r = b~o - S x_o, the inner CGNR solves S e = r/|r| in the
-//     requested storage precision, x_o += |r| e
+//   CGNR for S x_o = b~o, S = K_oo - K_oe K_ee^-1 K_eo, inside a restarted
+//     defect-correction loop (Sec. V.A): the FP64 outer loop forms
+//     r = b~o - S x_o, the inner CGNR solves (S D~^-1) f = r/|r| in the
+//     requested storage precision, x_o += |r| D~^-1 f
 //   x_e = K_ee^-1 (b_e - K_eo x_o)                     reconstruction
 //   psi = D~(m1) psi'                                  undo the Cayley form
 //   true residual ||b - K psi'|| / ||b|| in FP64
@@ -1388,8 +1388,6 @@ eofa_status solve_batched_impl(eofa_ctx* const* cs, int n, const void* const* rh
     return first;
 }
 
-double* act_buf(eofa_ctx* c, size_t i);
-
 // The operator applications: one pass makes both parities' hop inputs, then
 // the hops (one launch for both where that fills the SMs better) read their
 // site-local part from the caller's field and write the caller's result: two
@@ -1400,14 +1398,12 @@ double* act_buf(eofa_ctx* c, size_t i);
 eofa_status apply_impl(eofa_ctx* c, const void* in, void* out, int which, cudaStream_t st) {
     // which: 0 = K, 1 = K^dag, 2 = H + beta Delta P = g5 R5 K D~^-1
     // the hop reads the input while it writes the output: fields that overlap
-    // need the input's copy
+    // go through the context's own, y in x and the results in ro and qo
     const size_t bytes = (size_t)c->n5 * 2 * 24 * sizeof(double);
-    if ((const char*)in < (const char*)out + bytes && (const char*)out < (const char*)in + bytes) {
-        double* copy = act_buf(c, 2);
-        if (!copy) return EOFA_ERR_OOM;
-        CK(cudaMemcpyAsync(copy, in, bytes, cudaMemcpyDeviceToDevice, st), "cudaMemcpyAsync");
-        in = copy;
-    }
+    const bool overlap = (const char*)in < (const char*)out + bytes && (const char*)out < (const char*)in + bytes;
+    VecRef res[2] = {c->ro, c->qo};
+    for (int par = 0; par < 2 && overlap; ++par)
+        CKL(layout_import(c->x[par], (const double*)in, c->g, par, 0, st), "import");
     CKL(import_hop(c->t[0], c->t[1], (const double*)in, c->g, which == 0, c->c64.zb, c->c64.mzb, st), "import");
     HopPair p;
     std::memset(&p, 0, sizeof(p));
@@ -1422,8 +1418,17 @@ eofa_status apply_impl(eofa_ctx* c, const void* in, void* out, int which, cudaSt
         a.lk_out = c->links[EOFA_F64][par];
         a.lk_in = c->links[EOFA_F64][1 - par];
         a.canon = which == 2 ? 3 : 1;
+        if (overlap) {
+            a.y = c->x[par].d;
+            a.y_nrm = c->x[par].n;
+            a.out = res[par].d;
+            a.out_nrm = res[par].n;
+            a.canon = 0;
+        }
     }
     CKL(launch_apply_f64(which == 2 ? KIND_H : which == 0 ? KIND_FULL : KIND_FULL_DAG, p, c->c64, st), "apply");
+    for (int par = 0; par < 2 && overlap; ++par)
+        CKL(layout_export((double*)out, res[par], c->g, par, which == 2, st), "export");
     return EOFA_OK;
 }
 
@@ -1833,6 +1838,7 @@ static eofa_status create_impl(const eofa_params* p, const void* gauge, int gpma
         (e = cudaStreamSynchronize(st)) != cudaSuccess)
         return bail(cuda_fail(c, e, "gauge check"));
     if (bad) return bail(EOFA_ERR_ARG);
+    if ((e = setup_apply_f64(g.Ls, st)) != cudaSuccess) return bail(cuda_fail(c, e, "application set-up"));
     *out = c;
     return EOFA_OK;
 }

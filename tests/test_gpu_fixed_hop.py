@@ -123,3 +123,29 @@ def test_canonical_fields(env, which, shift):
         got = out.cpu().numpy()
         s.close()
         assert np.linalg.norm(got - ref) <= 1e-14 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("dims,Ls", [((4, 4, 4, 4), 4), ((16, 16, 16, 16), 16)])
+@pytest.mark.parametrize("shift", [0, 24])
+def test_applications_are_capturable(env, dims, Ls, shift):
+    """A new context's first application may be a captured one, with both
+    parities in one grid and in two, into a separate field and into one that
+    overlaps the input; the replay gives the eager result to the last bit."""
+    torch, B, _ = env
+    s = B.Solver(I.gauge_field(dims, 0.3, 5), dims, Ls, **ACT)
+    x = torch.from_numpy(I.gaussian_fermion(dims, Ls, 6)).cuda()
+    for f in (B.eofa_apply, B.eofa_apply_dag, B.eofa_apply_h):
+        buf = torch.empty(x.numel() + max(shift, 1) * 12, dtype=x.dtype, device="cuda")
+        a = buf[:x.numel()].view(x.shape)
+        a.copy_(x)
+        out = buf[shift * 12:shift * 12 + x.numel()].view(x.shape) if shift else torch.empty_like(a)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            f(s.ctx, a, out)
+        g.replay()
+        torch.cuda.synchronize()
+        ref = torch.empty_like(x)
+        f(s.ctx, x, ref)
+        assert torch.equal(torch.view_as_real(out), torch.view_as_real(ref))
+    s.close()
