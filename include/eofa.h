@@ -70,7 +70,9 @@ typedef enum {
 } eofa_status;
 
 /* Storage precision of the inner Krylov solver (arithmetic is FP64 for
- * EOFA_F64 and FP32 for the others). */
+ * EOFA_F64 and FP32 for the others; the FP64 hop sums its products in 64-bit
+ * fixed point where that loses nothing against FP64, every real relative to
+ * the terms that make it up, and in FP64 elsewhere). */
 typedef enum {
     EOFA_F64 = 0,
     EOFA_F32 = 1,

@@ -10,7 +10,8 @@ namespace eofa {
 
 struct VecRef {
     void* d;    // chunk array of one parity
-    float* n;   // FP16 per-site scales (NULL otherwise)
+    float* n;   // FP16 per-site scales, exponents of an FP64 hop input (NULL otherwise)
+    void* raw = nullptr;  // FP64 hop input that a hop kernel writes: its doubles
 };
 
 struct HopArgs;

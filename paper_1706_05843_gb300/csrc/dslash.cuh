@@ -12,8 +12,9 @@
 //            spinors, two-row links rebuilt in registers; h goes to shared
 //            memory.  An optional site-local input y is staged beside it.
 //            FP64: the products run in 64-bit fixed point on inputs prepared
-//            for it (fixed64.cuh), two lanes to a 5D site, and a pass over
-//            the input applies D~ where a kind wants it.
+//            for it, and in FP64 where a sum needs that (fixed64.cuh), two
+//            lanes to a 5D site; a pass over the input applies D~ where a
+//            kind wants it.
 //  2. fifth dimension: each thread takes complex columns (x_i, spin, colour)
 //            and applies an O(Ls) program: the cyclic bidiagonal
 //            A = alpha + gamma L (the site-diagonal block of D_DWF, App. B),
@@ -83,7 +84,7 @@ template <int K> struct KindTraits {
     // the operator applications: y and out may be the caller's canonical fields
     static constexpr bool APPLY = K == KIND_FULL || K == KIND_FULL_DAG || K == KIND_H;
     // FP64: the output is only ever the hop input of the next kernel and is
-    // stored in its fixed-point form (fixed64.cuh)
+    // stored in its fixed-point form (fixed64.cuh), its doubles beside it
     static constexpr bool FXOUT = K == KIND_EO_MINV || K == KIND_EO_MINV_DAG || K == KIND_D_EO ||
                                   K == KIND_D_EO_DAG || K == KIND_LOC_DTMINV || K == KIND_R_EO || K == KIND_R_EO_DAG;
     // site-local kinds: the fifth-dimension part reaches only slices s-1, s+1
@@ -97,15 +98,17 @@ struct HopArgs {
     int out_par;
     int tile_var;                            // CTA tile variant (autotuner)
     const void* in;  const float* in_nrm;    // hop input, parity 1 - out_par (FP64: fixed point, exponents in in_nrm)
+    const void* in_raw;                      // FP64: the field that the hop input was made from (without D~)
     const void* y;   const float* y_nrm;     // site-local input, parity out_par
     void* out;       float* out_nrm;         // output, parity out_par
+    void* out_raw;                           // KT::FXOUT: the output's doubles beside its fixed-point form
     const void* lk_out;                      // links of parity out_par
     const void* lk_in;                       // links of parity 1 - out_par
     Reduce rd;                               // rd.fin == FIN_NONE: no reduction
     const int* done;                         // early exit when *done != 0 (may be NULL)
     int* stop;                               // set by a launch that finds *done set (may be NULL)
-    int canon;                               // KT::APPLY kinds, bit 0: y and out are canonical complex128 fields
-                                             // of the whole lattice; bit 1: out takes gamma_5 R_5
+    int canon;                               // KT::APPLY kinds, bit 0: y, in_raw and out are canonical complex128
+                                             // fields of the whole lattice; bit 1: out takes gamma_5 R_5
     // dense kinds: the Ls x Ls s-space matrix of each chirality in compute
     // precision, [chirality][row][col] in mirrored coordinates
     // (A_ee^-1 for the EO kinds, A_oo for the OE kinds)
@@ -718,13 +721,20 @@ template <int LS, int VAR> struct MinBlocksCap {
 };
 
 // lanes per 5D site of a kernel (the FP64 hop kinds: two, one per upper spin),
-// and its CTA: the FP64 hop kinds take half the sites of the tile.  Against one
-// lane per site on the same half tile: K at 4^4 Ls = 8 53 -> 37 us, FP64 CG
-// iteration at 8^3x16 Ls = 8 157 -> 133 us, K^dag at 24^3x64 Ls = 12 8.85 ->
-// 6.94 ms; K at 16^3x32 Ls = 16 1.15 -> 1.20 ms is the only size that lost.
+// and its CTA: the FP64 hop kinds take half the sites of the tile (against one
+// lane per site on the same half tile, when both were FP64 hops without the
+// FP64 fallback: K at 4^4 Ls = 8 53 -> 37 us, FP64 CG iteration at 8^3x16
+// Ls = 8 157 -> 133 us, K^dag at 24^3x64 Ls = 12 8.85 -> 6.94 ms; K at
+// 16^3x32 Ls = 16 1.15 -> 1.20 ms lost).  The two applications with a column
+// phase take a quarter at Ls = 12: CTAs of three warps leave room for five,
+// with 128 registers, where those of six leave room for two (168) or three
+// (96).  4 sites, 8 sites in three CTAs: K^dag 354, 363 us and H 342, 359 us at
+// 12^3x24; K^dag 2.79, 2.84 ms at 24^4.  K itself, 4 sites or 8 in two CTAs:
+// 2.61, 2.49 ms at 24^4.
 template <typename S, int LS, int K, int VAR> struct HopTile {
     static constexpr int HV = sizeof(S) == 8 && KindTraits<K>::HOP ? 2 : 1;
-    static constexpr int NS = Tile<LS, VAR>::NS / HV;
+    static constexpr bool QUARTER = HV == 2 && LS == 12 && (K == KIND_FULL_DAG || K == KIND_H);
+    static constexpr int NS = Tile<LS, VAR>::NS / (QUARTER ? 4 : HV);
     static constexpr int NT = NS * LS * HV;
 };
 
@@ -791,41 +801,167 @@ __device__ __forceinline__ void link_from_raw(const unsigned char* raw, R* u) {
     }
 }
 
-// The hop sum of one 5D site in FP64 arithmetic from the fixed-point links:
-// the rare threads of hop_fixed whose neighbours are not finite or of
-// extreme magnitude.  LS is a runtime value here: one copy for all kernels.
-static __device__ __noinline__ void hop_fp64_slow(const longlong2* in, const int* ex, const int4* lk,
-                                                  const unsigned* nb, int s, int Ls, int FS, double* out) {
-    double acc[24];
-    for (int i = 0; i < 24; ++i) acc[i] = 0.0;
+// lanes and the other lanes of their sites
+__device__ __forceinline__ unsigned hop_sites(unsigned lanes) {
+    return lanes | ((lanes & 0x55555555u) << 1) | ((lanes >> 1) & 0x55555555u);
+}
+
+// The reals of hop_fixed's sums that some term is not exactly zero in: bit i
+// for up[i], bit 6 + i for lo[i] (as they are at the end).  A fixed-point real
+// and an element of rows 0 and 1 of a staged link are zero only if the double
+// is (fx_from); row 2 goes by its cofactors.  Sparse fields on links that keep
+// them sparse (a point source in the free field) have many exact zeros.
+static __device__ __forceinline__ unsigned hop_terms(const HopArgs* __restrict__ a, const int4* __restrict__ lk,
+                                                  const unsigned* __restrict__ nb, int s, int sp, int Ls,
+                                                  unsigned mask) {
+    unsigned up = 0, lo = 0;
+    auto swap = [](unsigned m) { return ((m & 0x15u) << 1) | ((m >> 1) & 0x15u); };
 #pragma unroll 1
     for (int k = 0; k < 8; ++k) {
-        const int l = (k & 1) * 4 + (k >> 1);
-        double p[24], W[18];
-        const long n = (long)(nb[l] & 0x7fffffffu);
-        const int e5 = ex[n * Ls + s];
-        for (int c = 0; c < 12; ++c) {
-            const longlong2 q = in[(n * 12 + c) * Ls + s];
-            p[2 * c] = e5 == kFxRaw ? __longlong_as_double(q.x) : fx_to(q.x, e5);
-            p[2 * c + 1] = e5 == kFxRaw ? __longlong_as_double(q.y) : fx_to(q.y, e5);
+        const int mu = k >> 1, low = mu < 2 ? 3 - sp : 2 + sp;
+        const bool back = k & 1, real = mu & 1;
+        if (k == 4) lo = __shfl_xor_sync(mask, lo, 1);
+        const longlong2* q = reinterpret_cast<const longlong2*>(a->in) +
+                             (long)(nb[4 * back + mu] & 0x7fffffffu) * 12 * Ls + s;
+        unsigned h[2] = {0, 0};  // real and imaginary parts of h, a bit a colour
+        for (int b = 0; b < 3; ++b) {
+            const longlong2 v = q[(3 * sp + b) * Ls], y = q[(3 * low + b) * Ls];
+            h[0] |= (unsigned)((v.x | (real ? y.x : y.y)) != 0) << b;
+            h[1] |= (unsigned)((v.y | (real ? y.y : y.x)) != 0) << b;
         }
-        for (int e = 0; e < 9; ++e) {
-            const int4 q = lk[l * 9 + e];
-            W[2 * e] = ldexp((double)(((i64)q.x << kFxLimb) + q.y), -2 * kFxLimb);
-            W[2 * e + 1] = ldexp((double)(((i64)q.z << kFxLimb) + q.w), -2 * kFxLimb);
+        unsigned u[3][2] = {};  // rows of U, a bit a column
+        const int4* W = lk + (4 * back + mu) * 9;
+        for (int r = 0; r < 2; ++r)
+            for (int c = 0; c < 3; ++c) {
+                const int4 e = W[back ? 3 * c + r : 3 * r + c];
+                u[r][0] |= (unsigned)((e.x | e.y) != 0) << c;
+                u[r][1] |= (unsigned)((e.z | e.w) != 0) << c;
+            }
+        auto next = [](unsigned m, int n) { return ((m | m << 3) >> n) & 7u; };  // bit c takes bit c + n (mod 3)
+        for (int i = 0; i < 2; ++i)
+            for (int j = 0; j < 2; ++j)
+                u[2][i ^ j] |= (next(u[0][i], 1) & next(u[1][j], 2)) | (next(u[0][i], 2) & next(u[1][j], 1));
+        unsigned w = 0;  // W h in the order of up
+        for (int c = 0; c < 3; ++c)
+            for (int b = 0; b < 3; ++b)
+                for (int i = 0; i < 2; ++i)
+                    for (int j = 0; j < 2; ++j)
+                        w |= ((back ? u[b][i] >> c : u[c][i] >> b) & (h[j] >> b) & 1u) << (2 * c + (i ^ j));
+        up |= w;
+        lo |= real ? w : swap(w);
+    }
+    return up | lo << 6;
+}
+
+// The hop sum of one 5D site in FP64 arithmetic by the two lanes of hop_fixed,
+// from the doubles behind the hop input and the links as stored: the sites
+// whose sums the integers cannot hold (fixed64.cuh).  small: the reals without
+// a large term (bits as in hop_terms), or bit 31 where a neighbour has no
+// integers; false, and nothing done, where the small ones are exact zeros.
+// pre: the input takes D~ / b5 (z, mz as in chi).  mask: the lanes that call,
+// both of a site.  Ls and fs are runtime values and one call serves both
+// steps: one copy for all kernels, few values to keep across it (two calls: H
+// at 24^3x64, Ls = 12 7.36 ms, one 7.20).  16^4, Ls = 16, all sites in FP64: K
+// 3.2 to 3.9 ms (2.36 ms for a kernel of FP64 arithmetic alone); all with zeros
+// that stay: 0.78 ms.
+static __device__ __noinline__ bool hop_fp64(const HopArgs* __restrict__ a, const int4* __restrict__ lk,
+                                             const unsigned* __restrict__ nb, long xcb, int s, int sp, int Ls, int fs,
+                                             bool pre, double z, double mz, unsigned mask, unsigned small,
+                                             double* __restrict__ out) {
+    const bool raw = small >> 31;
+    const unsigned held = __ballot_sync(mask, !raw);  // both lanes of a site alike
+    if (!raw) small &= hop_terms(a, lk, nb, s, sp, Ls, held);
+    mask = hop_sites(__ballot_sync(mask, small != 0));
+    if (!(mask >> (threadIdx.x & 31) & 1)) return false;
+    const bool canon = a->canon & 1;
+    const int cs = canon ? 1 : Ls, ss = canon ? 12 : 1;  // strides of components and of slices
+    double up[6], lo[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) up[i] = lo[i] = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < 8; ++k) {
+        const int mu = k >> 1;
+        const bool back = k & 1;
+        const unsigned e = nb[4 * back + mu];
+        const long n = (long)(e & 0x7fffffffu);
+        if (k == 4) {  // the lower sums so far belong to the other lane
+#pragma unroll
+            for (int i = 0; i < 6; ++i) lo[i] = __shfl_xor_sync(mask, lo[i], 1);
         }
-        switch (FS > 0 ? k : k ^ 1) {
-            case 0: hop_dir<double, 0, 1, false>(acc, p, W); break;
-            case 1: hop_dir<double, 0, -1, false>(acc, p, W); break;
-            case 2: hop_dir<double, 1, 1, false>(acc, p, W); break;
-            case 3: hop_dir<double, 1, -1, false>(acc, p, W); break;
-            case 4: hop_dir<double, 2, 1, false>(acc, p, W); break;
-            case 5: hop_dir<double, 2, -1, false>(acc, p, W); break;
-            case 6: hop_dir<double, 3, 1, false>(acc, p, W); break;
-            default: hop_dir<double, 3, -1, false>(acc, p, W); break;
+        const double2* p = reinterpret_cast<const double2*>(a->in_raw) +
+                           (canon ? lex_site(a->g, n, 1 - a->out_par) : n) * 12 * Ls;
+        auto load = [&](int spin, int b) {
+            const double2* q = p + (3 * spin + b) * cs;
+            double2 v = q[s * ss];
+            if (pre) {
+                const bool edge = spin < 2 ? s == 0 : s == Ls - 1;
+                const double2 w = q[(spin < 2 ? (edge ? Ls - 1 : s - 1) : (edge ? 0 : s + 1)) * ss];
+                const double f = edge ? -mz : z;
+                v.x += f * w.x;
+                v.y += f * w.y;
+            }
+            return v;
+        };
+        // h = psi_sp + f psi_low (mu = 1, 3) or psi_sp + i f psi_low
+        const bool real = mu & 1;
+        const double f = (back ? -fs : fs) * (mu == 0 || (mu != 3 && sp == 0) ? -1.0 : 1.0);
+        double2 h[3];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const double2 v = load(sp, b), y = load(mu < 2 ? 3 - sp : 2 + sp, b);
+            h[b] = make_double2(fma(f, real ? y.x : -y.y, v.x), fma(f, real ? y.y : y.x, v.y));
+        }
+        const double* rec = reinterpret_cast<const double*>(back ? a->lk_in : a->lk_out) +
+                            ((back ? n : xcb) * 4 + mu) * 12;
+        double u[18];
+#pragma unroll
+        for (int i = 0; i < 12; ++i) u[i] = rec[i];
+        // row 2 = conj(row 0 x row 1): lane 0 makes its real parts, lane 1 the imaginary ones
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const double* a1 = u + 2 * ((q + 1) % 3);
+            const double* a2 = u + 2 * ((q + 2) % 3);
+            const double *b1 = a1 + 6, *b2 = a2 + 6;
+            const double p1 = sp ? -b2[1] : b2[0], p2 = sp ? -b2[0] : -b2[1];
+            const double q1 = sp ? -b1[1] : b1[0], q2 = sp ? -b1[0] : -b1[1];
+            const double mine = (a1[0] * p1 + a1[1] * p2) - (a2[0] * q1 + a2[1] * q2);
+            const double other = __shfl_xor_sync(mask, mine, 1);
+            u[12 + 2 * q] = sp ? other : mine;
+            u[13 + 2 * q] = sp ? mine : other;
+        }
+        const bool neg = e >> 31;  // the boundary sign
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            if (neg) h[b] = make_double2(-h[b].x, -h[b].y);
+        }
+        double2 w[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) w[c] = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            if (h[b].x == 0.0 && h[b].y == 0.0) continue;  // the links are finite
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {  // U_cb, or conj(U_bc)
+                const int i = 6 * c + 2 * b, j = 6 * b + 2 * c;
+                const double x = back ? u[j] : u[i], y = back ? -u[j + 1] : u[i + 1];
+                w[c].x = fma(x, h[b].x, fma(-y, h[b].y, w[c].x));
+                w[c].y = fma(x, h[b].y, fma(y, h[b].x, w[c].y));
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            up[2 * c] += w[c].x;
+            up[2 * c + 1] += w[c].y;
+            lo[2 * c] = fma(f, real ? w[c].x : w[c].y, lo[2 * c]);
+            lo[2 * c + 1] = fma(f, real ? w[c].y : -w[c].x, lo[2 * c + 1]);
         }
     }
-    for (int i = 0; i < 24; ++i) out[i] = acc[i];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        out[i] = up[i];
+        out[6 + i] = lo[i];
+    }
+    return true;
 }
 
 // The hop sum of one 5D site in fixed point (fixed64.cuh) by two lanes: lane
@@ -835,38 +971,46 @@ static __device__ __noinline__ void hop_fp64_slow(const longlong2* in, const int
 // lower sums, so each ends with spins sp and 2 + sp.  sigma is the projector's
 // sign times the lane's sign in B (mu = 1: -, +; mu = 2: +, -); a lane takes
 // the direction with sigma = +1 first, so that the sign is the same for all.
-// Per lane: half the loads, products and sums and 96 registers instead of
-// 128 with spills (or 168).  lk: the site's 8 staged links (backward ones
-// daggered), nb its neighbour indices, mask: the lanes that call.  Two mu at
-// a time: four copies of the products fit the instruction cache, eight do not.
-template <int LS, bool DAG>
-__device__ __forceinline__ void hop_fixed(const void* __restrict__ in, const float* __restrict__ nrm,
-                                          const int4* __restrict__ lk, const unsigned* __restrict__ nb, int s, int sp,
-                                          unsigned mask, double* out) {
-    const longlong2* base = reinterpret_cast<const longlong2*>(in) + s;
-    const int* ex = reinterpret_cast<const int*>(nrm) + s;
+// Per lane: half the loads, products and sums of one lane for the site.  lk: the
+// site's 8 staged links (backward ones daggered), nb its neighbour indices,
+// mask: the lanes that call.  Two mu at a time: four copies of the products fit
+// the instruction cache, eight do not.  The units known beforehand and the
+// test for small terms cost 2 to 7% of the kernel (H at 24^3x64, Ls = 12 6.73 ->
+// 7.20 ms, K at 16^4, Ls = 16 598 -> 608 us, an FP64 CG iteration 1340 -> 1364).
+template <int LS, bool DAG, bool PRE>
+__device__ __forceinline__ void hop_fixed(const HopArgs& a, const SCoef<double>& cf, const int4* __restrict__ lk,
+                                          const unsigned* __restrict__ nb, long xcb, int s, int sp, unsigned mask,
+                                          double* out) {
+    const longlong2* base = reinterpret_cast<const longlong2*>(a.in) + s;
+    const int* ex = reinterpret_cast<const int*>(a.in_nrm) + s;
     i64 up[6], lo[6];
 #pragma unroll
     for (int i = 0; i < 6; ++i) up[i] = lo[i] = 0;
-    int E = 64;         // exponent field of the units of the sums
-    bool raw = false;   // a neighbour is kept as doubles
-    auto raise = [&](int e) {
-        if (e > E) {
-            const int sh = min(e - E, 63);
+    // E, the exponent field of the units of the sums, is the neighbours'
+    // largest; shl, shh: a byte for each direction, how far its own lies below
+    int E = 0;
+    unsigned shl = 0, shh = 0;
+    {
+        int e[8];
 #pragma unroll
-            for (int i = 0; i < 6; ++i) {
-                up[i] >>= sh;
-                lo[i] >>= sh;
-            }
-            E = e;
+        for (int l = 0; l < 8; ++l) {
+            e[l] = ex[(long)(nb[l] & 0x7fffffffu) * LS];
+            E = max(E, e[l]);
         }
-    };
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            shl |= (unsigned)min(E - e[l], 63) << (8 * l);
+            shh |= (unsigned)min(E - e[4 + l], 63) << (8 * l);
+        }
+    }
+    // a bit for each real of the upper and of the lower sums that some term of
+    // size 2^-kFxSmall of the unit's 2^56 or more has gone into
+    unsigned upm = 0, lom = 0;
     // B is -i times real for mu = 0, 2 and real for mu = 1, 3
     auto step = [&](auto real_c, auto plus_c, int l, int low) {
         constexpr bool REAL = decltype(real_c)::value, PLUS = decltype(plus_c)::value;
         const long n = (long)(nb[l] & 0x7fffffffu);
         const longlong2* q = base + n * (12 * LS);
-        const int e = ex[n * LS];
         const longlong2* qu = q + 3 * sp * LS;
         const longlong2* ql = q + low * LS;
         i64 h[6], w[6];
@@ -881,15 +1025,19 @@ __device__ __forceinline__ void hop_fixed(const void* __restrict__ in, const flo
                 h[2 * c + 1] = PLUS ? t.y - b.x : t.y + b.x;
             }
         }
-        raw = raw || e == kFxRaw;
-        raise(e);
-        if (e < E) {
-            const int sh = min(E - e, 63);
-            const i64 half = 1ll << (sh - 1);
+        const int sh = __byte_perm(shl, shh, l) & 63;
+        const i64 half = (i64)((1ull << sh) >> 1);
 #pragma unroll
-            for (int i = 0; i < 6; ++i) h[i] = (h[i] + half) >> sh;
-        }
+        for (int i = 0; i < 6; ++i) h[i] = (h[i] + half) >> sh;
         fx_mul(lk + l * 9, h, w);
+        unsigned big = 0;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            constexpr unsigned T = 1u << (kFxFrac - 32 - kFxSmall);
+            if ((unsigned)((int)(w[i] >> 32)) + T >= 2 * T) big |= 1u << i;
+        }
+        upm |= big;
+        lom |= REAL ? big : ((big & 0x15u) << 1) | ((big >> 1) & 0x15u);
 #pragma unroll
         for (int i = 0; i < 6; i += 2) {
             up[i] += w[i];
@@ -915,26 +1063,25 @@ __device__ __forceinline__ void hop_fixed(const void* __restrict__ in, const flo
         step(F{}, F{}, l + (fi ^ BACK ^ 4), low);
         step(T{}, T{}, l + 1 + (fr ^ BACK), low);
         step(T{}, F{}, l + 1 + (fr ^ BACK ^ 4), low);
-        if (half == 0) {
-            raise(__shfl_xor_sync(mask, E, 1));  // one unit for both lanes
+        if (half == 0) {  // both lanes have the same unit
 #pragma unroll
             for (int i = 0; i < 6; ++i) lo[i] = __shfl_xor_sync(mask, lo[i], 1);
+            lom = __shfl_xor_sync(mask, lom, 1);
         }
     }
-    if (!raw) {
 #pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            out[i] = fx_to(up[i], E);
-            out[6 + i] = fx_to(lo[i], E);
-        }
-    } else {
-        double r[24];
-        hop_fp64_slow(reinterpret_cast<const longlong2*>(in), reinterpret_cast<const int*>(nrm), lk, nb, s, LS,
-                      DAG ? 1 : -1, r);
+    for (int i = 0; i < 6; ++i) {
+        out[i] = fx_to(up[i], E);
+        out[6 + i] = fx_to(lo[i], E);
+    }
+    // sites for FP64 arithmetic (E = 0: every neighbour is zero)
+    const unsigned small = E == kFxRaw ? 1u << 31 : E > 0 ? ~(upm | lom << 6) & 0xfffu : 0u;
+    const unsigned slow = hop_sites(__ballot_sync(mask, small != 0));
+    if (slow >> (threadIdx.x & 31) & 1) {
+        double r[12];
+        if (hop_fp64(&a, lk, nb, xcb, s, sp, LS, DAG ? 1 : -1, PRE, cf.zb, cf.mzb, slow, small, r)) {
 #pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            out[i] = sp ? r[6 + i] : r[i];
-            out[6 + i] = sp ? r[18 + i] : r[12 + i];
+            for (int i = 0; i < 12; ++i) out[i] = r[i];
         }
     }
 }
@@ -1150,8 +1297,8 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
             if constexpr (KT::HOP) {
                 constexpr int FS = KT::DAG ? +1 : -1;  // forward projector 1 + FS gamma
                 if constexpr (FX) {
-                    hop_fixed<LS, KT::DAG>(a.in, a.in_nrm, reinterpret_cast<const int4*>(slc + il * 8 * LK),
-                                           snc + il * 8, s, sp, mask, acc);
+                    hop_fixed<LS, KT::DAG, KT::PRE>(a, cf, reinterpret_cast<const int4*>(slc + il * 8 * LK),
+                                                    snc + il * 8, xcb, s, sp, mask, acc);
                 } else
                 // hop k = 2 mu + dir (dir 0 forward, 1 backward)
 #pragma unroll
@@ -1249,10 +1396,13 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
                 for (int i = 0; i < NR; ++i)
                     o[i] = KIND == KIND_H ? cf.kTi * o[i] - (R)0.5 * acc[i] : o[i] + cf.fR * acc[i];
             }
+            void* out = a.out;
             if constexpr (FX && KT::FXOUT) {
-                if constexpr (HV == 2) fx_store_part(a.out, a.out_nrm, xcb, s, LS, sp, o, mask);
-                else fx_store(a.out, a.out_nrm, xcb, s, LS, o);
-            } else if (CANON && a.canon) {
+                if constexpr (HV == 2) fx_store_part(out, a.out_nrm, xcb, s, LS, sp, o, mask);
+                else fx_store(out, a.out_nrm, xcb, s, LS, o);
+                out = a.out_raw;
+            }
+            if (CANON && a.canon) {
                 const bool g5 = a.canon & 2;
                 double2* p = reinterpret_cast<double2*>(a.out) + (lex * LS + (g5 ? LS - 1 - s : s)) * 12 + 3 * sp;
                 const double f = g5 ? -1.0 : 1.0;
@@ -1262,14 +1412,14 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
                     p[6 + c] = make_double2(f * o[HF + 2 * c], f * o[HF + 2 * c + 1]);
                 }
             } else if constexpr (HV == 2) {
-                double2* p = reinterpret_cast<double2*>(a.out) + (xcb * 12 + 3 * sp) * LS + s;
+                double2* p = reinterpret_cast<double2*>(out) + (xcb * 12 + 3 * sp) * LS + s;
 #pragma unroll
                 for (int c = 0; c < HF / 2; ++c) {
                     p[c * LS] = make_double2(o[2 * c], o[2 * c + 1]);
                     p[(6 + c) * LS] = make_double2(o[HF + 2 * c], o[HF + 2 * c + 1]);
                 }
             } else {
-                store_sp<S, R>(a.out, a.out_nrm, xcb, s, LS, o);
+                store_sp<S, R>(out, a.out_nrm, xcb, s, LS, o);
             }
             if (a.rd.fin != FIN_NONE) {
 #pragma unroll
@@ -1285,14 +1435,17 @@ __device__ __forceinline__ void hop_body(const HopArgs& a, const SCoef<typename 
     if (a.rd.fin != FIN_NONE) block_reduce_finalize<NT>(nn, a.rd);
 }
 
-// the kernel with the compiler's own register choice (variants 0, 1; the FP64
-// hop kinds: 20 warps per SM, 96 registers; caps of 16 and 24 warps measured
-// 428 and 408 us against 370 us for K^dag at 12^3x24, Ls = 12, and 7.65 and
-// 6.50 ms against 6.94 ms for H at 24^3x64, Ls = 12) ...
+// Threads per SM that the FP64 hop kinds leave registers for (128 a thread).
+// 512 against 640 threads: K at 16^4, Ls = 16 587 against 616 us, FP64 CG
+// iteration 1357 against 1377 us, at 4^4, Ls = 8 76 against 80 us, at 12^3x24,
+// Ls = 12 689 against 716 us; 768 threads lost everywhere.
+constexpr int kFp64Threads = 512;
+
+// the kernel with the compiler's own register choice (variants 0, 1) ...
 template <typename S, int LS, int KIND, int VAR = 0>
 __global__ void __launch_bounds__(HopTile<S, LS, KIND, VAR>::NT,
-                                  HopTile<S, LS, KIND, VAR>::HV == 2 ? 640 / HopTile<S, LS, KIND, VAR>::NT : 1)
-    hop_kernel(const HopArgs a, const SCoef<typename Traits<S>::R> cf) {
+                                  HopTile<S, LS, KIND, VAR>::HV == 2 ? kFp64Threads / HopTile<S, LS, KIND, VAR>::NT : 1)
+    hop_kernel(const __grid_constant__ HopArgs a, const SCoef<typename Traits<S>::R> cf) {
     hop_body<S, LS, KIND, VAR>(a, cf);
 }
 
@@ -1301,7 +1454,7 @@ struct HopPair {
     HopArgs a[2];
 };
 template <typename S, int LS, int KIND>
-__global__ void __launch_bounds__(HopTile<S, LS, KIND, 0>::NT, 640 / HopTile<S, LS, KIND, 0>::NT)
+__global__ void __launch_bounds__(HopTile<S, LS, KIND, 0>::NT, kFp64Threads / HopTile<S, LS, KIND, 0>::NT)
     hop_kernel_pair(const __grid_constant__ HopPair p, const SCoef<typename Traits<S>::R> cf) {
     hop_body<S, LS, KIND, 0>(p.a[blockIdx.y], cf);
 }
@@ -1309,7 +1462,7 @@ __global__ void __launch_bounds__(HopTile<S, LS, KIND, 0>::NT, 640 / HopTile<S, 
 // ... and with capped registers (variants 2, 3; FP32 arithmetic)
 template <typename S, int LS, int KIND, int VAR>
 __global__ void __launch_bounds__(Tile<LS, VAR>::NT, MinBlocksCap<LS, VAR>::V)
-    hop_kernel_rc(const HopArgs a, const SCoef<typename Traits<S>::R> cf) {
+    hop_kernel_rc(const __grid_constant__ HopArgs a, const SCoef<typename Traits<S>::R> cf) {
     hop_body<S, LS, KIND, VAR>(a, cf);
 }
 

@@ -145,8 +145,8 @@ eofa_status dalloc(eofa_ctx* c, void** p, size_t bytes) {
 }
 
 // hop_in: the vector may hold an FP64 hop input (fixed point with an exponent
-// per 5D site)
-eofa_status vec_alloc(eofa_ctx* c, int prec, VecRef* v, bool hop_in = false) {
+// per 5D site); raw: one that a hop kernel writes, with its doubles
+eofa_status vec_alloc(eofa_ctx* c, int prec, VecRef* v, bool hop_in = false, bool raw = false) {
     eofa_status s = dalloc(c, &v->d, (size_t)c->n5 * 24 * kWidth[prec]);
     if (s != EOFA_OK) return s;
     v->n = nullptr;
@@ -156,7 +156,8 @@ eofa_status vec_alloc(eofa_ctx* c, int prec, VecRef* v, bool hop_in = false) {
         if (s != EOFA_OK) return s;
         v->n = (float*)n;
     }
-    return EOFA_OK;
+    v->raw = nullptr;
+    return raw ? dalloc(c, &v->raw, (size_t)c->n5 * 24 * sizeof(double)) : EOFA_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -319,19 +320,22 @@ int hop_input_pass(int kind) {
 
 eofa_status hop(eofa_ctx* c, int prec, int kind, int out_par, VecRef in, VecRef y, VecRef out, Reduce rd,
                 const int* done, cudaStream_t st, bool timed = false, int* stop = nullptr) {
+    const void* in_raw = in.raw;
     if (const int pass = prec == EOFA_F64 ? hop_input_pass(kind) : 0) {
         // into c->ro, which holds nothing live at any of these launches
         // (outer_residual writes it last)
         CKL(blas_hop_input(c->ro, in, c->n5, c->g.Ls, pass == 2, c->c64.zb, c->c64.mzb, st, done), "hop input");
+        in_raw = in.d;
         in = c->ro;
     }
+    if (prec == EOFA_F64 && in.d && !in_raw) return fail(c, EOFA_ERR_ARG, "FP64 hop input without its doubles");
     HopArgs a;
     std::memset(&a, 0, sizeof(a));
     a.g = c->g;
     a.out_par = out_par;
-    a.in = in.d; a.in_nrm = in.n;
+    a.in = in.d; a.in_nrm = in.n; a.in_raw = in_raw;
     a.y = y.d; a.y_nrm = y.n;
-    a.out = out.d; a.out_nrm = out.n;
+    a.out = out.d; a.out_nrm = out.n; a.out_raw = out.raw;
     a.lk_out = c->links[prec][out_par];
     a.lk_in = c->links[prec][1 - out_par];
     a.rd = rd;
@@ -395,7 +399,7 @@ eofa_status ensure_inner(eofa_ctx* c, int P) {
     if (in.ready) return EOFA_OK;
     eofa_status s;
     if ((s = vec_alloc(c, P, &in.r)) || (s = vec_alloc(c, P, &in.p)) || (s = vec_alloc(c, P, &in.q)) ||
-        (s = vec_alloc(c, P, &in.z)) || (s = vec_alloc(c, P, &in.t, P == EOFA_F64)) ||
+        (s = vec_alloc(c, P, &in.z)) || (s = vec_alloc(c, P, &in.t, P == EOFA_F64, P == EOFA_F64)) ||
         (s = vec_alloc(c, P == EOFA_F64 ? EOFA_F64 : EOFA_F32, &in.x)))
         return s;
     in.ready = true;
@@ -1413,12 +1417,14 @@ eofa_status apply_impl(eofa_ctx* c, const void* in, void* out, int which, cudaSt
         a.out_par = par;
         a.in = c->t[1 - par].d;
         a.in_nrm = c->t[1 - par].n;
+        a.in_raw = in;
         a.y = in;
         a.out = out;
         a.lk_out = c->links[EOFA_F64][par];
         a.lk_in = c->links[EOFA_F64][1 - par];
         a.canon = which == 2 ? 3 : 1;
         if (overlap) {
+            a.in_raw = c->x[1 - par].d;
             a.y = c->x[par].d;
             a.y_nrm = c->x[par].n;
             a.out = res[par].d;
@@ -1795,7 +1801,7 @@ static eofa_status create_impl(const eofa_params* p, const void* gauge, int gpma
             if ((s = dalloc(c, &c->links[pr][par], (size_t)g.Vh * 4 * 12 * kWidth[pr]))) return bail(s);
     for (int par = 0; par < 2; ++par) {
         if ((s = vec_alloc(c, 0, &c->b[par])) || (s = vec_alloc(c, 0, &c->x[par])) ||
-            (s = vec_alloc(c, 0, &c->t[par], true)))
+            (s = vec_alloc(c, 0, &c->t[par], true, par == 0)))
             return bail(s);
     }
     if ((s = vec_alloc(c, 0, &c->ro, true)) || (s = vec_alloc(c, 0, &c->bto)) || (s = vec_alloc(c, 0, &c->qo)))
@@ -2250,6 +2256,7 @@ extern "C" eofa_status eofa_apply_noalloc(const eofa_params* p, const void* gaug
         a.out_par = par;
         a.in = chi.d;
         a.in_nrm = chi.n;
+        a.in_raw = fin[1 - par].d;
         a.y = fin[par].d;
         a.out = fout[par].d;
         a.lk_out = links[EOFA_F64][par];

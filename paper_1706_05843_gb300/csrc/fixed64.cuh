@@ -8,30 +8,39 @@
 //  * a spinor that a hop reads is kept in memory as 24 signed integers in
 //    units of 2^(E-56) and E, the exponent field of its largest real (fx_pack,
 //    by the kernel that makes it): 57 bits, so every real within 2^-4 of the
-//    largest is exact and the others keep an absolute error below one unit,
-//    2^-3 of the ulp of the largest;
+//    largest is exact and the others are rounded to half a unit, 2^-5 of the
+//    ulp of the largest;
 //  * spin projection and reconstruction are 64-bit integer additions (exact);
 //  * a link's reals are 58-bit fixed point (Uh, Ul): u = (Uh 2^29 + Ul) 2^-58,
 //    |Ul| <= 2^28; a projected component is H = Hh 2^29 + Hl likewise, and
 //    U H = sum Uh Hh + 2^-29 sum (Uh Hl + Ul Hh): three mad.wide a product.
 //    The dropped 2^-58 Ul Hl is below 1/4 unit and has zero mean;
-//  * the eight directions accumulate in 64-bit integers at the largest
-//    exponent met so far (a larger one shifts the sums right).  Bound: reals
-//    below 2^57 units, |h| <= sqrt(3) 2 sqrt(2) 2^57 for a projected colour
-//    vector, |U h| = |h|, eight directions: below 2^62.3.
+//  * the eight directions accumulate in 64-bit integers at the largest of
+//    their eight exponents, to which each projected vector is rounded.  Bound:
+//    reals below 2^57 units, |h| <= sqrt(3) 2 sqrt(2) 2^57 for a projected
+//    colour vector, |U h| = |h|, eight directions: below 2^62.3.
 //
-// The result is rounded to FP64 once.  A spinor with Inf, NaN or extreme
-// magnitude (exponent field of the largest real outside [64, 2030]) is kept
-// as its doubles (E = kFxRaw); threads that meet one redo their sums in FP64
-// arithmetic (hop_fp64_slow).
+// The result is rounded to FP64 once.  Error of a real: at most 96 units (per
+// direction 4.9 from the reals, which are off by half a unit, or one where they
+// are smaller than that; 1.2 from the alignment, 2.8 from the low products, 3
+// from the links; 3 units rms in all), which relative to the neighbours'
+// largest real is below that of FP64 sums.  But a real can be made of small
+// terms alone (a colour or a spin that is small all over the neighbourhood,
+// links that hardly mix colours), and FP64 keeps its 53 bits.  So the sums are
+// taken only where each of them has a term U h of at least 2^-kFxSmall of the
+// unit's 2^56 in it, or nothing but exact zeros (hop_terms): then the error is
+// at most 96 2^-51 of the largest term (3 2^-51 rms).  Other sites, and those
+// with a neighbour of Inf, NaN or extreme magnitude (exponent field of the
+// largest real outside [64, 2030]: E = kFxRaw), are computed again in FP64
+// from the doubles behind the integers and from the links as they are stored
+// (hop_fp64).  Where the eight terms are alike in size, one real in 2^37 finds
+// all of them small.
 //
-// Measured, one launch at 16^4, Ls = 16 (524288 5D sites): FP64 arithmetic
-// 1.04 ms (mean of kinds 0 to 3, FP64 pipe 88-90% busy), this form 0.24 to
-// 0.36 ms (the fifth dimension is FP64 still: 42% of its pipe; the integer
-// pipes 40-52%, 46% of the issue slots: fixed-latency dependencies at 19
-// warps per SM) plus 0.025 to 0.041 ms for the input pass.  Error of K, K^dag and H against extended
-// precision (random SU(3), Ls 4 to 16): 1.61e-16 to 1.69e-16 relative,
-// 1.66e-16 to 1.99e-16 with FP64 arithmetic.
+// Measured, a half of S at 16^4, Ls = 16 with its input pass (524288 5D sites):
+// FP64 arithmetic 0.90 to 1.15 ms (FP64 pipe 88-90% busy), this form 0.28 to
+// 0.31 ms.  Error of K, K^dag and H against extended precision (random SU(3),
+// Ls 4 to 16): 1.61e-16 to 1.69e-16 relative, 1.66e-16 to 1.99e-16 with FP64
+// arithmetic.
 #pragma once
 
 #include "common.cuh"
@@ -49,13 +58,14 @@ __device__ __forceinline__ int2 fx_split(i64 v) {
     return make_int2((int)((v + (1 << (kFxLimb - 1))) >> kFxLimb), lo);
 }
 
-// the double (hi, lo) in units of 2^(E - 1023 - frac), truncated; E at least
-// its exponent field, frac 56 (spinors) or 58 (links)
+// the double (hi, lo) in units of 2^(E - 1023 - frac), rounded, but 1 or -1
+// where that would make 0 of another number; E at least its exponent field and
+// 64, frac 56 (spinors) or 58 (links)
 template <int FRAC>
 __device__ __forceinline__ i64 fx_from(int hi, unsigned lo, int E) {
-    const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
-    const int sh = min(E - (int)(((unsigned)hi >> 20) & 0x7ffu), 63);
-    const i64 m = (i64)((((unsigned long long)mh << 32) | lo) << (FRAC - 52) >> sh);
+    const unsigned mh = ((unsigned)hi & 0xfffffu) | (((unsigned)hi & 0x7fffffffu) | lo ? 0x100000u : 0u);
+    const int sh = min(E - (int)(((unsigned)hi >> 20) & 0x7ffu), FRAC + 1);
+    const i64 m = (i64)((((((unsigned long long)mh << 32) | lo) << (FRAC - 51) >> sh) + 1) >> 1);
     return hi < 0 ? -m : m;
 }
 
@@ -64,10 +74,11 @@ __device__ __forceinline__ i64 fx_link(double u) {
     return fx_from<2 * kFxLimb>(__double2hiint(u), (unsigned)__double2loint(u), 1023);
 }
 
-constexpr int kFxRaw = 2047;  // exponent mark of a spinor kept as doubles
+constexpr int kFxRaw = 2047;     // exponent mark of a spinor that has no integer form
+constexpr int kFxSmall = 5;      // a term below 2^-5 of the unit's 2^56 is small
 
 // N reals of a spinor -> their fixed-point form; returns E (0 for a zero
-// spinor).  N = 12: the two lanes (sp = 0, 1) of a spinor share its exponent;
+// spinor, kFxRaw for one that has no such form).  N = 12: the two lanes (sp = 0, 1) of a spinor share its exponent;
 // mask: the lanes that call.
 template <int N>
 __device__ __forceinline__ int fx_pack(const double* v, i64* m, unsigned mask = 0) {
@@ -86,7 +97,7 @@ __device__ __forceinline__ int fx_pack(const double* v, i64* m, unsigned mask = 
     if (E < 64 || E > 2030) {
         const bool zero = top == 0 && low == 0;
 #pragma unroll
-        for (int i = 0; i < N; ++i) m[i] = zero ? 0 : __double_as_longlong(v[i]);
+        for (int i = 0; i < N; ++i) m[i] = 0;
         return zero ? 0 : kFxRaw;
     }
 #pragma unroll
@@ -94,8 +105,7 @@ __device__ __forceinline__ int fx_pack(const double* v, i64* m, unsigned mask = 
     return E;
 }
 
-// the fixed-point spinor of 5D site (xcb, s) stored in place of 24 doubles,
-// its exponent in the site's scale slot
+// the fixed-point spinor of 5D site (xcb, s), its exponent in the site's scale slot
 __device__ __forceinline__ void fx_store(void* base, float* nrm, long xcb, int s, int Ls, const double* v) {
     i64 m[24];
     const int E = fx_pack<24>(v, m);
@@ -105,7 +115,7 @@ __device__ __forceinline__ void fx_store(void* base, float* nrm, long xcb, int s
     reinterpret_cast<int*>(nrm)[xcb * Ls + s] = E;
 }
 
-// units of 2^(E - 1023 - 56) -> double, E in [64, 2030]
+// units of 2^(E - 1023 - 56) -> double, E in [64, 2030] unless v = 0
 __device__ __forceinline__ double fx_to(i64 v, int E) {
     const double d = (double)v;  // |v| < 2^63: rounded to nearest
     const int hi = __double2hiint(d) + ((E - 1023 - kFxFrac) << 20);
