@@ -10,6 +10,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 namespace eofa {
 
@@ -430,6 +431,10 @@ __global__ void __launch_bounds__(kCvThreads, 1)
 // k16 products in the tensor cores, then FP32 registers over the CTA's share,
 // one atomic per element and CTA.  Bound by the mma.sync rate (math pipe
 // throttle leads the stalls; nine warps of 32 channels: 0.93 ms).
+// The zero rows of dy would turn an Inf of in into NaN: a CTA whose sums are
+// not all finite makes them again with the halo's rows of in zero as well
+// (that in every pass: the network's gradients at 16^3 x 32, 8 slices 4.31 ->
+// 4.81 ms; on demand 4.27 -> 4.37 ms, the second walk's registers).
 // ---------------------------------------------------------------------------
 constexpr int kWgThreads = 576;
 constexpr int kWgStages = 3;
@@ -442,6 +447,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     const int stage_elems = (kCvRows + 3 * pl.np) * 32;
     bf16* st0 = reinterpret_cast<bf16*>(wg_smem);                                   // [stages][dy | in dz 0..2]
     int2* tab = reinterpret_cast<int2*>(st0 + (size_t)kWgStages * stage_elems);     // [np]: (y X + x, z or -1 - z)
+    __shared__ unsigned s_rows[kWgStages][kCvRows / 32];                            // a bit for each row of the lattice
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int dt = blockIdx.x % 3 - 1, rank = blockIdx.x / 3, ranks = gridDim.x / 3;
     const long steps = (long)g.S * pl.nxb * pl.tiles * g.T;
@@ -449,6 +455,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     const long slice = (long)g.Z * g.Y * g.X;
 
     long tab_col = -1;
+    bool redo = false;
     auto issue = [&](long s, int buf) {
         const long col = s / g.T;
         const int t = (int)(s - col * g.T);
@@ -466,6 +473,10 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 tab[pos] = make_int2(wrapi(yp - 1, g.Y) * g.X + wrapi(xr, g.X), valid ? z : -1 - z);
             }
             __syncthreads();
+        }
+        if (redo && tid < kCvRows) {
+            const unsigned rows = __ballot_sync(0xffffffffu, tab[tid + pl.line + 1].y >= 0);
+            if (lane == 0) s_rows[buf][warp] = rows;
         }
         bf16* sD = st0 + (size_t)buf * stage_elems;
         const int ti = wrapi(t + dt, g.T);
@@ -500,45 +511,65 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         }
     };
 
-    for (int i = 0; i < kWgStages - 1; ++i) {
-        if (s0 + i < s1) issue(s0 + i, i);
-        cp_commit();
-        __syncthreads();  // the table may be rewritten by the next issue
-    }
     const int dz = warp % 9 / 3, dyy = warp % 3, nh = warp / 9;
     const int i8 = lane >> 3;
-    int buf = 0;
-    for (long s = s0; s < s1; ++s) {
-        cp_wait<kWgStages - 2>();
-        __syncthreads();  // this step's stage has arrived; the oldest stage and the table are free
-        const long nx = s + kWgStages - 1;
-        if (nx < s1) issue(nx, buf == 0 ? kWgStages - 1 : buf - 1);
-        cp_commit();
-        const bf16* D = st0 + (size_t)buf * stage_elems;
-        const bf16* In = D + (kCvRows + dz * pl.np) * 32;
-        const int off = dyy * pl.line;
-#pragma unroll 2
-        for (int kb = 0; kb < kCvRows / 16; ++kb) {
-            unsigned af[2][4], bfr[3][4];
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)   // A = dy^T: (co, k) from rows k, columns co
-                ldsm_x4_t(af[mt], D + swz(kb * 16 + (lane & 7) + (i8 >> 1) * 8, mt * 2 + (i8 & 1)));
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx)   // B = in_shift: (k, ci) rows k
-                ldsm_x4_t(bfr[dx], In + swz(off + dx + kb * 16 + (lane & 7) + (i8 & 1) * 8, nh * 2 + (i8 >> 1)));
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-                for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt)
-                        mma16816(acc[dx][mt][nt], af[mt], bfr[dx][nt * 2], bfr[dx][nt * 2 + 1]);
+    auto walk = [&](auto masked) {
+        for (int i = 0; i < kWgStages - 1; ++i) {
+            if (s0 + i < s1) issue(s0 + i, i);
+            cp_commit();
+            __syncthreads();  // the table may be rewritten by the next issue
         }
-        if ((s - s0) % kWgFlush == kWgFlush - 1) flush();
-        buf = buf + 1 == kWgStages ? 0 : buf + 1;
+        int buf = 0;
+        for (long s = s0; s < s1; ++s) {
+            cp_wait<kWgStages - 2>();
+            __syncthreads();  // this step's stage has arrived; the oldest stage and the table are free
+            const long nx = s + kWgStages - 1;
+            if (nx < s1) issue(nx, buf == 0 ? kWgStages - 1 : buf - 1);
+            cp_commit();
+            const bf16* D = st0 + (size_t)buf * stage_elems;
+            const bf16* In = D + (kCvRows + dz * pl.np) * 32;
+            const int off = dyy * pl.line;
+#pragma unroll 2
+            for (int kb = 0; kb < kCvRows / 16; ++kb) {
+                unsigned af[2][4], bfr[3][4];
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt)   // A = dy^T: (co, k) from rows k, columns co
+                    ldsm_x4_t(af[mt], D + swz(kb * 16 + (lane & 7) + (i8 >> 1) * 8, mt * 2 + (i8 & 1)));
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx)   // B = in_shift: (k, ci) rows k
+                    ldsm_x4_t(bfr[dx], In + swz(off + dx + kb * 16 + (lane & 7) + (i8 & 1) * 8, nh * 2 + (i8 >> 1)));
+                if constexpr (decltype(masked)::value) {  // this lane's rows k: 2 (lane & 3) + 0, 1 and those + 8
+                    const unsigned rows = s_rows[buf][kb >> 1] >> ((kb & 1) * 16 + (lane & 3) * 2);
+                    const unsigned m0 = (rows & 1) * 0xffffu | (rows >> 1 & 1) * 0xffff0000u;
+                    const unsigned m1 = (rows >> 8 & 1) * 0xffffu | (rows >> 9 & 1) * 0xffff0000u;
+#pragma unroll
+                    for (int i = 0; i < 12; ++i) bfr[i / 4][i % 4] &= i % 2 ? m1 : m0;
+                }
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                        for (int nt = 0; nt < 2; ++nt)
+                            mma16816(acc[dx][mt][nt], af[mt], bfr[dx][nt * 2], bfr[dx][nt * 2 + 1]);
+            }
+            if ((s - s0) % kWgFlush == kWgFlush - 1) flush();
+            buf = buf + 1 == kWgStages ? 0 : buf + 1;
+        }
+        cp_wait<0>();
+        flush();
+    };
+    walk(std::integral_constant<bool, false>{});
+    float odd = 0.f;
+#pragma unroll
+    for (int i = 0; i < 48; ++i) odd += 0.f * (&sum[0][0][0][0])[i];
+    if (__syncthreads_or(odd != 0.f)) {  // (NaN: 0 x Inf or 0 x NaN)
+#pragma unroll
+        for (int i = 0; i < 48; ++i) (&sum[0][0][0][0])[i] = 0.f;
+        tab_col = -1;
+        redo = true;
+        walk(std::integral_constant<bool, true>{});
     }
-    cp_wait<0>();
-    flush();
     if (s0 == s1) return;
 #pragma unroll
     for (int dx = 0; dx < 3; ++dx) {
