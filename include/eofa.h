@@ -449,7 +449,7 @@ double eofa_hop_bytes(const eofa_ctx *ctx, int prec, int with_local);
  * of the inner solver (0: S step 1, 1: S step 2, 2: S^dag step 1, 3: S^dag
  * step 2) in precision prec; the default tile if that precision has not been
  * used by a solve yet.  Block and tile shapes are timed on the context's own
- * buffers at its first solve in a precision and cached per lattice shape. */
+ * buffers at its first solve in a precision and cached per device and lattice. */
 int eofa_tile_sites(const eofa_ctx *ctx, int prec, int kind);
 
 /* The tile variant chosen for the same kernel: bit 0 set for the
@@ -467,8 +467,8 @@ int eofa_tile_variant(const eofa_ctx *ctx, int prec, int kind);
  * (the dslash sweep over tile shapes; FP64 has variants 0 and 1 only).  0
  * when that variant was not timed (not compiled for the precision, the
  * variant fixed by EOFA_TILE_VARIANT, or no solve in that precision yet);
- * -1 for invalid arguments.  Contexts of a lattice shape already tuned in the
- * process report the first context's times. */
+ * -1 for invalid arguments.  Contexts of a lattice already tuned on the
+ * same device, with the same G-parity directions, report the first one's times. */
 double eofa_tile_time(const eofa_ctx *ctx, int prec, int kind, int variant);
 
 #ifdef __cplusplus

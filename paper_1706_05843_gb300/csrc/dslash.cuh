@@ -107,6 +107,7 @@ struct HopArgs {
     Reduce rd;                               // rd.fin == FIN_NONE: no reduction
     const int* done;                         // early exit when *done != 0 (may be NULL)
     int* stop;                               // set by a launch that finds *done set (may be NULL)
+    int prepare;                             // 1: set the kernel up on the current device, launch nothing
     int canon;                               // KT::APPLY kinds, bit 0: y, in_raw and out are canonical complex128
                                              // fields of the whole lattice; bit 1: out takes gamma_5 R_5
     // dense kinds: the Ls x Ls s-space matrix of each chirality in compute

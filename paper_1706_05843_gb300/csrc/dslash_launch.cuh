@@ -21,8 +21,9 @@ constexpr int kHopMaxDevices = 64;
 // The CTAs of one kernel that one SM holds, on the current device (the
 // persistent grids are that many per SM).  Once per kernel and device, before
 // its first launch there: the shared-memory limit, an attribute of the current
-// device; not inside a stream capture (the drivers launch every kernel once
-// before they capture it, and a context sets up its applications' kernels).
+// device; not inside a stream capture (a context sets up its applications'
+// kernels when it is created and a solve's before the first capture:
+// prepare_solve).
 struct HopResident {
     std::atomic<int> of[kHopMaxDevices] = {};
     std::mutex mu;
@@ -68,7 +69,7 @@ static cudaError_t launch_one(const HopArgs& a, const SCoef<typename Traits<S>::
     constexpr bool RCAP = (VAR & 2) != 0;
     int dev = 0, resident = 0;
     cudaError_t e = resident_one<S, LS, K, VAR>(st, &dev, &resident);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || a.prepare) return e;
     const long nblk = ((long)a.g.Vh + NS - 1) / NS;
     if (nblk == 0) return cudaSuccess;
     int sms = 0;

@@ -318,6 +318,15 @@ int hop_input_pass(int kind) {
     }
 }
 
+cudaError_t launch_hop(int prec, int kind, const HopArgs& a, const void* coef, cudaStream_t st) {
+    switch (prec) {
+        case EOFA_F64: return launch_hop_f64(kind, a, coef, st);
+        case EOFA_F32: return launch_hop_f32(kind, a, coef, st);
+        case EOFA_F16: return launch_hop_f16(kind, a, coef, st);
+        default: return launch_hop_bf16(kind, a, coef, st);
+    }
+}
+
 eofa_status hop(eofa_ctx* c, int prec, int kind, int out_par, VecRef in, VecRef y, VecRef out, Reduce rd,
                 const int* done, cudaStream_t st, bool timed = false, int* stop = nullptr) {
     const void* in_raw = in.raw;
@@ -356,13 +365,7 @@ eofa_status hop(eofa_ctx* c, int prec, int kind, int out_par, VecRef in, VecRef 
         }
         CK(cudaEventRecord(c->evs[c->ev_used], st), "cudaEventRecord");
     }
-    cudaError_t e;
-    switch (prec) {
-        case EOFA_F64: e = launch_hop_f64(kind, a, coef, st); break;
-        case EOFA_F32: e = launch_hop_f32(kind, a, coef, st); break;
-        case EOFA_F16: e = launch_hop_f16(kind, a, coef, st); break;
-        default: e = launch_hop_bf16(kind, a, coef, st); break;
-    }
+    const cudaError_t e = launch_hop(prec, kind, a, coef, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "hop kernel launch");
     ++c->launches;
     if (tm) {
@@ -409,33 +412,61 @@ eofa_status ensure_inner(eofa_ctx* c, int P) {
 // ---------------------------------------------------------------------------
 // autotuner: for each of the four inner-solver hop kinds of a precision,
 // time both CTA tile variants on this context's buffers and keep the faster.
-// Choices are cached per (precision, Ls, lattice) for every context of the
-// process; tuning happens before any CG graph is captured.
+// Choices are cached per device, precision, lattice and G-parity directions
+// for every context of the process; tuning, and the set-up of the kernels that
+// a captured solve launches, happen before any CG graph is captured.
 // ---------------------------------------------------------------------------
 std::mutex g_tune_mu;
 struct TuneChoice {
     int variant = 0;
     float ms[4] = {0.f, 0.f, 0.f, 0.f};  // per launch of each variant (0: not timed)
 };
-std::map<std::array<long, 5>, TuneChoice> g_tune_cache;  // (prec, Ls, X*Y, Z*T, kind) -> choice
+typedef std::array<int, 9> TuneKey;  // device, precision, Ls, X, Y, Z, T, G-parity directions, kind
+std::map<TuneKey, TuneChoice> g_tune_cache;
+
+TuneKey tune_key(int dev, int P, const Geom& g, int kind) {
+    return {dev, P, g.Ls, g.X, g.Y, g.Z, g.T, g.gpmask, kind};
+}
+
+// Set up, on the current device, the hop kernels that a captured solve of inner
+// precision P launches (a kernel's set-up must not run inside a capture).
+eofa_status prepare_solve(eofa_ctx* c, int P, cudaStream_t st) {
+    HopArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.g = c->g;
+    a.prepare = 1;
+    auto one = [&](int prec, int kind) {
+        return launch_hop(prec, kind, a, prec == EOFA_F64 ? (const void*)&c->c64 : (const void*)&c->c32, st);
+    };
+    cudaError_t e = one(P == EOFA_F64 ? EOFA_F64 : EOFA_F32, KIND_R_BACK);
+    for (int k = 0; k < 4 && e == cudaSuccess; ++k) {
+        a.tile_var = c->tile[P][k];
+        e = one(P, KIND_R_EO + k);
+    }
+    a.tile_var = 0;
+    for (int kind : {KIND_EO_MINV, KIND_OE_SCHUR})  // the outer residual
+        if (e == cudaSuccess) e = one(EOFA_F64, kind);
+    return e == cudaSuccess ? EOFA_OK : cuda_fail(c, e, "hop kernel set-up");
+}
 
 eofa_status autotune(eofa_ctx* c, int P, cudaStream_t st) {
     if (c->tuned[P]) return EOFA_OK;
     // EOFA_TILE_VARIANT=v fixes every inner-solver hop kind to variant v
     // (reproducible profiles); variants FP64 arithmetic lacks fall back to
-    // v & 1.  The kernels are still launched once here, before any graph
-    // capture needs them.
+    // v & 1.
     int forced = -1;
     if (const char* fv = std::getenv("EOFA_TILE_VARIANT")) {
         const int v = std::atoi(fv);
         if (v >= 0 && v <= 3) forced = (P == EOFA_F64) ? (v & 1) : v;
     }
     const Geom& g = c->g;
+    int dev = 0;
+    CK(cudaGetDevice(&dev), "cudaGetDevice");
     bool all = forced < 0;
     if (forced < 0) {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         for (int k = 0; k < 4; ++k) {
-            auto it = g_tune_cache.find({P, g.Ls, (long)g.X * g.Y, (long)g.Z * g.T, k});
+            auto it = g_tune_cache.find(tune_key(dev, P, g, k));
             if (it == g_tune_cache.end()) {
                 all = false;
             } else {
@@ -445,8 +476,9 @@ eofa_status autotune(eofa_ctx* c, int P, cudaStream_t st) {
         }
     }
     if (all) {
-        c->tuned[P] = true;
-        return EOFA_OK;
+        const eofa_status ps = prepare_solve(c, P, st);
+        c->tuned[P] = ps == EOFA_OK;
+        return ps;
     }
     // operands: the inner vectors of P, or the context's FP64 work vectors
     VecRef odd_a, even_t, odd_b;
@@ -465,15 +497,6 @@ eofa_status autotune(eofa_ctx* c, int P, cudaStream_t st) {
     CK(cudaEventCreate(&e1), "event");
     const VecRef none{};
     eofa_status s = EOFA_OK;
-    // the kinds that a captured solve launches beside the tuned ones: once
-    // here, because their set-up must not run inside a capture
-    const int xp = P == EOFA_F64 ? EOFA_F64 : EOFA_F32;
-    s = hop(c, xp, KIND_R_BACK, 1, none, P == EOFA_F64 ? odd_a : c->inner[P].x, VecRef{c->ro.d, nullptr},
-            red(c, FIN_NONE), nullptr, st);
-    if (s == EOFA_OK && P == EOFA_F64)
-        s = hop(c, P, KIND_EO_MINV, 0, odd_a, none, even_t, red(c, FIN_NONE), nullptr, st);
-    if (s == EOFA_OK && P == EOFA_F64)
-        s = hop(c, P, KIND_OE_SCHUR, 1, even_t, odd_a, odd_b, red(c, FIN_NONE), nullptr, st);
     for (int k = 0; k < 4 && s == EOFA_OK; ++k) {
         const bool even_out = (k & 1) == 0;  // kernel kinds KIND_R_EO + k
         const int nvar = (P == EOFA_F64) ? 2 : 4;  // register-capped variants for FP32 arithmetic
@@ -515,14 +538,12 @@ eofa_status autotune(eofa_ctx* c, int P, cudaStream_t st) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     c->launches = 0;
-    if (s != EOFA_OK) {
-        c->tuned[P] = false;
-        return s;
-    }
-    c->tuned[P] = true;
+    if (s == EOFA_OK) s = prepare_solve(c, P, st);
+    c->tuned[P] = s == EOFA_OK;
+    if (s != EOFA_OK) return s;
     std::lock_guard<std::mutex> lock(g_tune_mu);
     for (int k = 0; k < 4; ++k) {
-        TuneChoice& tc = g_tune_cache[{P, g.Ls, (long)g.X * g.Y, (long)g.Z * g.T, k}];
+        TuneChoice& tc = g_tune_cache[tune_key(dev, P, g, k)];
         tc.variant = c->tile[P][k];
         for (int v = 0; v < 4; ++v) tc.ms[v] = c->tune_ms[P][k][v];
     }
