@@ -662,9 +662,11 @@ def run_ours(args):
                              f"workload, {pi:.3f} s/iteration, scaled by the oracle's recorded {n_iter} "
                              f"iterations to r=1e-10"}
     f64 = extra.get("f64", {}).get("s_per_solve")
-    # the FP64 hop (the plain FP64 CG comparator).  Its products run in 64-bit
-    # fixed point on the integer pipes, so the FP64 FMA throughput is not its
-    # roofline: its algorithmic bytes are held against the copy bandwidth, and
+    # the FP64 hop (the plain FP64 CG comparator), its input pass included.  Its
+    # products run in 64-bit fixed point on the integer pipes, so the FP64 FMA
+    # throughput is not its roofline, and instruction issue and latency bound
+    # it, not memory: its algorithmic bytes are given against the copy
+    # bandwidth for scale, and
     # the algorithmic count of 1520 flops per 5D output site per launch (1320
     # Wilson hop, 50 for b5 + c5 L, 150 for the s-space inverse) is given
     # beside the FP64 FMA throughput that a floating-point hop could not pass
@@ -675,7 +677,8 @@ def run_ours(args):
         n5 = int(np.prod(w["dims"])) // 2 * w["Ls"]
         sec = extra["f64"]["hop_ms_per_launch"] * 1e-3
         gbs = hop_bytes_f64 / sec / 1e9
-        roofline_f64 = {"bound": "hbm", "kernel": "hop_kernel<double, Ls=16> (4 kinds, 64-bit fixed point)",
+        roofline_f64 = {"bound": "issue/latency",
+                        "kernel": "hop_kernel<double, Ls=16> (4 kinds, 64-bit fixed point, with the input pass)",
                         "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
                         "peak_kind": f"of {peak_kind} (MEASURED_PEAKS.json hbm_gbs)",
                         "algorithmic_tflops": FLOPS_PER_SITE * n5 / sec / 1e12, "flops_per_site": FLOPS_PER_SITE,

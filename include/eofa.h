@@ -125,8 +125,9 @@ typedef struct {
     double true_res;     /* FP64 ||rhs - A sol|| / ||rhs|| on the full lattice */
     double recur_res;    /* last recursively updated residual (relative) */
     double seconds;      /* wall-clock time of the call */
-    double hop_ms;       /* summed time of the timed hop kernels */
-    double hop_bytes;    /* algorithmic bytes moved by the timed hop kernels */
+    double hop_ms;       /* summed time of the timed hop kernels (inner F64: with the pass that
+                            prepares the input of every second one) */
+    double hop_bytes;    /* algorithmic bytes moved by the timed hop kernels (eofa_hop_bytes) */
     long kernel_launches;/* kernels this library launched during the call */
     int precond_iters;   /* flexible-GCR steps with the learned preconditioner (precond = 1) */
     int precond_fallbacks; /* inner solves handed to CGNR because a GCR cycle did not halve |r| */

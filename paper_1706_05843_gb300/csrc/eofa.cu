@@ -329,6 +329,18 @@ cudaError_t launch_hop(int prec, int kind, const HopArgs& a, const void* coef, c
 
 eofa_status hop(eofa_ctx* c, int prec, int kind, int out_par, VecRef in, VecRef y, VecRef out, Reduce rd,
                 const int* done, cudaStream_t st, bool timed = false, int* stop = nullptr) {
+    // (the time of a hop includes its input pass, here and in the graph sample)
+    const bool tm = timed && c->timing;
+    if (tm) {
+        if (c->ev_used + 2 > (int)c->evs.size()) {
+            for (int i = 0; i < 64; ++i) {
+                cudaEvent_t e;
+                CK(cudaEventCreate(&e), "cudaEventCreate");
+                c->evs.push_back(e);
+            }
+        }
+        CK(cudaEventRecord(c->evs[c->ev_used], st), "cudaEventRecord");
+    }
     const void* in_raw = in.raw;
     if (const int pass = prec == EOFA_F64 ? hop_input_pass(kind) : 0) {
         // into c->ro, which holds nothing live at any of these launches
@@ -354,17 +366,6 @@ eofa_status hop(eofa_ctx* c, int prec, int kind, int out_par, VecRef in, VecRef 
     if (kind >= KIND_D_EO && kind <= KIND_D_OE_DAG && prec <= EOFA_F32)
         a.dense = c->dense[prec][(kind == KIND_D_OE || kind == KIND_D_OE_DAG) ? 1 : 0];
     const void* coef = prec == EOFA_F64 ? (const void*)&c->c64 : (const void*)&c->c32;
-    const bool tm = timed && c->timing;
-    if (tm) {
-        if (c->ev_used + 2 > (int)c->evs.size()) {
-            for (int i = 0; i < 64; ++i) {
-                cudaEvent_t e;
-                CK(cudaEventCreate(&e), "cudaEventCreate");
-                c->evs.push_back(e);
-            }
-        }
-        CK(cudaEventRecord(c->evs[c->ev_used], st), "cudaEventRecord");
-    }
     const cudaError_t e = launch_hop(prec, kind, a, coef, st);
     if (e != cudaSuccess) return cuda_fail(c, e, "hop kernel launch");
     ++c->launches;
