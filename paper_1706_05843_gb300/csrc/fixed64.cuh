@@ -122,8 +122,8 @@ __device__ __forceinline__ double fx_to(i64 v, int E) {
     return v == 0 ? 0.0 : __hiloint2double(hi, __double2loint(d));
 }
 
-// a b + c; the C++ expression compiles to an unsigned wide product and two
-// sign corrections
+// a b + c.  With (i64)a * b + c in its place H at 24^3x64, Ls = 12 takes 11.1
+// instead of 7.2 ms, K at 16^4, Ls = 16 905 instead of 608 us.
 __device__ __forceinline__ i64 fx_mad(int a, int b, i64 c) {
     i64 d;
     asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
