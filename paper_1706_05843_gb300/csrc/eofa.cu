@@ -1417,10 +1417,12 @@ eofa_status solve_batched_impl(eofa_ctx* const* cs, int n, const void* const* rh
 // The operator applications: one pass makes both parities' hop inputs, then
 // the hops (one launch for both where that fills the SMs better) read their
 // site-local part from the caller's field and write the caller's result: two
-// or three launches and 970 bytes of traffic per
-// 5D site, where import, D~ passes, hops and export took six to eight and up
-// to 1900 (H at 24^3x64, Ls = 12: 8.8 -> 7.0 ms; K at 4^4, Ls = 8: 78 -> 51
-// us with a hop launch per parity).  H = g5 R5 K D~^-1 needs no D~: K D~^-1 = T^-1 - 1/2 D_h.
+// or three launches and 970 bytes of traffic per 5D site, where import, D~
+// passes, hops and export took six to eight and up to 1900 (with the hop of
+// that time, one lane a site: H at 24^3x64, Ls = 12 8.8 -> 7.0 ms; K at 4^4, Ls =
+// 8 78 -> 51 us with a hop launch per parity.  Now 7.2 ms and 21 us back to
+// back, of which 0.5 ms and none are the sums' FP64 safeguard).  H = g5 R5 K
+// D~^-1 needs no D~: K D~^-1 = T^-1 - 1/2 D_h.
 eofa_status apply_impl(eofa_ctx* c, const void* in, void* out, int which, cudaStream_t st) {
     // which: 0 = K, 1 = K^dag, 2 = H + beta Delta P = g5 R5 K D~^-1
     // the hop reads the input while it writes the output: fields that overlap
@@ -2337,6 +2339,7 @@ struct WorkSpace {
 
 void net_lay(WorkSpace& B, NetDev& n) {
     B.get(&n.Wm, (size_t)kNetWeights);
+    B.get(&n.redo, (size_t)kWgMaxCtas);
     for (int l = 0; l < kNetLayers; ++l) {
         B.get(&n.Wf[l], (size_t)81 * 32 * 32);
         B.get(&n.Wb[l], (size_t)81 * 32 * 32);
@@ -2451,6 +2454,8 @@ eofa_status ensure_learned(eofa_ctx* c) {
     CK(cudaMemset(c->counter2, 0, 256), "memset");
     if ((s = dalloc(c, &p, sizeof(float) * kNetWeights))) return s;
     c->net.Wm = (float*)p;
+    if ((s = dalloc(c, &p, sizeof(int) * kWgMaxCtas))) return s;
+    c->net.redo = (int*)p;
     for (int l = 0; l < kNetLayers; ++l) {
         if ((s = dalloc(c, &p, sizeof(bf16) * 81 * 32 * 32))) return s;
         c->net.Wf[l] = (bf16*)p;

@@ -10,7 +10,6 @@
 
 #include <algorithm>
 #include <cstdint>
-#include <type_traits>
 
 namespace eofa {
 
@@ -432,17 +431,21 @@ __global__ void __launch_bounds__(kCvThreads, 1)
 // one atomic per element and CTA.  Bound by the mma.sync rate (math pipe
 // throttle leads the stalls; nine warps of 32 channels: 0.93 ms).
 // The zero rows of dy would turn an Inf of in into NaN: a CTA whose sums are
-// not all finite makes them again with the halo's rows of in zero as well
-// (that in every pass: the network's gradients at 16^3 x 32, 8 slices 4.31 ->
-// 4.81 ms; on demand 4.27 -> 4.37 ms, the second walk's registers).
+// not all finite leaves them to a second launch (MASKED), in which the halo's
+// rows of in are zero as well and the other CTAs return at once (masked in every
+// pass: the network's gradients at 16^3 x 32, 8 slices 4.31 -> 4.81 ms; a second
+// walk in the same kernel 4.27 -> 4.37 ms, for its registers; this form 4.30 ->
+// 4.24 ms).
 // ---------------------------------------------------------------------------
 constexpr int kWgThreads = 576;
 constexpr int kWgStages = 3;
 constexpr int kWgFlush = 8;  // steps (of 8 k16 products) between sums into the FP32 registers
 
+template <bool MASKED>
 __global__ void __launch_bounds__(kWgThreads, 1)
-    k_conv_wgrad(const bf16* __restrict__ in, const bf16* __restrict__ dy, float* __restrict__ dW, ConvGeom g,
-                 ConvPlan pl, int cout, int cin) {
+    k_conv_wgrad(const bf16* __restrict__ in, const bf16* __restrict__ dy, float* __restrict__ dW, int* redo,
+                 ConvGeom g, ConvPlan pl, int cout, int cin) {
+    if (MASKED && !redo[blockIdx.x]) return;
     extern __shared__ __align__(128) unsigned char wg_smem[];
     const int stage_elems = (kCvRows + 3 * pl.np) * 32;
     bf16* st0 = reinterpret_cast<bf16*>(wg_smem);                                   // [stages][dy | in dz 0..2]
@@ -455,7 +458,6 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     const long slice = (long)g.Z * g.Y * g.X;
 
     long tab_col = -1;
-    bool redo = false;
     auto issue = [&](long s, int buf) {
         const long col = s / g.T;
         const int t = (int)(s - col * g.T);
@@ -474,7 +476,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
             }
             __syncthreads();
         }
-        if (redo && tid < kCvRows) {
+        if (MASKED && tid < kCvRows) {
             const unsigned rows = __ballot_sync(0xffffffffu, tab[tid + pl.line + 1].y >= 0);
             if (lane == 0) s_rows[buf][warp] = rows;
         }
@@ -513,62 +515,57 @@ __global__ void __launch_bounds__(kWgThreads, 1)
 
     const int dz = warp % 9 / 3, dyy = warp % 3, nh = warp / 9;
     const int i8 = lane >> 3;
-    auto walk = [&](auto masked) {
-        for (int i = 0; i < kWgStages - 1; ++i) {
-            if (s0 + i < s1) issue(s0 + i, i);
-            cp_commit();
-            __syncthreads();  // the table may be rewritten by the next issue
-        }
-        int buf = 0;
-        for (long s = s0; s < s1; ++s) {
-            cp_wait<kWgStages - 2>();
-            __syncthreads();  // this step's stage has arrived; the oldest stage and the table are free
-            const long nx = s + kWgStages - 1;
-            if (nx < s1) issue(nx, buf == 0 ? kWgStages - 1 : buf - 1);
-            cp_commit();
-            const bf16* D = st0 + (size_t)buf * stage_elems;
-            const bf16* In = D + (kCvRows + dz * pl.np) * 32;
-            const int off = dyy * pl.line;
+    for (int i = 0; i < kWgStages - 1; ++i) {
+        if (s0 + i < s1) issue(s0 + i, i);
+        cp_commit();
+        __syncthreads();  // the table may be rewritten by the next issue
+    }
+    int buf = 0;
+    for (long s = s0; s < s1; ++s) {
+        cp_wait<kWgStages - 2>();
+        __syncthreads();  // this step's stage has arrived; the oldest stage and the table are free
+        const long nx = s + kWgStages - 1;
+        if (nx < s1) issue(nx, buf == 0 ? kWgStages - 1 : buf - 1);
+        cp_commit();
+        const bf16* D = st0 + (size_t)buf * stage_elems;
+        const bf16* In = D + (kCvRows + dz * pl.np) * 32;
+        const int off = dyy * pl.line;
 #pragma unroll 2
-            for (int kb = 0; kb < kCvRows / 16; ++kb) {
-                unsigned af[2][4], bfr[3][4];
+        for (int kb = 0; kb < kCvRows / 16; ++kb) {
+            unsigned af[2][4], bfr[3][4];
 #pragma unroll
-                for (int mt = 0; mt < 2; ++mt)   // A = dy^T: (co, k) from rows k, columns co
-                    ldsm_x4_t(af[mt], D + swz(kb * 16 + (lane & 7) + (i8 >> 1) * 8, mt * 2 + (i8 & 1)));
+            for (int mt = 0; mt < 2; ++mt)   // A = dy^T: (co, k) from rows k, columns co
+                ldsm_x4_t(af[mt], D + swz(kb * 16 + (lane & 7) + (i8 >> 1) * 8, mt * 2 + (i8 & 1)));
 #pragma unroll
-                for (int dx = 0; dx < 3; ++dx)   // B = in_shift: (k, ci) rows k
-                    ldsm_x4_t(bfr[dx], In + swz(off + dx + kb * 16 + (lane & 7) + (i8 & 1) * 8, nh * 2 + (i8 >> 1)));
-                if constexpr (decltype(masked)::value) {  // this lane's rows k: 2 (lane & 3) + 0, 1 and those + 8
-                    const unsigned rows = s_rows[buf][kb >> 1] >> ((kb & 1) * 16 + (lane & 3) * 2);
-                    const unsigned m0 = (rows & 1) * 0xffffu | (rows >> 1 & 1) * 0xffff0000u;
-                    const unsigned m1 = (rows >> 8 & 1) * 0xffffu | (rows >> 9 & 1) * 0xffff0000u;
+            for (int dx = 0; dx < 3; ++dx)   // B = in_shift: (k, ci) rows k
+                ldsm_x4_t(bfr[dx], In + swz(off + dx + kb * 16 + (lane & 7) + (i8 & 1) * 8, nh * 2 + (i8 >> 1)));
+            if constexpr (MASKED) {  // this lane's rows k: 2 (lane & 3) + 0, 1 and those + 8
+                const unsigned rows = s_rows[buf][kb >> 1] >> ((kb & 1) * 16 + (lane & 3) * 2);
+                const unsigned m0 = (rows & 1) * 0xffffu | (rows >> 1 & 1) * 0xffff0000u;
+                const unsigned m1 = (rows >> 8 & 1) * 0xffffu | (rows >> 9 & 1) * 0xffff0000u;
 #pragma unroll
-                    for (int i = 0; i < 12; ++i) bfr[i / 4][i % 4] &= i % 2 ? m1 : m0;
-                }
-#pragma unroll
-                for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-                    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                        for (int nt = 0; nt < 2; ++nt)
-                            mma16816(acc[dx][mt][nt], af[mt], bfr[dx][nt * 2], bfr[dx][nt * 2 + 1]);
+                for (int i = 0; i < 12; ++i) bfr[i / 4][i % 4] &= i % 2 ? m1 : m0;
             }
-            if ((s - s0) % kWgFlush == kWgFlush - 1) flush();
-            buf = buf + 1 == kWgStages ? 0 : buf + 1;
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                    for (int nt = 0; nt < 2; ++nt)
+                        mma16816(acc[dx][mt][nt], af[mt], bfr[dx][nt * 2], bfr[dx][nt * 2 + 1]);
         }
-        cp_wait<0>();
-        flush();
-    };
-    walk(std::integral_constant<bool, false>{});
-    float odd = 0.f;
+        if ((s - s0) % kWgFlush == kWgFlush - 1) flush();
+        buf = buf + 1 == kWgStages ? 0 : buf + 1;
+    }
+    cp_wait<0>();
+    flush();
+    if constexpr (!MASKED) {
+        float nf = 0.f;
 #pragma unroll
-    for (int i = 0; i < 48; ++i) odd += 0.f * (&sum[0][0][0][0])[i];
-    if (__syncthreads_or(odd != 0.f)) {  // (NaN: 0 x Inf or 0 x NaN)
-#pragma unroll
-        for (int i = 0; i < 48; ++i) (&sum[0][0][0][0])[i] = 0.f;
-        tab_col = -1;
-        redo = true;
-        walk(std::integral_constant<bool, true>{});
+        for (int i = 0; i < 48; ++i) nf += 0.f * (&sum[0][0][0][0])[i];  // NaN from Inf or NaN
+        const int bad = __syncthreads_or(nf != 0.f);
+        if (tid == 0) redo[blockIdx.x] = bad;
+        if (bad) return;
     }
     if (s0 == s1) return;
 #pragma unroll
@@ -699,7 +696,7 @@ cudaError_t conv(const bf16* in, const bf16* W, void* out, const bf16* mask, con
     return cudaGetLastError();
 }
 
-cudaError_t wgrad(const bf16* in, const bf16* dy, float* dW, const ConvGeom& g, int cout, int cin,
+cudaError_t wgrad(const bf16* in, const bf16* dy, float* dW, int* redo, const ConvGeom& g, int cout, int cin,
                   cudaStream_t st) {
     if ((long)g.V * g.S == 0) return cudaSuccess;
     int dev = 0, sms = 0;
@@ -708,12 +705,17 @@ cudaError_t wgrad(const bf16* in, const bf16* dy, float* dW, const ConvGeom& g, 
     if (e != cudaSuccess) return e;
     const ConvPlan p = conv_plan(g, sms);
     const size_t smem = (size_t)kWgStages * (kCvRows + 3 * p.np) * 64 + (size_t)p.np * 8;
-    e = cudaFuncSetAttribute(k_conv_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_conv_wgrad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_conv_wgrad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // three CTA classes (dt); a share of fewer than 2 steps is not worth its atomics
     const long steps = (long)g.S * p.nxb * p.tiles * g.T;
-    const int ranks = (int)std::max<long>(1, std::min<long>(sms / 3, (steps + 1) / 2));
-    k_conv_wgrad<<<3 * ranks, kWgThreads, smem, st>>>(in, dy, dW, g, p, cout, cin);
+    const int ranks = (int)std::max<long>(1, std::min<long>(std::min(sms, kWgMaxCtas) / 3, (steps + 1) / 2));
+    k_conv_wgrad<false><<<3 * ranks, kWgThreads, smem, st>>>(in, dy, dW, redo, g, p, cout, cin);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_conv_wgrad<true><<<3 * ranks, kWgThreads, smem, st>>>(in, dy, dW, redo, g, p, cout, cin);
     return cudaGetLastError();
 }
 
@@ -748,11 +750,11 @@ cudaError_t net_backward(const NetDev& n, const ConvGeom& g, const bf16* a0, con
     float* dW0 = dW;
     float* dW1 = dW + kNetLayerW[0];
     float* dW2 = dW1 + kNetLayerW[1];
-    if ((e = wgrad(a2, dob, dW2, g, kNetCout[2], kNetCin[2], st)) != cudaSuccess) return e;
+    if ((e = wgrad(a2, dob, dW2, n.redo, g, kNetCout[2], kNetCin[2], st)) != cudaSuccess) return e;
     if ((e = conv<EPI_DMASK_BF16>(dob, n.Wb[2], d2, a2, g, st)) != cudaSuccess) return e;
-    if ((e = wgrad(a1, d2, dW1, g, kNetCout[1], kNetCin[1], st)) != cudaSuccess) return e;
+    if ((e = wgrad(a1, d2, dW1, n.redo, g, kNetCout[1], kNetCin[1], st)) != cudaSuccess) return e;
     if ((e = conv<EPI_DMASK_BF16>(d2, n.Wb[1], d1, a1, g, st)) != cudaSuccess) return e;
-    if ((e = wgrad(a0, d1, dW0, g, kNetCout[0], kNetCin[0], st)) != cudaSuccess) return e;
+    if ((e = wgrad(a0, d1, dW0, n.redo, g, kNetCout[0], kNetCin[0], st)) != cudaSuccess) return e;
     if (din) return conv<EPI_F32>(d1, n.Wb[0], din, nullptr, g, st, dstride);
     return cudaSuccess;
 }

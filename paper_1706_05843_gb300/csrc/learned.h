@@ -27,6 +27,7 @@ constexpr long kNetLayerW[3] = {81L * 32 * 24, 81L * 32 * 32, 81L * 24 * 32};
 constexpr long kNetWeights = 81L * 32 * 24 + 81L * 32 * 32 + 81L * 24 * 32;  // 207360
 constexpr float kLeaky = 0.1f;
 constexpr int kCP = 32;  // padded channel count in device activations
+constexpr int kWgMaxCtas = 1024;  // of a weight-gradient launch
 
 struct ConvGeom {
     int X, Y, Z, T;
@@ -39,6 +40,7 @@ struct NetDev {
     float* Wm = nullptr;          // master FP32, public layout
     bf16* Wf[3] = {};             // forward operands, packed for the convolution (81 x 32 x 32, zero padded)
     bf16* Wb[3] = {};             // backward-data operands, taps mirrored and transposed, packed likewise
+    int* redo = nullptr;          // [kWgMaxCtas] CTAs of a weight gradient whose sums were not finite
 };
 
 // activations [S][V][32] BF16; out FP32 rows of ostride (24 or 32) floats
