@@ -89,10 +89,11 @@ static cudaError_t resident_pair(cudaStream_t st, int* dev, int* resident) {
 }
 
 // An application's two hops (p.a[0], p.a[1]; FP64).  Up to 8 rounds of
-// resident CTAs they share one grid (K at 4^4, Ls = 8: 26-31 us against 36 us
-// for a grid each; 8^3x16, Ls = 8: 52 against 62.5 us; 12^3x24, Ls = 12, six
-// rounds: 306 against 318 us); larger lattices fill the SMs with a grid each
-// (16^4, Ls = 16, eleven rounds: 609 us in one grid, 599 us in two).
+// resident CTAs they share one grid (K at 4^4, Ls = 8: 21 us against 36 us for
+// a grid each; 8^3x16, Ls = 8: 54 against 64 us; 16^4, Ls = 8, seven rounds: 325
+// against 335 us); larger lattices fill the SMs with a grid each (12^3x24, Ls =
+// 16, 8.5 rounds: 390 us in both; 16^4, Ls = 16, 13.5 rounds: K 613 us in one
+// grid, 608 us in two, H 704 and 692 us).
 template <typename S, int LS, int K>
 static cudaError_t launch_pair(const HopPair& p, const SCoef<typename Traits<S>::R>& c, cudaStream_t st) {
     constexpr int NS = HopTile<S, LS, K, 0>::NS;

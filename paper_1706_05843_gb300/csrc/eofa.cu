@@ -147,8 +147,10 @@ eofa_status dalloc(eofa_ctx* c, void** p, size_t bytes) {
 // hop_in: the vector may hold an FP64 hop input (fixed point with an exponent
 // per 5D site); raw: one that a hop kernel writes, with its doubles
 eofa_status vec_alloc(eofa_ctx* c, int prec, VecRef* v, bool hop_in = false, bool raw = false) {
-    eofa_status s = dalloc(c, &v->d, (size_t)c->n5 * 24 * kWidth[prec]);
+    const size_t bytes = (size_t)c->n5 * 24 * kWidth[prec];
+    eofa_status s = dalloc(c, &v->d, raw ? 2 * bytes : bytes);
     if (s != EOFA_OK) return s;
+    v->raw = raw ? (char*)v->d + bytes : nullptr;
     v->n = nullptr;
     if (prec == EOFA_F16 || hop_in) {
         void* n = nullptr;
@@ -156,8 +158,7 @@ eofa_status vec_alloc(eofa_ctx* c, int prec, VecRef* v, bool hop_in = false, boo
         if (s != EOFA_OK) return s;
         v->n = (float*)n;
     }
-    v->raw = nullptr;
-    return raw ? dalloc(c, &v->raw, (size_t)c->n5 * 24 * sizeof(double)) : EOFA_OK;
+    return EOFA_OK;
 }
 
 // ---------------------------------------------------------------------------

@@ -15,7 +15,7 @@ ACT = dict(M5=1.8, b=1.5, c=0.5, m1=0.04, m2=1.0, m3=0.04, beta=-1.0, pm=1, t_bc
 
 
 @pytest.mark.parametrize("dims,Ls,pm", [
-    ((12, 12, 12, 24), 12, -1),  # column phase for K^dag
+    ((12, 12, 12, 16), 12, -1),  # column phase for K^dag
     ((12, 12, 12, 10), 16, 1),   # shuffles
     ((10, 10, 10, 12), 8, 1),
     ((6, 10, 14, 18), 4, -1),    # 7560 sites a parity, 16 a block: the last one half full
