@@ -213,3 +213,19 @@ def test_gparity_components(env, gmask):
     s.close()
     ref = GOracle(O.Action(dims=dims, Ls=Ls, **ACT), U, gmask).hsys(x)
     assert worst(got, ref, majorant("h", ACT, U, x, gmask)) <= BOUND
+
+
+@pytest.mark.parametrize("dims,Ls,pm,link,field", CASES)
+def test_fp64_solve(env, dims, Ls, pm, link, field):
+    """The kernels of the FP64 CG, whose hops hand their output on as integers
+    and doubles, on the same fields: a solve to 1e-12 judged by the oracle."""
+    torch, B, O = env
+    act = dict(ACT, pm=pm, m1=0.2, m3=0.2)
+    U, x = links(dims, link), fields(dims, Ls, field)
+    s = B.Solver(U, dims, Ls, **act)
+    sol, st = s.solve(torch.from_numpy(x).cuda(), tol=1e-12, inner="f64")
+    sol = sol.cpu().numpy()
+    s.close()
+    r = x - O.Oracle(O.Action(dims=dims, Ls=Ls, **act), U).hsys(sol)
+    print(f"{dims} {Ls} {link} {field}: {st.inner_iters} iterations")
+    assert np.linalg.norm(r) <= 1e-12 * np.linalg.norm(x)
