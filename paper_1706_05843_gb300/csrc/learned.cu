@@ -428,8 +428,9 @@ __global__ void __launch_bounds__(kCvThreads, 1)
 // (before: one, each tap re-reading both fields through L1; 16^3 x 32, 8
 // slices: 1.6 -> 0.82 ms a layer).  Sums: 64
 // k16 products in the tensor cores, then FP32 registers over the CTA's share,
-// one atomic per element and CTA.  Bound by the mma.sync rate (math pipe
-// throttle leads the stalls; nine warps of 32 channels: 0.93 ms).
+// one atomic per element and CTA.  Bound by the rate of mma.sync, the
+// instruction chosen (math pipe throttle leads the stalls, tensor pipe 46%; nine
+// warps of 32 channels: 0.93 ms).
 // The zero rows of dy would turn an Inf of in into NaN: a CTA whose sums are
 // not all finite leaves them to a second launch (MASKED), in which the halo's
 // rows of in are zero as well and the other CTAs return at once (masked in every
