@@ -2340,7 +2340,7 @@ struct WorkSpace {
 
 void net_lay(WorkSpace& B, NetDev& n) {
     B.get(&n.Wm, (size_t)kNetWeights);
-    B.get(&n.redo, (size_t)kWgMaxCtas);
+    B.get(&n.redo, (size_t)kNetLayers * kWgMaxCtas);
     for (int l = 0; l < kNetLayers; ++l) {
         B.get(&n.Wf[l], (size_t)81 * 32 * 32);
         B.get(&n.Wb[l], (size_t)81 * 32 * 32);
@@ -2455,7 +2455,7 @@ eofa_status ensure_learned(eofa_ctx* c) {
     CK(cudaMemset(c->counter2, 0, 256), "memset");
     if ((s = dalloc(c, &p, sizeof(float) * kNetWeights))) return s;
     c->net.Wm = (float*)p;
-    if ((s = dalloc(c, &p, sizeof(int) * kWgMaxCtas))) return s;
+    if ((s = dalloc(c, &p, sizeof(int) * kNetLayers * kWgMaxCtas))) return s;
     c->net.redo = (int*)p;
     for (int l = 0; l < kNetLayers; ++l) {
         if ((s = dalloc(c, &p, sizeof(bf16) * 81 * 32 * 32))) return s;

@@ -432,21 +432,37 @@ __global__ void __launch_bounds__(kCvThreads, 1)
 // instruction chosen (math pipe throttle leads the stalls, tensor pipe 46%; nine
 // warps of 32 channels: 0.93 ms).
 // The zero rows of dy would turn an Inf of in into NaN: a CTA whose sums are
-// not all finite leaves them to a second launch (MASKED), in which the halo's
-// rows of in are zero as well and the other CTAs return at once (masked in every
-// pass: the network's gradients at 16^3 x 32, 8 slices 4.31 -> 4.81 ms; a second
-// walk in the same kernel 4.27 -> 4.37 ms, for its registers; this form 4.30 ->
-// 4.24 ms).
+// not all finite leaves them to a second launch for all layers (MASKED), in which
+// the halo's rows of in are zero as well and the other CTAs return at once (masked
+// in every pass: the network's gradients at 16^3 x 32, 8 slices 4.31 -> 4.81 ms; a
+// second walk in the same kernel 4.27 -> 4.37 ms, for its registers; this form
+// 4.27 -> 4.22 ms, and 435 -> 440 us at 4^4, one slice).
 // ---------------------------------------------------------------------------
 constexpr int kWgThreads = 576;
 constexpr int kWgStages = 3;
 constexpr int kWgFlush = 8;  // steps (of 8 k16 products) between sums into the FP32 registers
 
+struct WgLayer {
+    const bf16* in;
+    const bf16* dy;
+    float* dW;
+    int* redo;  // a flag for each CTA
+    int cout, cin;
+};
+struct WgLayers {
+    WgLayer l[kNetLayers];
+};
+
+// MASKED: blockIdx.y numbers the layers, otherwise layer 0 alone
 template <bool MASKED>
 __global__ void __launch_bounds__(kWgThreads, 1)
-    k_conv_wgrad(const bf16* __restrict__ in, const bf16* __restrict__ dy, float* __restrict__ dW, int* redo,
-                 ConvGeom g, ConvPlan pl, int cout, int cin) {
-    if (MASKED && !redo[blockIdx.x]) return;
+    k_conv_wgrad(const __grid_constant__ WgLayers layers, ConvGeom g, ConvPlan pl) {
+    const WgLayer& L = layers.l[MASKED ? blockIdx.y : 0];
+    if (MASKED && !L.redo[blockIdx.x]) return;
+    const bf16* __restrict__ in = L.in;
+    const bf16* __restrict__ dy = L.dy;
+    float* __restrict__ dW = L.dW;
+    const int cout = L.cout, cin = L.cin;
     extern __shared__ __align__(128) unsigned char wg_smem[];
     const int stage_elems = (kCvRows + 3 * pl.np) * 32;
     bf16* st0 = reinterpret_cast<bf16*>(wg_smem);                                   // [stages][dy | in dz 0..2]
@@ -565,7 +581,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
 #pragma unroll
         for (int i = 0; i < 48; ++i) nf += 0.f * (&sum[0][0][0][0])[i];  // NaN from Inf or NaN
         const int bad = __syncthreads_or(nf != 0.f);
-        if (tid == 0) redo[blockIdx.x] = bad;
+        if (tid == 0) L.redo[blockIdx.x] = bad;
         if (bad) return;
     }
     if (s0 == s1) return;
@@ -697,8 +713,10 @@ cudaError_t conv(const bf16* in, const bf16* W, void* out, const bf16* mask, con
     return cudaGetLastError();
 }
 
-cudaError_t wgrad(const bf16* in, const bf16* dy, float* dW, int* redo, const ConvGeom& g, int cout, int cin,
-                  cudaStream_t st) {
+// one layer's weight gradient, or (masked) the sums of all layers' that were
+// not finite
+template <bool MASKED>
+cudaError_t wgrad(const WgLayers& layers, const ConvGeom& g, cudaStream_t st) {
     if ((long)g.V * g.S == 0) return cudaSuccess;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -706,17 +724,12 @@ cudaError_t wgrad(const bf16* in, const bf16* dy, float* dW, int* redo, const Co
     if (e != cudaSuccess) return e;
     const ConvPlan p = conv_plan(g, sms);
     const size_t smem = (size_t)kWgStages * (kCvRows + 3 * p.np) * 64 + (size_t)p.np * 8;
-    e = cudaFuncSetAttribute(k_conv_wgrad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_conv_wgrad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_conv_wgrad<MASKED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // three CTA classes (dt); a share of fewer than 2 steps is not worth its atomics
     const long steps = (long)g.S * p.nxb * p.tiles * g.T;
     const int ranks = (int)std::max<long>(1, std::min<long>(std::min(sms, kWgMaxCtas) / 3, (steps + 1) / 2));
-    k_conv_wgrad<false><<<3 * ranks, kWgThreads, smem, st>>>(in, dy, dW, redo, g, p, cout, cin);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_conv_wgrad<true><<<3 * ranks, kWgThreads, smem, st>>>(in, dy, dW, redo, g, p, cout, cin);
+    k_conv_wgrad<MASKED><<<dim3(3 * ranks, MASKED ? kNetLayers : 1), kWgThreads, smem, st>>>(layers, g, p);
     return cudaGetLastError();
 }
 
@@ -748,14 +761,15 @@ cudaError_t net_forward(const NetDev& n, const ConvGeom& g, const bf16* a0, bf16
 cudaError_t net_backward(const NetDev& n, const ConvGeom& g, const bf16* a0, const bf16* a1, const bf16* a2,
                          const bf16* dob, float* dW, float* din, bf16* d1, bf16* d2, cudaStream_t st, int dstride) {
     cudaError_t e;
-    float* dW0 = dW;
-    float* dW1 = dW + kNetLayerW[0];
-    float* dW2 = dW1 + kNetLayerW[1];
-    if ((e = wgrad(a2, dob, dW2, n.redo, g, kNetCout[2], kNetCin[2], st)) != cudaSuccess) return e;
+    const WgLayer w0 = {a0, d1, dW, n.redo, kNetCout[0], kNetCin[0]};
+    const WgLayer w1 = {a1, d2, w0.dW + kNetLayerW[0], n.redo + kWgMaxCtas, kNetCout[1], kNetCin[1]};
+    const WgLayer w2 = {a2, dob, w1.dW + kNetLayerW[1], n.redo + 2 * kWgMaxCtas, kNetCout[2], kNetCin[2]};
+    if ((e = wgrad<false>({{w2}}, g, st)) != cudaSuccess) return e;
     if ((e = conv<EPI_DMASK_BF16>(dob, n.Wb[2], d2, a2, g, st)) != cudaSuccess) return e;
-    if ((e = wgrad(a1, d2, dW1, n.redo, g, kNetCout[1], kNetCin[1], st)) != cudaSuccess) return e;
+    if ((e = wgrad<false>({{w1}}, g, st)) != cudaSuccess) return e;
     if ((e = conv<EPI_DMASK_BF16>(d2, n.Wb[1], d1, a1, g, st)) != cudaSuccess) return e;
-    if ((e = wgrad(a0, d1, dW0, n.redo, g, kNetCout[0], kNetCin[0], st)) != cudaSuccess) return e;
+    if ((e = wgrad<false>({{w0}}, g, st)) != cudaSuccess) return e;
+    if ((e = wgrad<true>({{w0, w1, w2}}, g, st)) != cudaSuccess) return e;
     if (din) return conv<EPI_F32>(d1, n.Wb[0], din, nullptr, g, st, dstride);
     return cudaSuccess;
 }

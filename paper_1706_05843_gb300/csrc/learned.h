@@ -40,7 +40,7 @@ struct NetDev {
     float* Wm = nullptr;          // master FP32, public layout
     bf16* Wf[3] = {};             // forward operands, packed for the convolution (81 x 32 x 32, zero padded)
     bf16* Wb[3] = {};             // backward-data operands, taps mirrored and transposed, packed likewise
-    int* redo = nullptr;          // [kWgMaxCtas] CTAs of a weight gradient whose sums were not finite
+    int* redo = nullptr;          // [3][kWgMaxCtas] CTAs of the weight gradients whose sums were not finite
 };
 
 // activations [S][V][32] BF16; out FP32 rows of ostride (24 or 32) floats
